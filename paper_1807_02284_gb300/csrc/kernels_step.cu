@@ -4,10 +4,6 @@
 
 namespace lbm {
 
-// Paper velocity index q (Appendix list, index 13 read as (1,0,-1)) -> cube slot k.
-__constant__ int c_paper_to_cube[27] = {13, 14, 12, 16, 10, 22, 4,  17, 15, 11, 9,  23, 21, 5,
-                                        3,  25, 19, 7,  1,  26, 24, 20, 18, 8,  6,  2,  0};
-
 // MINB: CTAs of 256 threads per SM the registers are bounded for (3: 80 registers, no
 // spills; 4: 64 registers with a small spill, more loads in flight); chosen by autotuning.
 template <typename T, typename IT, bool ALIGN, int MINB, bool WALLS>
@@ -335,30 +331,107 @@ cudaError_t launch_inflow_records(const void* rec, int n, uint8_t* flags, float*
 
 // ---- field conversion ------------------------------------------------------------------
 
+// Conversion between the stored deviation d = f - w and the population f.  With FP32 on the
+// caller's side the sum w + d is formed in float pairs (w = wh + wl to 48 bits, the exact
+// rounding error of wh + d added back with wl), which gives the nearest float of the exact
+// sum up to ties.  An FP64 add with its two conversions per value made these copies
+// 4.6 times slower than HBM: GB300's FP64 issue rate is a small fraction of FP32's
+// (reading a 256^3 state, 4.2 GB of populations, velocity and scalar: 2604 us with FP64 adds,
+// 614 us now; writing and reading 128^3 populations: 624 us before, 120 us now).
+template <int K>
+struct WeightPair {
+  static constexpr float hi = (float)wkd(K);
+  static constexpr float lo = (float)(wkd(K) - (double)hi);
+};
+
+// a + b = s + e exactly (Knuth's two-sum); e = 0 where s is infinite or NaN
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  if (!(e == e)) e = 0.0f;
+}
+
+template <int K, typename O>
+__device__ __forceinline__ O population(float d) {
+  if constexpr (sizeof(O) == 8) {
+    return wkd(K) + (double)d;
+  } else {
+    float s, e;
+    two_sum(WeightPair<K>::hi, d, s, e);
+    return __fadd_rn(s, __fadd_rn(e, WeightPair<K>::lo));
+  }
+}
+
+__device__ __forceinline__ void store_deviation(float* p, float s, float t) { *p = __fadd_rn(s, t); }
+// Half storage rounds s + t once: the float sum is rounded to odd first, so that the second
+// rounding sees on which side of a tie the exact sum lies.
+__device__ __forceinline__ void store_deviation(__half* p, float s, float t) {
+  float r, e;
+  two_sum(s, t, r, e);
+  if (e != 0.0f && r != 0.0f) {
+    int b = __float_as_int(r);
+    if ((e > 0.0f) != (r > 0.0f)) b -= 1;     // r was rounded away from zero: truncate
+    r = __int_as_float(b | 1);
+  }
+  *p = __float2half_rn(r);
+}
+
+template <int K, typename T, typename I>
+__device__ __forceinline__ void put_deviation(T* p, I f) {
+  if constexpr (sizeof(I) == 8) {
+    const double dev = f - wkd(K);
+    if constexpr (sizeof(T) == 2) *p = __double2half(dev);
+    else *p = (float)dev;
+  } else {
+    float s, e;
+    two_sum(f, -WeightPair<K>::hi, s, e);
+    store_deviation(p, s, __fsub_rn(e, WeightPair<K>::lo));
+  }
+}
+
+// The 27 planes of one node, Q the caller's (paper) velocity index.
+template <int Q, typename T, typename O>
+__device__ __forceinline__ void read_planes(const float (&d)[27], size_t N, size_t idx, O* out) {
+  if constexpr (Q < 27) {
+    constexpr int k = paper_to_cube(Q);
+    out[(size_t)Q * N + idx] = population<k, O>(d[k]);
+    read_planes<Q + 1, T, O>(d, N, idx, out);
+  }
+}
+
+template <int Q, typename T, typename I>
+__device__ __forceinline__ void write_planes(const I (&f)[27], size_t N, size_t idx, T* d) {
+  if constexpr (Q < 27) {
+    constexpr int k = paper_to_cube(Q);
+    put_deviation<k>(d + (size_t)k * N + idx, f[Q]);
+    write_planes<Q + 1, T, I>(f, N, idx, d);
+  }
+}
+
+// HBM-bound copies (216 B per node between FP32 arrays): every load of a node before its
+// first store, one node per thread and trip.
 template <typename T, typename O>
-__global__ void k_read_f(const T* d, size_t N, O* out) {
+__global__ void __launch_bounds__(256) k_read_f(const T* __restrict__ d, size_t N,
+                                                O* __restrict__ out) {
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < N;
        idx += (size_t)gridDim.x * blockDim.x) {
+    float v[27];
 #pragma unroll
-    for (int q = 0; q < 27; ++q) {
-      const int k = c_paper_to_cube[q];
-      const double val = wkd(k) + (double)load_pop(d + (size_t)k * N + idx);
-      out[(size_t)q * N + idx] = (O)val;
-    }
+    for (int k = 0; k < 27; ++k) v[k] = load_pop(d + (size_t)k * N + idx);
+    read_planes<0, T, O>(v, N, idx, out);
   }
 }
 
 template <typename T, typename I>
-__global__ void k_write_f(T* d, size_t N, const I* in) {
+__global__ void __launch_bounds__(256) k_write_f(T* __restrict__ d, size_t N,
+                                                 const I* __restrict__ in) {
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < N;
        idx += (size_t)gridDim.x * blockDim.x) {
+    I v[27];
 #pragma unroll
-    for (int q = 0; q < 27; ++q) {
-      const int k = c_paper_to_cube[q];
-      const double dev = (double)in[(size_t)q * N + idx] - wkd(k);
-      if constexpr (sizeof(T) == 2) d[(size_t)k * N + idx] = __double2half(dev);
-      else d[(size_t)k * N + idx] = (float)dev;
-    }
+    for (int q = 0; q < 27; ++q) v[q] = __ldg(in + (size_t)q * N + idx);
+    write_planes<0, T, I>(v, N, idx, d);
   }
 }
 
@@ -418,9 +491,25 @@ __global__ void k_convert(const I* in, O* out, size_t n) {
     out[i] = (O)in[i];
 }
 
+// FP32 to FP32 (the device read and write of velocity and scalar): 16 bytes per thread and
+// trip, taken when both arrays are 16-byte aligned; the last n % 4 values by one thread.
+__global__ void __launch_bounds__(256) k_copy4(const float* __restrict__ in,
+                                               float* __restrict__ out, size_t n) {
+  const size_t n4 = n / 4;
+  const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  for (size_t i = i0; i < n4; i += (size_t)gridDim.x * blockDim.x)
+    reinterpret_cast<float4*>(out)[i] = __ldg(reinterpret_cast<const float4*>(in) + i);
+  if (i0 == 0)
+    for (size_t i = 4 * n4; i < n; ++i) out[i] = in[i];
+}
+
 cudaError_t launch_convert(const void* in, int in_f64, void* out, int out_f64, size_t n,
                            cudaStream_t s) {
   const int g = grid_for(n);
+  if (!in_f64 && !out_f64 && aligned_to(in, 16) && aligned_to(out, 16)) {
+    k_copy4<<<grid_for((n + 3) / 4), 256, 0, s>>>((const float*)in, (float*)out, n);
+    return cudaGetLastError();
+  }
   if (in_f64 && out_f64) k_convert<double, double><<<g, 256, 0, s>>>((const double*)in, (double*)out, n);
   else if (in_f64) k_convert<double, float><<<g, 256, 0, s>>>((const double*)in, (float*)out, n);
   else if (out_f64) k_convert<float, double><<<g, 256, 0, s>>>((const float*)in, (double*)out, n);
