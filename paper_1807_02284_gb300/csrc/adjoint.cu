@@ -161,34 +161,36 @@ __device__ __forceinline__ void push_all(const float (&A)[27], float* __restrict
 }
 
 // Transpose of the collision (and of the scale mapping, which is the same relaxation with
-// other keep factors): K holds the central moments before relaxation at velocity u (it is
-// overwritten), A the adjoint of the post-collision populations on entry and the adjoint of
+// other keep factors): K holds the central moments before relaxation at velocity u, A the
+// adjoint of the post-collision populations on entry and the adjoint of
 // the pre-collision populations on return; the velocity terms are added to ub and the
 // adjoint of the keep factors of the high-order groups to kbar.
 // With `local` set (the strain-rate mode of the adaptive factor), the factor's input g is
 // local_strain of the central moments K, so the keep factors' adjoint flows back into K, rho
 // and u here (between the relaxation's transpose and the shifts').
-__device__ __forceinline__ void collide_vjp(float (&K)[27], float (&A)[27], float drho, float ux,
+__device__ __forceinline__ void collide_vjp(const float (&K)[27], float (&A)[27], float drho, float ux,
                                             float uy, float uz, float inv, const Keep& kf,
                                             float (&ub)[3], float (&kbar)[4],
                                             const RelaxParams* local = nullptr, float g = 0.0f) {
-  float T[27];
-  // the inverse sweeps ran z, y, x: undo x first; its input is inv_y(inv_z(relaxed))
+  // adjoint of the post-collision raw moments, and those moments themselves
+  raw_inverse_vjp<1>(A);
+  raw_inverse_vjp<3>(A);
+  raw_inverse_vjp<9>(A);
+  {
+    float T[27];
 #pragma unroll
-  for (int k = 0; k < 27; ++k) T[k] = K[k];
-  relax_to_equilibrium(T, drho, ux, uy, uz, kf);
-  inv_axis<9>(T, uz);
-  inv_axis<3>(T, uy);
-  inv_axis_vjp<1>(T, A, ux, ub[0]);
-#pragma unroll
-  for (int k = 0; k < 27; ++k) T[k] = K[k];
-  relax_to_equilibrium(T, drho, ux, uy, uz, kf);
-  inv_axis<9>(T, uz);
-  inv_axis_vjp<3>(T, A, uy, ub[1]);
-#pragma unroll
-  for (int k = 0; k < 27; ++k) T[k] = K[k];
-  relax_to_equilibrium(T, drho, ux, uy, uz, kf);
-  inv_axis_vjp<9>(T, A, uz, ub[2]);
+    for (int k = 0; k < 27; ++k) T[k] = K[k];
+    relax_to_equilibrium(T, drho, ux, uy, uz, kf);
+    unshift_axis<9>(T, uz);
+    unshift_axis<3>(T, uy);
+    unshift_axis<1>(T, ux);
+    ub[0] += shift_dot<1>(A, T);
+    ub[1] += shift_dot<3>(A, T);
+    ub[2] += shift_dot<9>(A, T);
+  }
+  unshift_axis_vjp<1>(A, ux);
+  unshift_axis_vjp<3>(A, uy);
+  unshift_axis_vjp<9>(A, uz);            // A = adjoint of the relaxed central moments
   float bar[4] = {0.f, 0.f, 0.f, 0.f};     // d/d(rho - 1), d/du
   relax_vjp(K, A, drho, ux, uy, uz, kf, bar, kbar);
   ub[0] += bar[1];
@@ -230,13 +232,12 @@ __device__ __forceinline__ void collide_vjp(float (&K)[27], float (&A)[27], floa
       ub[2] += 2.0f * c * (uz * pzz + ux * pxz + uy * pyz);
     }
   }
-  // the shifts ran x, y, z: undo z first; its input is unshift_z(K)
-  unshift_axis<9>(K, uz);
-  shift_axis_vjp<9>(K, A, uz, ub[2]);
-  unshift_axis<3>(K, uy);
-  shift_axis_vjp<3>(K, A, uy, ub[1]);
-  unshift_axis<1>(K, ux);
-  shift_axis_vjp<1>(K, A, ux, ub[0]);
+  ub[0] -= shift_dot<1>(A, K);
+  ub[1] -= shift_dot<3>(A, K);
+  ub[2] -= shift_dot<9>(A, K);
+  unshift_axis_vjp<1>(A, -ux);
+  unshift_axis_vjp<3>(A, -uy);
+  unshift_axis_vjp<9>(A, -uz);           // A = adjoint of the raw moments of the pulled set
   // u = j / rho with rho = 1 + r_000, j = (r_100, r_010, r_001)
   drhob -= (ub[0] * ux + ub[1] * uy + ub[2] * uz) * inv;
   A[kap(0, 0, 0)] += drhob;
