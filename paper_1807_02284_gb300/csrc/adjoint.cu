@@ -8,8 +8,10 @@
 //   pass A (per fluid node x): recompute the forward at x, then the exact transpose of every
 //     stage; the population adjoints go to the pull sources (the pull, with bounce-back, reads
 //     every fluid slot exactly once, so these stores never collide), and the adjoint of the
-//     adaptive factor becomes 9 per-node terms mu_ab = dL/d(U_a(x+e_b) - U_a(x-e_b));
-//   pass B (per node y): Ups^n_a(y) = sum_b mu_ab(y - e_b) - mu_ab(y + e_b) and
+//     adaptive factor becomes one per-node number ms: the adjoint of the velocity difference
+//     diff_ab = U_a(x+e_b) - U_a(x-e_b) is mu_ab = ms diff_ab;
+//   pass B (per node y): Ups^n_a(y) = sum_b mu_ab(y - e_b) - mu_ab(y + e_b), the differences
+//     formed again from U^n, and
 //     Gam^n(y) = sum over the nodes x whose departure cell touches y of w_{x->y} Gam^{n+1}(x)
 //     (a gather over the 27 neighbours: deterministic, no atomics).
 // Initial state: D^0 = f^eq(rho_0, u_0) - w and U^0 = u_0, so
@@ -48,9 +50,7 @@ struct AdjArgs {
   float* lam_out;       // Lam^n
   float* ups_out;       // Ups^n
   float* gam_out;       // Gam^n
-  float* mu;            // 9 planes: adjoint of the velocity differences of the gradient norm
-  float* sw;            // 9 planes: departure-sample weights of each sender (put_sender)
-  float* sg;            // sender's scalar adjoint, 0 for non-senders
+  float* ms;            // adjoint of the gradient norm over 4 |grad|: dL/d(diff_ab) = ms diff_ab
   float* side;          // open faces: adjoints of the clamped pulls (FaceSide layout)
 };
 
@@ -60,10 +60,10 @@ struct AdjArgs {
 // not move with u: a displacement clamped at one node, or a departure point below an open
 // face's first node (the forward pins the sample to that node; at the upper face both
 // corners already coincide).
-__device__ __forceinline__ void scalar_u_vjp(const BlockView& v, int x, int y, int z, float ux,
-                                             float uy, float uz, float gam, float (&ub)[3]) {
+__device__ __forceinline__ void scalar_u_vjp(const BlockView& v, const ScalarCell& sc, int x, int y,
+                                             int z, float ux, float uy, float uz, float gam,
+                                             float (&ub)[3]) {
   if (gam == 0.0f) return;
-  const ScalarCell sc = scalar_corners<uint32_t>(v, x, y, z, ux, uy, uz);
   const float tx = sc.tx, ty = sc.ty, tz = sc.tz;
   const float dtx = (1 - ty) * (1 - tz) * (sc.c[1] - sc.c[0]) + ty * (1 - tz) * (sc.c[3] - sc.c[2]) +
                     (1 - ty) * tz * (sc.c[5] - sc.c[4]) + ty * tz * (sc.c[7] - sc.c[6]);
@@ -77,6 +77,12 @@ __device__ __forceinline__ void scalar_u_vjp(const BlockView& v, int x, int y, i
   if (fabsf(ux) < 1.0f && !lx) ub[0] -= gam * dtx;
   if (fabsf(uy) < 1.0f && !ly) ub[1] -= gam * dty;
   if (fabsf(uz) < 1.0f && !lz) ub[2] -= gam * dtz;
+}
+
+// A float copied asynchronously from global to shared memory.
+__device__ __forceinline__ void copy_async4(float* smem, const float* g) {
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(g) : "memory");
 }
 
 // Open faces.  A pull whose source x - e_K lies outside the block along a non-periodic axis
@@ -167,11 +173,13 @@ __device__ __forceinline__ void push_all(const float (&A)[27], float* __restrict
 // adjoint of the keep factors of the high-order groups to kbar.
 // With `local` set (the strain-rate mode of the adaptive factor), the factor's input g is
 // local_strain of the central moments K, so the keep factors' adjoint flows back into K, rho
-// and u here (between the relaxation's transpose and the shifts').
+// and u here (between the relaxation's transpose and the shifts').  late(ub) adds velocity
+// terms that are wanted only before u's own transpose (their loads are in flight until then).
+template <typename Late>
 __device__ __forceinline__ void collide_vjp(const float (&K)[27], float (&A)[27], float drho, float ux,
                                             float uy, float uz, float inv, const Keep& kf,
                                             float (&ub)[3], float (&kbar)[4],
-                                            const RelaxParams* local = nullptr, float g = 0.0f) {
+                                            const RelaxParams* local, float g, Late late) {
   // adjoint of the post-collision raw moments, and those moments themselves
   raw_inverse_vjp<1>(A);
   raw_inverse_vjp<3>(A);
@@ -238,6 +246,7 @@ __device__ __forceinline__ void collide_vjp(const float (&K)[27], float (&A)[27]
   unshift_axis_vjp<1>(A, -ux);
   unshift_axis_vjp<3>(A, -uy);
   unshift_axis_vjp<9>(A, -uz);           // A = adjoint of the raw moments of the pulled set
+  late(ub);
   // u = j / rho with rho = 1 + r_000, j = (r_100, r_010, r_001)
   drhob -= (ub[0] * ux + ub[1] * uy + ub[2] * uz) * inv;
   A[kap(0, 0, 0)] += drhob;
@@ -343,45 +352,6 @@ __global__ void k_face_gather(float* __restrict__ lam, float* __restrict__ side,
   }
 }
 
-// Weight at this node of the departure sample of the node D steps away along one axis, when
-// neither clamping nor wrap-around can move that sample's cell (the axis is periodic with >= 4
-// nodes, or this node is >= 2 nodes from both ends of an open axis): the sample sits at
-// dsp = clamp(-u, -1, 1) from its node, in the cell [f, f + 1] with f = floor(dsp) and
-// fraction t = dsp - f, so this node is the cell's lower corner when f = -D (weight 1 - t) and
-// its upper corner when f = -D - 1 (weight t).  Same values as sl_axis followed by the corner
-// test of the general gather.
-template <int D>
-__device__ __forceinline__ float sl_weight_interior(float u) {
-  float dsp = -u;
-  if (!(dsp == dsp)) dsp = 0.0f;
-  dsp = fminf(fmaxf(dsp, -1.0f), 1.0f);
-  const float f = floorf(dsp);
-  const float t = dsp - f;
-  float w = f == (float)(-D) ? 1.0f - t : 0.0f;
-  if constexpr (D <= 0) w = f == (float)(-D - 1) ? t : w;
-  return w;
-}
-
-// Pass A's part of the scalar gather: this node's departure-sample weights toward the three
-// nodes that can receive from it along each axis (receiver at offset e = -1, 0, +1: plane
-// 3 a + e + 1 of sw) and its scalar adjoint in sg, 0 where the node sends nothing (obstacle,
-// scalar source, scale boundary).  Pass B's interior gather reads these instead of the
-// velocities and flags of its 27 neighbours.  Values for nodes next to an open face are not
-// used (their receivers take the general gather).
-__device__ __forceinline__ void put_sender(const AdjArgs& a, uint32_t N, uint32_t idx, float g,
-                                           float ux, float uy, float uz) {
-  const float u[3] = {ux, uy, uz};
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    a.sw[(uint32_t)(3 * c + 0) * N + idx] = sl_weight_interior<1>(u[c]);
-    a.sw[(uint32_t)(3 * c + 1) * N + idx] = sl_weight_interior<0>(u[c]);
-    a.sw[(uint32_t)(3 * c + 2) * N + idx] = sl_weight_interior<-1>(u[c]);
-  }
-  a.sg[idx] = g;
-}
-
-// MINB: CTAs per SM the register allocation is bounded for (3: no spills; 4: some spills,
-// more warps in flight); the faster one is chosen at run time.
 // The populations of a wall node (face wall or obstacle surface) pulled from beyond the wall:
 // the set wall_regularize completes (same tests).
 template <typename IT>
@@ -452,44 +422,94 @@ __device__ __forceinline__ void wall_regularize_vjp(float (&A)[27], const BlockV
   }
 }
 
-// OPEN: some face of the block is open (clamped pulls go to the side buffer).  ACC: the
-// adjoints of the input level are added to (multi-block reverse), and scale-boundary (ghost)
-// nodes, which the step does not update, are left to the mapping that wrote them.  WALLS:
-// the block has wall faces or obstacle-surface walls (wall_regularize and its transpose).
+// Pushes the adjoint of a node's pulled populations to their sources when none of them is
+// wrapped, clamped or bounced back along y or z: the offsets of pull_inner.
+template <bool ACC, int K = 0>
+__device__ __forceinline__ void push_inner(const float (&A)[27], float* __restrict__ lam, uint32_t N,
+                                           uint32_t nx, uint32_t nxy, uint32_t am, uint32_t a0,
+                                           uint32_t ap) {
+  if constexpr (K < 27) {
+    constexpr int cx = cxk(K), cy = cyk(K), cz = czk(K);
+    const uint32_t slot = ((uint32_t)K * N - (uint32_t)cz * nxy - (uint32_t)cy * nx) +
+                          (cx > 0 ? am : cx < 0 ? ap : a0);
+    if (ACC) lam[slot] += A[K];
+    else lam[slot] = A[K];
+    push_inner<ACC, K + 1>(A, lam, N, nx, nxy, am, a0, ap);
+  }
+}
+
+constexpr int ADJ_THREADS = 128;
+
+// Pass A.  OPEN: some face of the block is open (clamped pulls go to the side buffer).  ACC:
+// the adjoints of the input level are added to (multi-block reverse), and scale-boundary
+// (ghost) nodes, which the step does not update, are left to the mapping that wrote them.
+// WALLS: the block has wall faces or obstacle-surface walls (wall_regularize and its
+// transpose).
+// One thread per node, consecutive threads over the nodes of a plane (no idle lanes when nx is
+// not a multiple of the CTA).  Three 27-arrays are live in the transposed collision, which
+// holds the kernel at 16 warps per SM, too few to hide its chain of dependent loads; so
+// everything known from the node index alone is requested first (the pull and the velocity
+// neighbourhood in registers, the 31 adjoints by cp.async into this thread's shared-memory
+// column, 4 bytes each), the scalar corners as soon as u is known, and each is waited for
+// only where it is used.  128^3: 245 -> 169 us (1935 instructions per node, 63 % of issue slots,
+// 56 % of DRAM peak; before, the flags, the pull, the corners and the adjoints waited for one
+// another in turn and 19 words per node went to pass B), 72 x 60 x 51 with open faces
+// 64 -> 34 us (rows of 72 nodes left 44 % of a 128-thread row's lanes idle).
 template <int MINB, bool OPEN, bool ACC, bool WALLS>
-__global__ void __launch_bounds__(128, MINB) k_adj_a(AdjArgs a) {
+__global__ void __launch_bounds__(ADJ_THREADS, MINB) k_adj_a(AdjArgs a) {
+  __shared__ float sadj[31][ADJ_THREADS];     // lam, ups, gam of the node
+  __shared__ float scor[8][ADJ_THREADS];      // scalar corners of its departure cell
   const BlockView& v = a.fwd;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y;
-  const int z = blockIdx.z;
-  if (x >= v.nx) return;
+  const int t = threadIdx.x;
+  const uint32_t nx = (uint32_t)v.nx, nxy = nx * (uint32_t)v.ny;
+  const uint32_t i = blockIdx.x * ADJ_THREADS + t;
+  if (i >= nxy) return;
+  const int y = (int)(i / nx), x = (int)(i - (uint32_t)y * nx), z = blockIdx.y;
   const uint32_t N = (uint32_t)v.N;
-  const Nbr<uint32_t> n = neighbours<uint32_t>(v, x, y, z);
-  const uint32_t idx = n.p0 + n.r0 + n.x0;
-  const uint8_t fl = v.flags[idx];
-  // the adjoint of this node's 27 populations is needed only after the recompute: start
-  // bringing it into L2 now (measured: +1.7 % on the 128^3 reverse sweep)
+  const uint32_t idx = nxy * (uint32_t)z + i;
 #pragma unroll
-  for (int k = 0; k < 27; ++k) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.lam_in + (size_t)k * N + idx));
+  for (int k = 0; k < 27; ++k) copy_async4(&sadj[k][t], a.lam_in + ((uint32_t)k * N + idx));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) copy_async4(&sadj[27 + c][t], a.ups_in + ((uint32_t)c * N + idx));
+  copy_async4(&sadj[30][t], a.gam_in + idx);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  const uint8_t fl = __ldg(v.flags + idx);
+  const bool inner = inner_yz(v, y, z);
+  const float* __restrict__ din = static_cast<const float*>(v.d_in);
+  const uint32_t row = idx - (uint32_t)x;
+  const uint32_t am = row + (uint32_t)nbr(x, -1, v.nx, v.per[0]);
+  const uint32_t ap = row + (uint32_t)nbr(x, 1, v.nx, v.per[0]);
+  const bool local = v.rp.adaptive && v.rp.local;
+  const bool lagged = v.rp.adaptive && !local;
+  float K[27], g = 0.0f;
+  if (inner) {
+    pull_inner<float, uint32_t>(K, din, N, nx, nxy, am, idx, ap);
+    if (lagged) g = grad_norm_inner<uint32_t>(v.u_in, N, nx, nxy, idx, am, ap);
+  } else {
+    const Nbr<uint32_t> n = neighbours<uint32_t>(v, x, y, z);
+    pull_all<float, uint32_t>(K, din, N, n);
+    if (lagged) g = grad_norm<uint32_t>(v.u_in, N, n);
+  }
   if ((fl & F_SOLID) || (ACC && (fl & F_GHOST))) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a.mu[(uint32_t)i * N + idx] = 0.0f;
-    put_sender(a, N, idx, 0.0f, 0.0f, 0.0f, 0.0f);
+    a.ms[idx] = 0.0f;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     return;
   }
   if (fl & F_INFLOW) {
     // D^{n+1} = f^eq(1, U^n) - w, U^{n+1} = U^n, C^{n+1} sampled at x - U^n: the pulled
     // populations are unused (their slots get a zero adjoint) and every adjoint goes to U^n,
     // which pass B completes with the lagged-gradient terms of the neighbours
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     const float u[3] = {v.u_in[idx], v.u_in[N + idx], v.u_in[2 * N + idx]};
-    put_sender(a, N, idx, (fl & F_SCALAR_SRC) ? 0.0f : a.gam_in[idx], u[0], u[1], u[2]);
-    float ub[3] = {a.ups_in[idx], a.ups_in[N + idx], a.ups_in[2 * N + idx]};
-    if (!(fl & F_SCALAR_SRC)) scalar_u_vjp(v, x, y, z, u[0], u[1], u[2], a.gam_in[idx], ub);
+    float ub[3] = {sadj[27][t], sadj[28][t], sadj[29][t]};
+    if (!(fl & F_SCALAR_SRC))
+      scalar_u_vjp(v, scalar_corners<uint32_t>(v, x, y, z, u[0], u[1], u[2]), x, y, z, u[0], u[1],
+                   u[2], sadj[30][t], ub);
 #pragma unroll
     for (int k = 0; k < 27; ++k) {
       const float c[3] = {(float)cxk(k), (float)cyk(k), (float)czk(k)};
       const float cu = c[0] * u[0] + c[1] * u[1] + c[2] * u[2];
-      const float l = a.lam_in[(uint32_t)k * N + idx] * wk(k);
+      const float l = sadj[k][t] * wk(k);
 #pragma unroll
       for (int a2 = 0; a2 < 3; ++a2) ub[a2] = fmaf(l, 3.0f * c[a2] + 9.0f * cu * c[a2] - 3.0f * u[a2], ub[a2]);
     }
@@ -504,75 +524,65 @@ __global__ void __launch_bounds__(128, MINB) k_adj_a(AdjArgs a) {
       float Z[27];
 #pragma unroll
       for (int k = 0; k < 27; ++k) Z[k] = 0.0f;
-      push_all<OPEN, false>(Z, a.lam_out, N, n, idx, v.flags, (fl & F_NEAR_SOLID) != 0,
-                            clamp_mask<OPEN>(v, x, y, z), v, x, y, z, a.side);
+      push_all<OPEN, false>(Z, a.lam_out, N, neighbours<uint32_t>(v, x, y, z), idx, v.flags,
+                            (fl & F_NEAR_SOLID) != 0, clamp_mask<OPEN>(v, x, y, z), v, x, y, z, a.side);
     }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a.mu[(uint32_t)i * N + idx] = 0.0f;
+    a.ms[idx] = 0.0f;
     return;
   }
-  const float* __restrict__ din = static_cast<const float*>(v.d_in);
 
   // ---- forward recompute up to the central moments
-  float K[27];
-  pull_all<float, uint32_t>(K, din, N, n);
   // as in cell_update: an obstacle wall node completes what comes from inside the obstacle
   // itself (no bounce-back), every wall node is regularized before the collision
   const bool near = (fl & F_NEAR_SOLID) != 0 && !(WALLS && (fl & F_OBST_WALL));
-  if (near) bounce_back<float, uint32_t>(K, din, N, v.flags, n, idx);
+  if (near) bounce_back<float, uint32_t>(K, din, N, v.flags, neighbours<uint32_t>(v, x, y, z), idx);
   const bool wall = WALLS && (fl & (F_WALL | F_OBST_WALL));
   if constexpr (WALLS) {
-    if (wall) wall_regularize<uint32_t>(K, v, x, y, z, fl, n);
+    if (wall) wall_regularize<uint32_t>(K, v, x, y, z, fl, neighbours<uint32_t>(v, x, y, z));
   }
   raw_moments(K);
   const float drho = K[kap(0, 0, 0)];
   const float inv = fast_rcp(1.0f + drho);
   const float ux = K[kap(1, 0, 0)] * inv, uy = K[kap(0, 1, 0)] * inv, uz = K[kap(0, 0, 1)] * inv;
-  put_sender(a, N, idx, (fl & F_SCALAR_SRC) ? 0.0f : a.gam_in[idx], ux, uy, uz);
-  float diff[9];
-  float g = 0.0f;
-  const bool local = v.rp.adaptive && v.rp.local;
-  if (v.rp.adaptive && !local) {
-    float s = 0.0f;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float* Uc = v.u_in + (uint32_t)c * N;
-      diff[3 * c + 0] = __ldg(Uc + (n.p0 + n.r0 + n.xp)) - __ldg(Uc + (n.p0 + n.r0 + n.xm));
-      diff[3 * c + 1] = __ldg(Uc + (n.p0 + n.rp + n.x0)) - __ldg(Uc + (n.p0 + n.rm + n.x0));
-      diff[3 * c + 2] = __ldg(Uc + (n.pp + n.r0 + n.x0)) - __ldg(Uc + (n.pm + n.r0 + n.x0));
-      s = fmaf(diff[3 * c + 0], diff[3 * c + 0],
-               fmaf(diff[3 * c + 1], diff[3 * c + 1], fmaf(diff[3 * c + 2], diff[3 * c + 2], s)));
-    }
-    g = 0.5f * sqrtf(s);
-  }
-  shift_axis<1>(K, ux);
-  shift_axis<3>(K, uy);
-  shift_axis<9>(K, uz);                  // K = central moments before relaxation
+  const bool src = (fl & F_SCALAR_SRC) != 0;
+  if (!src) scalar_corners_async<uint32_t>(v, x, y, z, ux, uy, uz, &scor[0][t], ADJ_THREADS);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  central_from_raw(K, ux, uy, uz);       // K = central moments before relaxation
   if (local) g = local_strain(K, drho, ux, uy, uz, v.rp.s_nu);
   const Keep kf = keep_factors(v.rp, g);
 
-  // ---- adjoint of the stored velocity and of the scalar step
-  float ub[3];
-  ub[0] = a.ups_in[idx];
-  ub[1] = a.ups_in[N + idx];
-  ub[2] = a.ups_in[2 * N + idx];
-  if (!(fl & F_SCALAR_SRC)) scalar_u_vjp(v, x, y, z, ux, uy, uz, a.gam_in[idx], ub);
-
-  // ---- adjoint of the collision
+  // ---- adjoint of the collision, of the stored velocity and of the scalar step
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
   float A[27];
 #pragma unroll
-  for (int k = 0; k < 27; ++k) A[k] = a.lam_in[(uint32_t)k * N + idx];
+  for (int k = 0; k < 27; ++k) A[k] = sadj[k][t];
+  float ub[3] = {sadj[27][t], sadj[28][t], sadj[29][t]};
   float kbar[4] = {0.f, 0.f, 0.f, 0.f};    // d/d(keep factor) of the high-order groups
-  collide_vjp(K, A, drho, ux, uy, uz, inv, kf, ub, kbar, local ? &v.rp : nullptr, g);
+  collide_vjp(K, A, drho, ux, uy, uz, inv, kf, ub, kbar, local ? &v.rp : nullptr, g,
+              [&](float (&b)[3]) {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                if (src) return;
+                ScalarCell sc;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) sc.c[c] = scor[c][t];
+                sc.tx = sl_axis(x, ux, v.nx, v.per[0]).t;
+                sc.ty = sl_axis(y, uy, v.ny, v.per[1]).t;
+                sc.tz = sl_axis(z, uz, v.nz, v.per[2]).t;
+                scalar_u_vjp(v, sc, x, y, z, ux, uy, uz, sadj[30][t], b);
+              });
   if constexpr (WALLS) {
-    if (wall) wall_regularize_vjp<uint32_t>(A, v, x, y, z, fl, n);
+    if (wall) wall_regularize_vjp<uint32_t>(A, v, x, y, z, fl, neighbours<uint32_t>(v, x, y, z));
   }
-  push_all<OPEN, ACC>(A, a.lam_out, N, n, idx, v.flags, near, clamp_mask<OPEN>(v, x, y, z), v, x,
-                      y, z, a.side);
+  const ClampMask cm = clamp_mask<OPEN>(v, x, y, z);
+  if (inner && !near && cm == 0u)
+    push_inner<ACC>(A, a.lam_out, N, nx, nxy, am, idx, ap);
+  else
+    push_all<OPEN, ACC>(A, a.lam_out, N, neighbours<uint32_t>(v, x, y, z), idx, v.flags, near, cm, v,
+                        x, y, z, a.side);
 
   // ---- adjoint of the adaptive factor: K_g = 1 - 1/(phi nu3_g + 1/2)
-  float mu_scale = 0.0f;          // (the local-strain mode has no lagged-velocity dependence)
-  if (v.rp.adaptive && !local && g > 0.0f && g * v.rp.inv_gmax < 1.0f) {
+  float ms = 0.0f;                // (the local-strain mode has no lagged-velocity dependence)
+  if (lagged && g > 0.0f && g * v.rp.inv_gmax < 1.0f) {
     float phib = 0.0f;
 #pragma unroll
     for (int gi = 0; gi < 4; ++gi) {
@@ -580,15 +590,252 @@ __global__ void __launch_bounds__(128, MINB) k_adj_a(AdjArgs a) {
       phib = fmaf(kbar[gi], v.rp.nuh3[gi] * S * S, phib);
     }
     const float gb = phib * v.rp.a * v.rp.inv_gmax;   // phi = a g / g_max + b below the clamp
-    mu_scale = gb * 0.25f / g;                        // dg/d(diff) = diff / (4 g)
+    ms = gb * 0.25f / g;                              // dg/d(diff) = diff / (4 g)
   }
+  a.ms[idx] = ms;
+}
+
+// A node as sender of the scalar gather along one axis: its departure sample sits dsp =
+// clamp(-u, -1, 1) away and is shared between two neighbouring nodes by the hat weights
+// max(0, -dsp), 1 - |dsp|, max(0, dsp) of the nodes -1, 0, +1 away.  On an open face a sample
+// beyond the face is pinned to the face's node: dsp is bounded by 0 on that side.
+struct SenderAxis {
+  float lo, hi;
+};
+__device__ __forceinline__ SenderAxis sender_axis(int c, int n, int periodic) {
+  return SenderAxis{!periodic && c == 0 ? 0.0f : -1.0f, !periodic && c == n - 1 ? 0.0f : 1.0f};
+}
+__device__ __forceinline__ void sender_weights(const SenderAxis& s, float u, float (&w)[3]) {
+  const float dsp = fminf(fmaxf(-u, s.lo), s.hi);
+  w[0] = fmaxf(-dsp, 0.0f);
+  w[1] = 1.0f - fabsf(dsp);
+  w[2] = fmaxf(dsp, 0.0f);
+}
+
+// The nodes -2, -1, +1, +2 away along one axis as wrapped or clamped indices, and the signs of
+// the neighbours' difference adjoints: node q's difference along the axis is U(q+1) - U(q-1) with
+// the indices wrapped or clamped, so node c receives +mu(c - 1) and -mu(c + 1) where those nodes
+// exist, and on an open face also its own +mu (upper: its + neighbour is itself) or -mu (lower).
+struct AxisStar {
+  int m2, m1, p1, p2;
+  float wm, wp, own;
+};
+__device__ __forceinline__ AxisStar axis_star(int c, int n, int periodic) {
+  AxisStar s;
+  s.m1 = nbr(c, -1, n, periodic);
+  s.p1 = nbr(c, 1, n, periodic);
+  s.m2 = nbr(s.m1, -1, n, periodic);
+  s.p2 = nbr(s.p1, 1, n, periodic);
+  s.wm = periodic || c > 0 ? 1.0f : 0.0f;
+  s.wp = periodic || c < n - 1 ? 1.0f : 0.0f;
+  s.own = periodic ? 0.0f : (c == 0 ? -1.0f : (c == n - 1 ? 1.0f : 0.0f));
+  return s;
+}
+
+constexpr int ADJ_BX = 32, ADJ_BY = 8;                     // receivers of one plane of a CTA
+constexpr int ADJ_SX = ADJ_BX + 2, ADJ_SENDERS = ADJ_SX * (ADJ_BY + 2);
+
+// A column of senders (fixed x, y): its offset in a plane, its bounds along x and y, and
+// whether it lies in the block (a tile may reach past nx or ny, or beyond an open face).
+struct SenderColumn {
+  uint32_t off;
+  SenderAxis x, y;
+  bool in;
+};
+// What a sender holds: its scalar adjoint (0 where it sends nothing: obstacle, scalar source,
+// scale boundary, outside the block) and its departure velocity.
+struct Sender {
+  float g, u[3];
+};
+
+__device__ __forceinline__ SenderColumn sender_column(const BlockView& v, int x, int y) {
+  if (v.per[0]) x += x < 0 ? v.nx : (x == v.nx ? -v.nx : 0);
+  if (v.per[1]) y += y < 0 ? v.ny : (y == v.ny ? -v.ny : 0);
+  SenderColumn c;
+  c.in = x >= 0 && x < v.nx && y >= 0 && y < v.ny;
+  c.off = c.in ? (uint32_t)y * (uint32_t)v.nx + (uint32_t)x : 0u;
+  c.x = sender_axis(x, v.nx, v.per[0]);
+  c.y = sender_axis(y, v.ny, v.per[1]);
+  return c;
+}
+
+__device__ __forceinline__ Sender load_sender(const AdjArgs& a, const SenderColumn& c, int z) {
+  const BlockView& v = a.fwd;
+  Sender s{0.0f, {0.0f, 0.0f, 0.0f}};
+  if (v.per[2]) z += z < 0 ? v.nz : (z >= v.nz ? -v.nz : 0);
+  if (c.in && z >= 0 && z < v.nz) {
+    const uint32_t N = (uint32_t)v.N;
+    const uint32_t j = (uint32_t)z * ((uint32_t)v.nx * (uint32_t)v.ny) + c.off;
+    const float g = __ldg(a.gam_in + j);
+    s.g = (__ldg(v.flags + j) & (F_SOLID | F_SCALAR_SRC | F_GHOST)) ? 0.0f : g;
+    s.u[0] = __ldg(a.u_next + j);
+    s.u[1] = __ldg(a.u_next + (N + j));
+    s.u[2] = __ldg(a.u_next + (2 * N + j));
+  }
+  return s;
+}
+
+// The lagged velocity's adjoint at one node: the six neighbours' (and on an open face its own)
+// difference adjoints.  Inflow nodes add it to what pass A left there.  INNER: the node is at
+// least two nodes from both ends along y and z, so those neighbours are plain offsets.
+template <bool ACC, bool INNER>
+__device__ __forceinline__ void lagged_adjoint(const AdjArgs& a, int x, int y, int z, uint32_t idx) {
+  const BlockView& v = a.fwd;
+  const uint32_t N = (uint32_t)v.N, nx = (uint32_t)v.nx, nxy = nx * (uint32_t)v.ny;
+  const AxisStar ax = axis_star(x, v.nx, v.per[0]);
+  const uint32_t row = idx - (uint32_t)x;
+  const uint32_t xm2 = row + ax.m2, xm1 = row + ax.m1, xp1 = row + ax.p1, xp2 = row + ax.p2;
+  uint32_t ym2, ym1, yp1, yp2, zm2, zm1, zp1, zp2;
+  AxisStar ay, az;
+  if constexpr (INNER) {
+    ym2 = idx - 2 * nx; ym1 = idx - nx; yp1 = idx + nx; yp2 = idx + 2 * nx;
+    zm2 = idx - 2 * nxy; zm1 = idx - nxy; zp1 = idx + nxy; zp2 = idx + 2 * nxy;
+    ay.wm = ay.wp = az.wm = az.wp = 1.0f;
+    ay.own = az.own = 0.0f;
+  } else {
+    ay = axis_star(y, v.ny, v.per[1]);
+    az = axis_star(z, v.nz, v.per[2]);
+    const uint32_t oy = idx - nx * (uint32_t)y, oz = idx - nxy * (uint32_t)z;
+    ym2 = oy + nx * (uint32_t)ay.m2; ym1 = oy + nx * (uint32_t)ay.m1;
+    yp1 = oy + nx * (uint32_t)ay.p1; yp2 = oy + nx * (uint32_t)ay.p2;
+    zm2 = oz + nxy * (uint32_t)az.m2; zm1 = oz + nxy * (uint32_t)az.m1;
+    zp1 = oz + nxy * (uint32_t)az.p1; zp2 = oz + nxy * (uint32_t)az.p2;
+  }
+  const float* __restrict__ ms = a.ms;
+  const float mx = ax.wm * __ldg(ms + xm1), px = ax.wp * __ldg(ms + xp1);
+  const float my = ay.wm * __ldg(ms + ym1), py = ay.wp * __ldg(ms + yp1);
+  const float mz = az.wm * __ldg(ms + zm1), pz = az.wp * __ldg(ms + zp1);
+  const bool face = ax.own != 0.0f || ay.own != 0.0f || az.own != 0.0f;
+  const bool keep = ACC || (__ldg(v.flags + idx) & (F_INFLOW | F_SOLID)) == F_INFLOW;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) a.mu[(uint32_t)i * N + idx] = (v.rp.adaptive && !local) ? mu_scale * diff[i] : 0.0f;
+  for (int k = 0; k < 3; ++k) {
+    const float* __restrict__ U = v.u_in + (uint32_t)k * N;
+    const float c = __ldg(U + idx);
+    float sum = mx * (c - __ldg(U + xm2));
+    sum = fmaf(-px, __ldg(U + xp2) - c, sum);
+    sum = fmaf(my, c - __ldg(U + ym2), sum);
+    sum = fmaf(-py, __ldg(U + yp2) - c, sum);
+    sum = fmaf(mz, c - __ldg(U + zm2), sum);
+    sum = fmaf(-pz, __ldg(U + zp2) - c, sum);
+    if (face) {
+      const float own = __ldg(ms + idx);
+      sum = fmaf(own * ax.own, __ldg(U + xp1) - __ldg(U + xm1), sum);
+      sum = fmaf(own * ay.own, __ldg(U + yp1) - __ldg(U + ym1), sum);
+      sum = fmaf(own * az.own, __ldg(U + zp1) - __ldg(U + zm1), sum);
+    }
+    float* o = a.ups_out + ((uint32_t)k * N + idx);
+    *o = keep ? *o + sum : sum;
+  }
+}
+
+// Pass B, lagged velocity (only where the adaptive factor depends on it): one thread per node
+// without shared memory, so that enough warps are resident to cover its 27 loads (as part of
+// the marching kernel below they were waited for plane by plane: 128^3 76 us together, 33 + 33
+// us apart; 90 us before the two were rewritten).
+template <bool ACC>
+__global__ void __launch_bounds__(256, 6) k_adj_lagged(AdjArgs a) {
+  const BlockView& v = a.fwd;
+  const uint32_t nx = (uint32_t)v.nx, nxy = nx * (uint32_t)v.ny;
+  const uint32_t i = blockIdx.x * 256u + threadIdx.x;
+  if (i >= nxy) return;
+  const int z = blockIdx.y, y = (int)(i / nx), x = (int)(i - nx * (uint32_t)y);
+  const uint32_t idx = nxy * (uint32_t)z + i;
+  if (y >= 2 && y < v.ny - 2 && z >= 2 && z < v.nz - 2) lagged_adjoint<ACC, true>(a, x, y, z, idx);
+  else lagged_adjoint<ACC, false>(a, x, y, z, idx);
+}
+
+// Pass B, scalar.  A CTA covers 32 x 8 receivers and marches `zc` planes in z.  Every node of
+// the tile and its halo is a sender: its three weights along x and the nine products of its y
+// and z weights with its scalar adjoint go to shared memory once per plane (a ring of three
+// planes, 48 KB), and a receiver adds 27 products of two shared-memory values.  Before, pass A
+// stored nine weights per node and every receiver fetched four values from each of its 27
+// neighbours through L1 (923 instructions per node, latency-bound).  The next plane's senders
+// are loaded into registers before the current plane's sums.  LAGGED false: no k_adj_lagged
+// ran, so ups_out is set here.
+template <bool ACC, bool LAGGED>
+__global__ void __launch_bounds__(ADJ_BX * ADJ_BY) k_adj_b(AdjArgs a, int zc) {
+  __shared__ float ring[3][12][ADJ_SENDERS];     // wx(-1, 0, +1), then wy wz g: 3 ez + ey
+  const BlockView& v = a.fwd;
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * ADJ_BX + tx;
+  const int x0 = blockIdx.x * ADJ_BX, y0 = blockIdx.y * ADJ_BY;
+  const int x = x0 + tx, y = y0 + ty;
+  const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, v.nz);
+  const bool mine = x < v.nx && y < v.ny;
+  const uint32_t N = (uint32_t)v.N, nx = (uint32_t)v.nx, nxy = nx * (uint32_t)v.ny;
+  // this thread's senders of a plane: slots tid and tid + 256 (the latter for tid < 84)
+  const int sb = tid + ADJ_BX * ADJ_BY;
+  const bool two = sb < ADJ_SENDERS;
+  const SenderColumn ca = sender_column(v, x0 - 1 + tid % ADJ_SX, y0 - 1 + tid / ADJ_SX);
+  const SenderColumn cb = sender_column(v, x0 - 1 + sb % ADJ_SX, y0 - 1 + sb / ADJ_SX);
+  auto put = [&](int slot, int at, const SenderColumn& c, int z, const Sender& s) {
+    float wx[3], wy[3], wz[3];
+    sender_weights(c.x, s.u[0], wx);
+    sender_weights(c.y, s.u[1], wy);
+    sender_weights(sender_axis(z, v.nz, v.per[2]), s.u[2], wz);
+    float* o = &ring[slot][0][at];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) o[e * ADJ_SENDERS] = wx[e];
+#pragma unroll
+    for (int ez = 0; ez < 3; ++ez) {
+      const float gz = wz[ez] * s.g;
+#pragma unroll
+      for (int ey = 0; ey < 3; ++ey) o[(3 + 3 * ez + ey) * ADJ_SENDERS] = wy[ey] * gz;
+    }
+  };
+  for (int p = -1; p <= 0; ++p) {
+    put(p + 1, tid, ca, z0 + p, load_sender(a, ca, z0 + p));
+    if (two) put(p + 1, sb, cb, z0 + p, load_sender(a, cb, z0 + p));
+  }
+  Sender na = load_sender(a, ca, z0 + 1), nb{};
+  if (two) nb = load_sender(a, cb, z0 + 1);
+  int lo = 0;                                    // ring slot of plane z - 1
+  for (int z = z0; z < z1; ++z) {
+    const int mid = lo == 2 ? 0 : lo + 1, hi = mid == 2 ? 0 : mid + 1;
+    put(hi, tid, ca, z + 1, na);
+    if (two) put(hi, sb, cb, z + 1, nb);
+    __syncthreads();
+    if (z + 1 < z1) {
+      na = load_sender(a, ca, z + 2);
+      if (two) nb = load_sender(a, cb, z + 2);
+    }
+    if (mine) {
+      const uint32_t idx = nxy * (uint32_t)z + nx * (uint32_t)y + (uint32_t)x;
+      if constexpr (!LAGGED && !ACC) {
+        if ((__ldg(v.flags + idx) & (F_INFLOW | F_SOLID)) != F_INFLOW) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) a.ups_out[(uint32_t)k * N + idx] = 0.0f;
+        }
+      }
+      // scalar adjoint: the sender at offset (dx, dy, dz) sends to offset -d
+      float part[3] = {0.0f, 0.0f, 0.0f};        // one chain per plane
+      const int at = (ty + 1) * ADJ_SX + tx + 1;
+#pragma unroll
+      for (int dz = -1; dz <= 1; ++dz) {
+        const float(*R)[ADJ_SENDERS] = ring[dz < 0 ? lo : (dz == 0 ? mid : hi)];
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+          for (int dx = -1; dx <= 1; ++dx) {
+            const int s = at + dy * ADJ_SX + dx;
+            part[dz + 1] = fmaf(R[1 - dx][s], R[3 + 3 * (1 - dz) + (1 - dy)][s], part[dz + 1]);
+          }
+      }
+      const float gam = (part[0] + part[1]) + part[2];
+      a.gam_out[idx] = ACC ? a.gam_out[idx] + gam : gam;
+    }
+    __syncthreads();                             // plane z - 1's slot is overwritten next
+    lo = mid;
+  }
+}
+
+// Grids of the two passes.
+static dim3 pass_a_grid(const BlockView& v) {
+  return dim3((unsigned)(((size_t)v.nx * v.ny + ADJ_THREADS - 1) / ADJ_THREADS), (unsigned)v.nz, 1);
 }
 
 template <bool WALLS>
-static void launch_pass_a_t(const AdjArgs& a, int minb, bool open, dim3 grd, dim3 blk,
-                            cudaStream_t s, bool acc) {
+static void launch_pass_a_t(const AdjArgs& a, int minb, bool open, cudaStream_t s, bool acc) {
+  const dim3 grd = pass_a_grid(a.fwd), blk(ADJ_THREADS, 1, 1);
   if (acc) {   // multi-block reverse: 3 CTAs/SM, open faces (every refined block has them)
     if (open) k_adj_a<3, true, true, WALLS><<<grd, blk, 0, s>>>(a);
     else k_adj_a<3, false, true, WALLS><<<grd, blk, 0, s>>>(a);
@@ -601,107 +848,30 @@ static void launch_pass_a_t(const AdjArgs& a, int minb, bool open, dim3 grd, dim
   }
 }
 
-static void launch_pass_a(const AdjArgs& a, int minb, bool open, dim3 grd, dim3 blk, cudaStream_t s,
-                          bool acc = false) {
-  if (a.fwd.walls) launch_pass_a_t<true>(a, minb, open, grd, blk, s, acc);
-  else launch_pass_a_t<false>(a, minb, open, grd, blk, s, acc);
+static void launch_pass_a(const AdjArgs& a, int minb, bool open, cudaStream_t s, bool acc = false) {
+  if (a.fwd.walls) launch_pass_a_t<true>(a, minb, open, s, acc);
+  else launch_pass_a_t<false>(a, minb, open, s, acc);
 }
 
 template <bool ACC>
-__global__ void __launch_bounds__(128) k_adj_b(AdjArgs a) {
+static void launch_pass_b(const AdjArgs& a, cudaStream_t s) {
   const BlockView& v = a.fwd;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y;
-  const int z = blockIdx.z;
-  if (x >= v.nx) return;
-  const uint32_t N = (uint32_t)v.N;
-  const Nbr<uint32_t> n = neighbours<uint32_t>(v, x, y, z);
-  const uint32_t idx = n.p0 + n.r0 + n.x0;
-  // lagged-velocity adjoint (inflow nodes add it to what pass A left there)
-  const bool inflow = (v.flags[idx] & (F_INFLOW | F_SOLID)) == F_INFLOW;
-  // node q's difference along axis b is U(q+e_b) - U(q-e_b) with the indices wrapped or
-  // clamped: this node receives +mu_b(q) from q = this - e_b and -mu_b(q) from q = this + e_b
-  // when those nodes exist, and on an open face also its own +mu_b (top: its + neighbour is
-  // itself) or -mu_b (bottom: its - neighbour is itself)
-  const int cc[3] = {x, y, z}, nn[3] = {v.nx, v.ny, v.nz};
-  float wm[3], wp[3], ws[3];            // weights of mu(this - e_b), mu(this + e_b), mu(this)
-#pragma unroll
-  for (int b = 0; b < 3; ++b) {
-    const bool per = v.per[b] != 0;
-    wm[b] = (per || cc[b] > 0) ? 1.0f : 0.0f;
-    wp[b] = (per || cc[b] < nn[b] - 1) ? -1.0f : 0.0f;
-    ws[b] = per ? 0.0f : (cc[b] == nn[b] - 1 ? 1.0f : 0.0f) - (cc[b] == 0 ? 1.0f : 0.0f);
+  const unsigned gx = (unsigned)(v.nx + ADJ_BX - 1) / ADJ_BX, gy = (unsigned)(v.ny + ADJ_BY - 1) / ADJ_BY;
+  // planes per CTA: the waves of 4 CTAs on each of 152 SMs times the sender planes of a CTA
+  int zc = 1;
+  size_t best = ~(size_t)0;
+  for (int c = 2; c <= 32; ++c) {
+    const size_t ctas = (size_t)gx * gy * ((v.nz + c - 1) / c);
+    const size_t cost = (ctas + 607) / 608 * (size_t)(c + 2);
+    if (cost < best) { best = cost; zc = c; }
   }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const float* m0 = a.mu + (uint32_t)(3 * c + 0) * N;
-    const float* m1 = a.mu + (uint32_t)(3 * c + 1) * N;
-    const float* m2 = a.mu + (uint32_t)(3 * c + 2) * N;
-    float s = wm[0] * __ldg(m0 + (n.p0 + n.r0 + n.xm)) + wp[0] * __ldg(m0 + (n.p0 + n.r0 + n.xp)) +
-              wm[1] * __ldg(m1 + (n.p0 + n.rm + n.x0)) + wp[1] * __ldg(m1 + (n.p0 + n.rp + n.x0)) +
-              wm[2] * __ldg(m2 + (n.pm + n.r0 + n.x0)) + wp[2] * __ldg(m2 + (n.pp + n.r0 + n.x0));
-    s = fmaf(ws[0], __ldg(m0 + idx), fmaf(ws[1], __ldg(m1 + idx), fmaf(ws[2], __ldg(m2 + idx), s)));
-    a.ups_out[(uint32_t)c * N + idx] = (ACC || inflow) ? a.ups_out[(uint32_t)c * N + idx] + s : s;
+  const dim3 grd(gx, gy, (unsigned)((v.nz + zc - 1) / zc)), blk(ADJ_BX, ADJ_BY, 1);
+  if (v.rp.adaptive && !v.rp.local) {
+    k_adj_lagged<ACC><<<dim3((unsigned)(((size_t)v.nx * v.ny + 255) / 256), (unsigned)v.nz, 1), 256, 0, s>>>(a);
+    k_adj_b<ACC, true><<<grd, blk, 0, s>>>(a, zc);
+  } else {
+    k_adj_b<ACC, false><<<grd, blk, 0, s>>>(a, zc);
   }
-  // scalar adjoint: gather from the neighbours whose departure cell contains this node
-  const uint32_t xs[3] = {n.xm, n.x0, n.xp};
-  const uint32_t rs[3] = {n.rm, n.r0, n.rp};
-  const uint32_t ps[3] = {n.pm, n.p0, n.pp};
-  bool interior = true;
-#pragma unroll
-  for (int b = 0; b < 3; ++b)
-    interior = interior && (v.per[b] ? nn[b] >= 4 : (cc[b] >= 2 && cc[b] <= nn[b] - 3));
-  if (interior) {
-    // every neighbour is distinct and its sample's cell neither clamps nor wraps; the sum
-    // runs over the 27 neighbours in the order of the general gather below, a skipped
-    // neighbour adding 0
-    float gam = 0.0f;
-#pragma unroll
-    for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-      for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx) {
-          // neighbour j = this + (dx - 1, dy - 1, dz - 1) sends to offset e = 1 - d: its
-          // weights were stored by pass A (put_sender), plane 3 axis + 2 - d
-          const uint32_t j = ps[dz] + rs[dy] + xs[dx];
-          const float G = __ldg(a.sg + j);
-          const float wx = __ldg(a.sw + (uint32_t)(0 + 2 - dx) * N + j);
-          const float wy = __ldg(a.sw + (uint32_t)(3 + 2 - dy) * N + j);
-          const float wz = __ldg(a.sw + (uint32_t)(6 + 2 - dz) * N + j);
-          gam = fmaf(wx * wy * wz, G, gam);
-        }
-    a.gam_out[idx] = ACC ? a.gam_out[idx] + gam : gam;
-    return;
-  }
-  const int cx[3] = {(int)n.xm, x, (int)n.xp};
-  const int cy[3] = {(int)(n.rm / (uint32_t)v.nx), y, (int)(n.rp / (uint32_t)v.nx)};
-  const int cz[3] = {(int)(n.pm / ((uint32_t)v.nx * v.ny)), z, (int)(n.pp / ((uint32_t)v.nx * v.ny))};
-  float gam = 0.0f;
-#pragma unroll
-  for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-    for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-      for (int dx = 0; dx < 3; ++dx) {
-        // a clamped neighbour index repeats the node itself: count every node once
-        if ((dx == 0 && xs[0] == xs[1]) || (dx == 2 && xs[2] == xs[1]) ||
-            (dy == 0 && rs[0] == rs[1]) || (dy == 2 && rs[2] == rs[1]) ||
-            (dz == 0 && ps[0] == ps[1]) || (dz == 2 && ps[2] == ps[1]))
-          continue;
-        const uint32_t j = ps[dz] + rs[dy] + xs[dx];
-        if (__ldg(v.flags + j) & (F_SOLID | F_SCALAR_SRC | F_GHOST)) continue;
-        const float G = __ldg(a.gam_in + j);
-        if (G == 0.0f) continue;
-        const Axis1 ax = sl_axis(cx[dx], __ldg(a.u_next + j), v.nx, v.per[0]);
-        const Axis1 ay = sl_axis(cy[dy], __ldg(a.u_next + N + j), v.ny, v.per[1]);
-        const Axis1 az = sl_axis(cz[dz], __ldg(a.u_next + 2 * N + j), v.nz, v.per[2]);
-        const float wx = (ax.i0 == x ? 1.0f - ax.t : 0.0f) + (ax.i1 == x ? ax.t : 0.0f);
-        const float wy = (ay.i0 == y ? 1.0f - ay.t : 0.0f) + (ay.i1 == y ? ay.t : 0.0f);
-        const float wz = (az.i0 == z ? 1.0f - az.t : 0.0f) + (az.i1 == z ? az.t : 0.0f);
-        gam = fmaf(wx * wy * wz, G, gam);
-      }
-  a.gam_out[idx] = ACC ? a.gam_out[idx] + gam : gam;
 }
 
 // dL/du_0 = Ups^0 + (dD^0/du_0)^T Lam^0 with D^0_k = w_k (drho + rho (3 cu + 9/2 cu^2 - 3/2 u^2)).
@@ -813,7 +983,8 @@ __global__ void __launch_bounds__(128) k_map_vjp(MapArgs a, AdjLevel dst, AdjLev
   kf.nu = a.khat;
   kf.g[0] = kf.g[1] = kf.g[2] = kf.g[3] = 1.0f;
   float kbar[4] = {0.f, 0.f, 0.f, 0.f};
-  collide_vjp(K, A, drho, ux, uy, uz, inv, kf, ub, kbar);   // A = adjoint of the interpolant
+  collide_vjp(K, A, drho, ux, uy, uz, inv, kf, ub, kbar, nullptr, 0.0f,
+              [](float (&)[3]) {});                       // A = adjoint of the interpolant
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const float wc = w[c] * inv_w;
@@ -899,7 +1070,7 @@ struct TapeState {
   float* lam[2] = {nullptr, nullptr};
   float* ups[2] = {nullptr, nullptr};
   float* gam[2] = {nullptr, nullptr};
-  float* mu = nullptr;
+  float* ms = nullptr;
   float* side = nullptr;      // clamped pulls of open faces (all zeros between launches)
   // continuous-scale domains (several blocks)
   bool multi = false;
@@ -931,7 +1102,7 @@ void release_tape(lbm_domain* dom) {
     dom->dev_free(t->ups[i]);
     dom->dev_free(t->gam[i]);
   }
-  dom->dev_free(t->mu);
+  dom->dev_free(t->ms);
   dom->dev_free(t->side);
   for (auto& v : t->mck) for (Level& L : v) free_level(dom, L);
   for (auto& v : t->snap) for (Level& L : v) free_level(dom, L);
@@ -1225,20 +1396,17 @@ static cudaError_t ms_reverse_op(lbm_domain* dom, TapeState* t, const MsOp& o, c
   a.lam_in = lout.f; a.ups_in = lout.u; a.gam_in = lout.c;
   a.u_next = u_next;
   a.lam_out = lin.f; a.ups_out = lin.u; a.gam_out = lin.c;
-  a.mu = t->mu;
-  a.sw = t->mu + 9 * N;
-  a.sg = t->mu + 18 * N;
+  a.ms = t->ms;
   a.side = t->side;
   const bool open = o.b != 0 || !dom->desc.periodic[0] || !dom->desc.periodic[1] || !dom->desc.periodic[2];
-  const dim3 blk(128, 1, 1), grd((B.nx + 127) / 128, B.ny, B.nz);
-  launch_pass_a(a, 3, open, grd, blk, s, true);
+  launch_pass_a(a, 3, open, s, true);
   if (open) {
     const int px = a.fwd.per[0], py = a.fwd.per[1], pz = a.fwd.per[2];
     const int per3[3] = {px, py, pz};
     const int fg = (int)std::max<size_t>(1, std::min<size_t>((open_face_threads(B.nx, B.ny, B.nz, per3) + 255) / 256, 4096));
     k_face_gather<<<fg, 256, 0, s>>>(lin.f, t->side, B.nx, B.ny, B.nz, px, py, pz);
   }
-  k_adj_b<true><<<grd, blk, 0, s>>>(a);
+  launch_pass_b<true>(a, s);
   k_zero_stepped<<<g, 256, 0, s>>>(lout, B.flags, N);
   return cudaGetLastError();
 }
@@ -1286,11 +1454,11 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
       t->grad[b] = static_cast<float*>(dom->dev_alloc(N * 3 * sizeof(float)));
       if (!t->grad[b]) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
     }
-    t->mu = static_cast<float*>(dom->dev_alloc(nmax * 19 * sizeof(float)));   // mu, sw, sg
+    t->ms = static_cast<float*>(dom->dev_alloc(nmax * sizeof(float)));
     size_t side = 0;
     for (const Block& B : dom->blocks) side = std::max(side, face_side_floats(B.nx, B.ny, B.nz));
     t->side = static_cast<float*>(dom->dev_alloc(side * sizeof(float)));
-    if (!t->mu || !t->side) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
+    if (!t->ms || !t->side) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
     cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
     if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");
   }
@@ -1402,8 +1570,8 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
     if (!t->gam[i]) t->gam[i] = static_cast<float*>(dom->dev_alloc(N * sizeof(float)));
     if (!t->lam[i] || !t->ups[i] || !t->gam[i]) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
   }
-  if (!t->mu) t->mu = static_cast<float*>(dom->dev_alloc(N * 19 * sizeof(float)));   // mu, sw, sg
-  if (!t->mu) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
+  if (!t->ms) t->ms = static_cast<float*>(dom->dev_alloc(N * sizeof(float)));
+  if (!t->ms) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
   if (!t->side) {
     const size_t side = face_side_floats(B.nx, B.ny, B.nz);
     t->side = static_cast<float*>(dom->dev_alloc(side * sizeof(float)));
@@ -1438,8 +1606,6 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
   const bool open_faces = !dom->desc.periodic[0] || !dom->desc.periodic[1] || !dom->desc.periodic[2];
   const int per3[3] = {dom->desc.periodic[0], dom->desc.periodic[1], dom->desc.periodic[2]};
   const int zgrid = (int)std::max<size_t>(1, std::min<size_t>((open_face_threads(B.nx, B.ny, B.nz, per3) + 255) / 256, 4096));
-  const dim3 blk(128, 1, 1);
-  const dim3 grd((B.nx + 127) / 128, B.ny, B.nz);
   for (int sg = n_seg - 1; sg >= 0; --sg) {
     const int s0 = sg * t->every;
     const int len = std::min(t->every, n_steps - s0);
@@ -1459,21 +1625,19 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
       a.lam_out = t->lam[c ^ 1];
       a.ups_out = t->ups[c ^ 1];
       a.gam_out = t->gam[c ^ 1];
-      a.mu = t->mu;
-      a.sw = t->mu + 9 * N;
-      a.sg = t->mu + 18 * N;
+      a.ms = t->ms;
       a.side = t->side;
       if (t->pass_a_minb == 0) {
-        // time both register bounds on this step's inputs (pass A only writes lam_out, mu and
+        // time both register bounds on this step's inputs (pass A only writes lam_out, ms and
         // the inflow nodes' ups_out, which the launches below rewrite), keep the faster
         cudaEvent_t e0, e1, e2;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
         cudaEventCreate(&e2);
         cudaEventRecord(e0, s);
-        for (int r = 0; r < 2; ++r) launch_pass_a(a, 3, open_faces, grd, blk, s);
+        for (int r = 0; r < 2; ++r) launch_pass_a(a, 3, open_faces, s);
         cudaEventRecord(e1, s);
-        for (int r = 0; r < 2; ++r) launch_pass_a(a, 4, open_faces, grd, blk, s);
+        for (int r = 0; r < 2; ++r) launch_pass_a(a, 4, open_faces, s);
         cudaEventRecord(e2, s);
         e = cudaEventSynchronize(e2);
         float m3 = 0.f, m4 = 0.f;
@@ -1489,11 +1653,11 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
       if (open_faces)
         k_zero_face_slots<<<zgrid, 256, 0, s>>>(a.lam_out, B.nx, B.ny, B.nz, dom->desc.periodic[0],
                                                 dom->desc.periodic[1], dom->desc.periodic[2]);
-      launch_pass_a(a, t->pass_a_minb, open_faces, grd, blk, s);
+      launch_pass_a(a, t->pass_a_minb, open_faces, s);
       if (open_faces)
         k_face_gather<<<zgrid, 256, 0, s>>>(a.lam_out, t->side, B.nx, B.ny, B.nz, dom->desc.periodic[0],
                                             dom->desc.periodic[1], dom->desc.periodic[2]);
-      k_adj_b<false><<<grd, blk, 0, s>>>(a);
+      launch_pass_b<false>(a, s);
       e = cudaGetLastError();
       if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint step");
       c ^= 1;
