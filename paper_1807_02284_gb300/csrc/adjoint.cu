@@ -260,49 +260,33 @@ __device__ __forceinline__ void collide_vjp(const float (&K)[27], float (&A)[27]
 
 // The nodes of a block's open faces, each once: thread t walks the open faces in the order
 // x-, x+, y-, y+, z-, z+ and skips a node that an earlier open face already holds.
-__device__ __forceinline__ bool open_face_node(size_t t, int nx, int ny, int nz, const int (&per)[3],
+__device__ __forceinline__ bool open_face_node(uint32_t t, const int (&nn)[3], const int (&per)[3],
                                                int (&p)[3]) {
-  const int nn[3] = {nx, ny, nz};
 #pragma unroll
   for (int f = 0; f < 6; ++f) {
     const int a = f >> 1;
     if (per[a]) continue;
     const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
-    const size_t area = (size_t)nn[b] * nn[c];
+    const uint32_t area = (uint32_t)nn[b] * (uint32_t)nn[c];
     if (t >= area) {
       t -= area;
       continue;
     }
     p[a] = (f & 1) ? nn[a] - 1 : 0;
-    p[b] = (int)(t % nn[b]);
-    p[c] = (int)(t / nn[b]);
-    for (int a2 = 0; a2 < a; ++a2)
-      if (!per[a2] && (p[a2] == 0 || p[a2] == nn[a2] - 1)) return false;
+    const uint32_t q = t / (uint32_t)nn[b];
+    p[b] = (int)(t - q * (uint32_t)nn[b]);
+    p[c] = (int)q;
+#pragma unroll
+    for (int a2 = 0; a2 < 3; ++a2)
+      if (a2 < a && !per[a2] && (p[a2] == 0 || p[a2] == nn[a2] - 1)) return false;
     return true;
   }
   return false;
 }
 
-__host__ __device__ __forceinline__ size_t open_face_threads(int nx, int ny, int nz, const int (&per)[3]) {
-  return (per[0] ? 0 : 2 * (size_t)ny * nz) + (per[1] ? 0 : 2 * (size_t)nx * nz) +
-         (per[2] ? 0 : 2 * (size_t)nx * ny);
-}
-
-// Zeroes the adjoint slots of the nodes on open faces before pass A: a face slot that no pull
-// reads unclamped only receives the clamped pulls' sum, which k_face_gather adds.
-__global__ void k_zero_face_slots(float* __restrict__ lam, int nx, int ny, int nz, int px,
-                                  int py, int pz) {
-  const size_t N = (size_t)nx * ny * nz;
-  const int per[3] = {px, py, pz};
-  const size_t T = open_face_threads(nx, ny, nz, per);
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < T;
-       t += (size_t)gridDim.x * blockDim.x) {
-    int p[3];
-    if (!open_face_node(t, nx, ny, nz, per, p)) continue;
-    const size_t idx = ((size_t)p[2] * ny + p[1]) * nx + p[0];
-#pragma unroll
-    for (int k = 0; k < 27; ++k) lam[(size_t)k * N + idx] = 0.0f;
-  }
+__host__ __device__ __forceinline__ uint32_t open_face_threads(int nx, int ny, int nz, const int (&per)[3]) {
+  return (per[0] ? 0u : 2u * (uint32_t)ny * (uint32_t)nz) + (per[1] ? 0u : 2u * (uint32_t)nx * (uint32_t)nz) +
+         (per[2] ? 0u : 2u * (uint32_t)nx * (uint32_t)ny);
 }
 
 // After pass A: every open-face slot (k, s) adds the adjoints of the clamped pulls that read
@@ -311,45 +295,63 @@ __global__ void k_zero_face_slots(float* __restrict__ lam, int nx, int ny, int n
 // a, either x_a = s_a + e_k,a (unclamped) or x_a = s_a where s_a is the face that the pull
 // leaves (e_k,a = +1 at s_a = 0, -1 at s_a = n_a - 1); the combinations with at least one
 // clamped axis are taken in the order of their axis bits.
-__global__ void k_face_gather(float* __restrict__ lam, float* __restrict__ side, int nx, int ny,
-                              int nz, int px, int py, int pz) {
-  const size_t N = (size_t)nx * ny * nz;
+// zero (may be null): the buffer pass A read, whose face slots are cleared for the next step,
+// where it is pass A's output and a slot that no pull reads unclamped only receives this sum.
+// One thread per face node and direction (grid.y): a loop over the 27 directions in one thread
+// was a chain of 27 dependent rounds of loads (72 x 60 x 51: 51 us, and 5 us more for clearing
+// the slots in a launch of its own).
+__global__ void __launch_bounds__(256) k_face_gather(float* __restrict__ lam, float* __restrict__ side,
+                                                     float* __restrict__ zero, int nx, int ny,
+                                                     int nz, int px, int py, int pz) {
   const int per[3] = {px, py, pz}, nn[3] = {nx, ny, nz};
-  const size_t T = open_face_threads(nx, ny, nz, per);
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < T;
-       t += (size_t)gridDim.x * blockDim.x) {
-    int s[3];
-    if (!open_face_node(t, nx, ny, nz, per, s)) continue;
-    const size_t idx = ((size_t)s[2] * ny + s[1]) * nx + s[0];
-    for (int k = 0; k < 27; ++k) {
-      const int e[3] = {k % 3 - 1, (k / 3) % 3 - 1, k / 9 - 1};
-      float sum = 0.0f;
-      bool any = false;
-      for (int combo = 1; combo < 8; ++combo) {
-        int xr[3];
-        bool ok = true;
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t >= open_face_threads(nx, ny, nz, per)) return;
+  int s[3];
+  if (!open_face_node(t, nn, per, s)) return;
+  const int k = blockIdx.y;
+  const int e[3] = {k % 3 - 1, (k / 3) % 3 - 1, k / 9 - 1};
+  const size_t slot = (size_t)k * ((size_t)nx * ny * nz) + ((size_t)s[2] * ny + s[1]) * nx + s[0];
+  if (zero) zero[slot] = 0.0f;
+  int can = 0;                              // axes on which a reader's pull can be clamped
+  bool in[3];                               // whether s + e lies in the block on that axis
+  int q[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          if (combo & (1 << a)) {   // clamped on axis a
-            ok = ok && !per[a] && ((e[a] == 1 && s[a] == 0) || (e[a] == -1 && s[a] == nn[a] - 1));
-            xr[a] = s[a];
-          } else {
-            int q = s[a] + e[a];
-            if (per[a]) q = q < 0 ? q + nn[a] : (q >= nn[a] ? q - nn[a] : q);
-            ok = ok && q >= 0 && q < nn[a];
-            xr[a] = q;
-          }
-        }
-        if (!ok) continue;
-        const int a0 = (combo & 1) ? 0 : ((combo & 2) ? 1 : 2);
-        const uint32_t si = face_side_index(nx, ny, nz, a0, e[a0] == -1 ? 1 : 0, xr, e);
-        sum += side[si];
-        side[si] = 0.0f;
-        any = true;
-      }
-      if (any) lam[(size_t)k * N + idx] += sum;
-    }
+  for (int a = 0; a < 3; ++a) {
+    if (!per[a] && ((e[a] == 1 && s[a] == 0) || (e[a] == -1 && s[a] == nn[a] - 1))) can |= 1 << a;
+    q[a] = s[a] + e[a];
+    if (per[a]) q[a] = q[a] < 0 ? q[a] + nn[a] : (q[a] >= nn[a] ? q[a] - nn[a] : q[a]);
+    in[a] = q[a] >= 0 && q[a] < nn[a];
   }
+  if (!can) return;
+  float sum = 0.0f;
+  bool any = false;
+#pragma unroll
+  for (int combo = 1; combo < 8; ++combo) {
+    if ((combo & can) != combo) continue;
+    int xr[3];
+    bool ok = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const bool clamped = (combo >> a) & 1;
+      xr[a] = clamped ? s[a] : q[a];
+      ok = ok && (clamped || in[a]);
+    }
+    if (!ok) continue;
+    const int a0 = (combo & 1) ? 0 : ((combo & 2) ? 1 : 2);
+    const uint32_t si = face_side_index(nx, ny, nz, a0, e[a0] == -1 ? 1 : 0, xr, e);
+    sum += side[si];
+    side[si] = 0.0f;
+    any = true;
+  }
+  if (any) lam[slot] += sum;
+}
+
+static void launch_face_gather(float* lam, float* side, float* zero, const BlockView& v,
+                               cudaStream_t s) {
+  const int per[3] = {v.per[0], v.per[1], v.per[2]};
+  const unsigned g = (open_face_threads(v.nx, v.ny, v.nz, per) + 255) / 256;
+  if (g == 0) return;
+  k_face_gather<<<dim3(g, 27, 1), 256, 0, s>>>(lam, side, zero, v.nx, v.ny, v.nz, per[0], per[1], per[2]);
 }
 
 // The populations of a wall node (face wall or obstacle surface) pulled from beyond the wall:
@@ -1400,12 +1402,7 @@ static cudaError_t ms_reverse_op(lbm_domain* dom, TapeState* t, const MsOp& o, c
   a.side = t->side;
   const bool open = o.b != 0 || !dom->desc.periodic[0] || !dom->desc.periodic[1] || !dom->desc.periodic[2];
   launch_pass_a(a, 3, open, s, true);
-  if (open) {
-    const int px = a.fwd.per[0], py = a.fwd.per[1], pz = a.fwd.per[2];
-    const int per3[3] = {px, py, pz};
-    const int fg = (int)std::max<size_t>(1, std::min<size_t>((open_face_threads(B.nx, B.ny, B.nz, per3) + 255) / 256, 4096));
-    k_face_gather<<<fg, 256, 0, s>>>(lin.f, t->side, B.nx, B.ny, B.nz, px, py, pz);
-  }
+  if (open) launch_face_gather(lin.f, t->side, nullptr, a.fwd, s);
   launch_pass_b<true>(a, s);
   k_zero_stepped<<<g, 256, 0, s>>>(lout, B.flags, N);
   return cudaGetLastError();
@@ -1604,8 +1601,6 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
 
   const int n_seg = (n_steps + t->every - 1) / t->every;
   const bool open_faces = !dom->desc.periodic[0] || !dom->desc.periodic[1] || !dom->desc.periodic[2];
-  const int per3[3] = {dom->desc.periodic[0], dom->desc.periodic[1], dom->desc.periodic[2]};
-  const int zgrid = (int)std::max<size_t>(1, std::min<size_t>((open_face_threads(B.nx, B.ny, B.nz, per3) + 255) / 256, 4096));
   for (int sg = n_seg - 1; sg >= 0; --sg) {
     const int s0 = sg * t->every;
     const int len = std::min(t->every, n_steps - s0);
@@ -1650,13 +1645,8 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
         t->pass_a_minb = m4 < m3 ? 4 : 3;
       }
       // (the tuning launches store the same values pass A stores below, side entries included)
-      if (open_faces)
-        k_zero_face_slots<<<zgrid, 256, 0, s>>>(a.lam_out, B.nx, B.ny, B.nz, dom->desc.periodic[0],
-                                                dom->desc.periodic[1], dom->desc.periodic[2]);
       launch_pass_a(a, t->pass_a_minb, open_faces, s);
-      if (open_faces)
-        k_face_gather<<<zgrid, 256, 0, s>>>(a.lam_out, t->side, B.nx, B.ny, B.nz, dom->desc.periodic[0],
-                                            dom->desc.periodic[1], dom->desc.periodic[2]);
+      if (open_faces) launch_face_gather(a.lam_out, t->side, t->lam[c], a.fwd, s);
       launch_pass_b<false>(a, s);
       e = cudaGetLastError();
       if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint step");
