@@ -457,8 +457,9 @@ constexpr int ADJ_THREADS = 128;
 // 56 % of DRAM peak; before, the flags, the pull, the corners and the adjoints waited for one
 // another in turn and 19 words per node went to pass B), 72 x 60 x 51 with open faces
 // 64 -> 34 us (rows of 72 nodes left 44 % of a 128-thread row's lanes idle).
-template <int MINB, bool OPEN, bool ACC, bool WALLS>
-__global__ void __launch_bounds__(ADJ_THREADS, MINB) k_adj_a(AdjArgs a) {
+// 4 CTAs per SM (128 registers, no spills) against 3: 169 against 192 us at 128^3.
+template <bool OPEN, bool ACC, bool WALLS>
+__global__ void __launch_bounds__(ADJ_THREADS, 4) k_adj_a(AdjArgs a) {
   __shared__ float sadj[31][ADJ_THREADS];     // lam, ups, gam of the node
   __shared__ float scor[8][ADJ_THREADS];      // scalar corners of its departure cell
   const BlockView& v = a.fwd;
@@ -836,23 +837,20 @@ static dim3 pass_a_grid(const BlockView& v) {
 }
 
 template <bool WALLS>
-static void launch_pass_a_t(const AdjArgs& a, int minb, bool open, cudaStream_t s, bool acc) {
+static void launch_pass_a_t(const AdjArgs& a, bool open, bool acc, cudaStream_t s) {
   const dim3 grd = pass_a_grid(a.fwd), blk(ADJ_THREADS, 1, 1);
-  if (acc) {   // multi-block reverse: 3 CTAs/SM, open faces (every refined block has them)
-    if (open) k_adj_a<3, true, true, WALLS><<<grd, blk, 0, s>>>(a);
-    else k_adj_a<3, false, true, WALLS><<<grd, blk, 0, s>>>(a);
-  } else if (open) {
-    if (minb == 4) k_adj_a<4, true, false, WALLS><<<grd, blk, 0, s>>>(a);
-    else k_adj_a<3, true, false, WALLS><<<grd, blk, 0, s>>>(a);
+  if (acc) {   // multi-block reverse
+    if (open) k_adj_a<true, true, WALLS><<<grd, blk, 0, s>>>(a);
+    else k_adj_a<false, true, WALLS><<<grd, blk, 0, s>>>(a);
   } else {
-    if (minb == 4) k_adj_a<4, false, false, WALLS><<<grd, blk, 0, s>>>(a);
-    else k_adj_a<3, false, false, WALLS><<<grd, blk, 0, s>>>(a);
+    if (open) k_adj_a<true, false, WALLS><<<grd, blk, 0, s>>>(a);
+    else k_adj_a<false, false, WALLS><<<grd, blk, 0, s>>>(a);
   }
 }
 
-static void launch_pass_a(const AdjArgs& a, int minb, bool open, cudaStream_t s, bool acc = false) {
-  if (a.fwd.walls) launch_pass_a_t<true>(a, minb, open, s, acc);
-  else launch_pass_a_t<false>(a, minb, open, s, acc);
+static void launch_pass_a(const AdjArgs& a, bool open, bool acc, cudaStream_t s) {
+  if (a.fwd.walls) launch_pass_a_t<true>(a, open, acc, s);
+  else launch_pass_a_t<false>(a, open, acc, s);
 }
 
 template <bool ACC>
@@ -1066,7 +1064,6 @@ __global__ void k_inflow_grad(const float* __restrict__ du0, const uint8_t* __re
 
 struct TapeState {
   int every = 0;
-  int pass_a_minb = 0;        // chosen launch bound of pass A (0: not yet timed)
   std::vector<Level> ckpt;    // states at steps 0, every, 2 every, ...
   std::vector<Level> seg;     // recompute levels 1..every of one segment
   float* lam[2] = {nullptr, nullptr};
@@ -1401,7 +1398,7 @@ static cudaError_t ms_reverse_op(lbm_domain* dom, TapeState* t, const MsOp& o, c
   a.ms = t->ms;
   a.side = t->side;
   const bool open = o.b != 0 || !dom->desc.periodic[0] || !dom->desc.periodic[1] || !dom->desc.periodic[2];
-  launch_pass_a(a, 3, open, s, true);
+  launch_pass_a(a, open, true, s);
   if (open) launch_face_gather(lin.f, t->side, nullptr, a.fwd, s);
   launch_pass_b<true>(a, s);
   k_zero_stepped<<<g, 256, 0, s>>>(lout, B.flags, N);
@@ -1576,7 +1573,8 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
     cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
     if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");
   }
-  const int seg_len = std::min(t->every, std::max(1, n_steps));
+  const bool fp32 = dom->desc.storage == LBM_FP32;
+  const int seg_len = std::min(t->every, std::max(1, n_steps)) - (fp32 ? 1 : 0);
   while ((int)t->seg.size() < seg_len) {
     Level L;
     if (!alloc_level(dom, N, L)) {
@@ -1604,9 +1602,14 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
   for (int sg = n_seg - 1; sg >= 0; --sg) {
     const int s0 = sg * t->every;
     const int len = std::min(t->every, n_steps - s0);
-    // recompute the segment's states 1..len from its checkpoint
+    // recompute the segment's states 1..n_replay from its checkpoint.  The last step's result
+    // is wanted for its velocity alone, which the forward kept: it is the next checkpoint's, or
+    // the domain's current one (bit for bit what the replay computes with FP32 storage; an FP16
+    // run's replay follows unrounded states, so its own result is taken there)
     auto level = [&](int i) -> const Level& { return i == 0 ? t->ckpt[sg] : t->seg[i - 1]; };
-    for (int i = 0; i < len; ++i) {
+    const int n_replay = fp32 ? len - 1 : len;
+    const float* u_end = !fp32 ? nullptr : sg == n_seg - 1 ? B.lv[B.cur].u : t->ckpt[sg + 1].u;
+    for (int i = 0; i < n_replay; ++i) {
       e = launch_step(view_of(dom, level(i), level(i + 1)), ST_FP32, B.bx, B.by, s, B.minb);
       if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint recompute");
     }
@@ -1616,36 +1619,13 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
       a.lam_in = t->lam[c];
       a.ups_in = t->ups[c];
       a.gam_in = t->gam[c];
-      a.u_next = level(i + 1).u;
+      a.u_next = i + 1 <= n_replay ? level(i + 1).u : u_end;
       a.lam_out = t->lam[c ^ 1];
       a.ups_out = t->ups[c ^ 1];
       a.gam_out = t->gam[c ^ 1];
       a.ms = t->ms;
       a.side = t->side;
-      if (t->pass_a_minb == 0) {
-        // time both register bounds on this step's inputs (pass A only writes lam_out, ms and
-        // the inflow nodes' ups_out, which the launches below rewrite), keep the faster
-        cudaEvent_t e0, e1, e2;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        cudaEventCreate(&e2);
-        cudaEventRecord(e0, s);
-        for (int r = 0; r < 2; ++r) launch_pass_a(a, 3, open_faces, s);
-        cudaEventRecord(e1, s);
-        for (int r = 0; r < 2; ++r) launch_pass_a(a, 4, open_faces, s);
-        cudaEventRecord(e2, s);
-        e = cudaEventSynchronize(e2);
-        float m3 = 0.f, m4 = 0.f;
-        if (e == cudaSuccess) cudaEventElapsedTime(&m3, e0, e1);
-        if (e == cudaSuccess) cudaEventElapsedTime(&m4, e1, e2);
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        cudaEventDestroy(e2);
-        if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint tuning");
-        t->pass_a_minb = m4 < m3 ? 4 : 3;
-      }
-      // (the tuning launches store the same values pass A stores below, side entries included)
-      launch_pass_a(a, t->pass_a_minb, open_faces, s);
+      launch_pass_a(a, open_faces, false, s);
       if (open_faces) launch_face_gather(a.lam_out, t->side, t->lam[c], a.fwd, s);
       launch_pass_b<false>(a, s);
       e = cudaGetLastError();
