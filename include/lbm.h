@@ -144,9 +144,10 @@ typedef struct {
   int32_t substeps;  /* sub-steps per reference step (1 for s0) */
   int64_t steps;     /* reference steps taken by the domain */
   int32_t tile[2];   /* x, y extent in nodes of one CTA of the collide-stream kernel (chosen
-                        by autotuning) */
+                        from the block's extents and storage); tile[1] = 1: tile[0] nodes of
+                        a plane in x-fastest order, running on over the ends of rows */
   int32_t ctas_per_sm; /* CTAs per SM the collide-stream kernel's registers are bounded for
-                          (chosen by autotuning together with the tile) */
+                          (chosen together with the tile) */
   int32_t parent;      /* a refined block's prior-mapping source (the finest coarser block
                           containing it); -1 for the reference block and far-field blocks */
   int32_t nodes_per_thread; /* 1: one node per thread (tile[0] x tile[1] threads per CTA,

@@ -1108,10 +1108,6 @@ extern "C" lbm_status lbm_step_phase(lbm_domain* dom, int32_t phase, int32_t blo
       for (int b = 1; b < nb; ++b)
         if (dom->blocks[b].far)
           return dom->fail(LBM_ERR_UNSUPPORTED, "phased steps cover refined blocks, not far-field blocks");
-      for (int b = 0; b < nb; ++b) {
-        lbm_status st = dom->autotune_tiles(b);
-        if (st != LBM_OK) return st;
-      }
       dom->phase_saved.assign(nb, 0);
       for (int b = 0; b < nb; ++b) dom->phase_saved[b] = dom->blocks[b].cur;
       dom->phase_done.assign(nb, 0);

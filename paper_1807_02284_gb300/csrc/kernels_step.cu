@@ -5,24 +5,23 @@
 namespace lbm {
 
 // MINB: CTAs of 256 threads per SM the registers are bounded for (3: 80 registers, no
-// spills; 4: 64 registers with a small spill, more loads in flight); chosen by autotuning.
-template <typename T, typename IT, bool ALIGN, int MINB, bool WALLS>
+// spills; 4: 64 registers with a small spill, more loads in flight); pick_tiles chooses.
+template <typename T, typename IT, bool ALIGN, int MINB, bool WALLS, bool LINEAR>
 __global__ void __launch_bounds__(256, MINB) k_step(BlockView v) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int x, y;
+  if (!thread_column<LINEAR>(v.nx, v.ny, x, y)) return;
   const int z = blockIdx.z + v.z_first;
-  if (x >= v.nx || y >= v.ny) return;
   cell_update<T, IT, ALIGN, WALLS>(v, x, y, z);
 }
 
 // Two nodes (x, x + 1) per thread, x = 2 (thread's column): MINB CTAs of at most 128 threads
 // per SM (128 registers per thread at 4; 96 at 5 and 80 at 6, with small spills).
-template <typename T, typename IT, int MINB, bool WALLS>
+template <typename T, typename IT, int MINB, bool WALLS, bool LINEAR>
 __global__ void __launch_bounds__(128, MINB) k_step2(BlockView v) {
-  const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int x, y;
+  if (!thread_column<LINEAR>(v.nx / 2, v.ny, x, y)) return;
+  x *= 2;
   const int z = blockIdx.z + v.z_first;
-  if (x >= v.nx || y >= v.ny) return;
   if constexpr (pair_corners_async<T>()) {
     __shared__ float corners[16][128];     // each thread's scalar corners, column t
     const int t = threadIdx.y * blockDim.x + threadIdx.x;
@@ -34,17 +33,20 @@ __global__ void __launch_bounds__(128, MINB) k_step2(BlockView v) {
 
 bool fits_32bit_index(size_t N) { return 27ull * (unsigned long long)N < 0xFFFFFFFFull; }
 
-template <typename T, typename IT, int MINB>
+template <typename T, typename IT, int MINB, bool LINEAR>
 static void launch_step2_b(const BlockView& v, dim3 grid, dim3 block, cudaStream_t s) {
-  if (v.walls) k_step2<T, IT, MINB, true><<<grid, block, 0, s>>>(v);
-  else k_step2<T, IT, MINB, false><<<grid, block, 0, s>>>(v);
+  if (v.walls) k_step2<T, IT, MINB, true, LINEAR><<<grid, block, 0, s>>>(v);
+  else k_step2<T, IT, MINB, false, LINEAR><<<grid, block, 0, s>>>(v);
 }
 
+// linear one-row CTAs run at the bound pick_tiles takes for the storage
 template <typename T, typename IT>
 static void launch_step2_t(const BlockView& v, dim3 grid, dim3 block, int b, cudaStream_t s) {
-  if (b >= 6) launch_step2_b<T, IT, 6>(v, grid, block, s);
-  else if (b == 5) launch_step2_b<T, IT, 5>(v, grid, block, s);
-  else launch_step2_b<T, IT, 4>(v, grid, block, s);
+  if (tile_linear(v.nx / 2, (int)block.x, (int)block.y))
+    launch_step2_b<T, IT, sizeof(T) == 2 ? 5 : 4, true>(v, grid, block, s);
+  else if (b >= 6) launch_step2_b<T, IT, 6, false>(v, grid, block, s);
+  else if (b == 5) launch_step2_b<T, IT, 5, false>(v, grid, block, s);
+  else launch_step2_b<T, IT, 4, false>(v, grid, block, s);
 }
 
 static bool aligned_to(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
@@ -63,7 +65,7 @@ static void launch_step2(const BlockView& v, int storage, int bx, int by, int b,
                          cudaStream_t s) {
   const int tx = bx / 2;
   dim3 block(tx, by, 1);
-  dim3 grid((v.nx / 2 + tx - 1) / tx, (v.ny + by - 1) / by, planes);
+  const dim3 grid = tile_grid(v.nx / 2, v.ny, planes, tx, by);
   const bool i32 = fits_32bit_index(v.N);
   if (storage == ST_FP16) {
     if (i32) launch_step2_t<__half, uint32_t>(v, grid, block, b, s);
@@ -74,16 +76,17 @@ static void launch_step2(const BlockView& v, int storage, int bx, int by, int b,
   }
 }
 
+template <typename T, typename IT, bool ALIGN, int MINB, bool LINEAR>
+static void launch_step_b(const BlockView& v, dim3 grid, dim3 block, cudaStream_t s) {
+  if (v.walls) k_step<T, IT, ALIGN, MINB, true, LINEAR><<<grid, block, 0, s>>>(v);
+  else k_step<T, IT, ALIGN, MINB, false, LINEAR><<<grid, block, 0, s>>>(v);
+}
+
 template <typename T, typename IT, bool ALIGN>
 static void launch_step_t(const BlockView& v, dim3 grid, dim3 block, int minb, cudaStream_t s) {
-  minb = step_scalar_bound(minb);
-  if (v.walls) {
-    if (minb >= 4) k_step<T, IT, ALIGN, 4, true><<<grid, block, 0, s>>>(v);
-    else k_step<T, IT, ALIGN, 3, true><<<grid, block, 0, s>>>(v);
-  } else {
-    if (minb >= 4) k_step<T, IT, ALIGN, 4, false><<<grid, block, 0, s>>>(v);
-    else k_step<T, IT, ALIGN, 3, false><<<grid, block, 0, s>>>(v);
-  }
+  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_b<T, IT, ALIGN, 4, true>(v, grid, block, s);
+  else if (step_scalar_bound(minb) >= 4) launch_step_b<T, IT, ALIGN, 4, false>(v, grid, block, s);
+  else launch_step_b<T, IT, ALIGN, 3, false>(v, grid, block, s);
 }
 
 cudaError_t launch_step(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
@@ -93,7 +96,7 @@ cudaError_t launch_step(const BlockView& v, int storage, int bx, int by, cudaStr
     return cudaGetLastError();
   }
   dim3 block(bx, by, 1);
-  dim3 grid((v.nx + bx - 1) / bx, (v.ny + by - 1) / by, v.nz);
+  const dim3 grid = tile_grid(v.nx, v.ny, (unsigned)v.nz, bx, by);
   const bool i32 = fits_32bit_index(v.N);
   if (storage == ST_FP16) {
     if (i32) launch_step_t<__half, uint32_t, false>(v, grid, block, minb, s);
@@ -116,7 +119,7 @@ cudaError_t launch_step_planes(const BlockView& v, int storage, int bx, int by, 
     return cudaGetLastError();
   }
   dim3 block(bx, by, 1);
-  dim3 grid((v.nx + bx - 1) / bx, (v.ny + by - 1) / by, count);
+  const dim3 grid = tile_grid(v.nx, v.ny, (unsigned)count, bx, by);
   const bool i32 = fits_32bit_index(v.N);
   if (storage == ST_FP16) {
     if (i32) launch_step_t<__half, uint32_t, false>(w, grid, block, minb, s);
@@ -132,7 +135,7 @@ cudaError_t launch_step_planes(const BlockView& v, int storage, int bx, int by, 
 // 32-bit indexing: refined blocks are limited to 27 N < 2^32).
 cudaError_t launch_step_align(const BlockView& v, int bx, int by, cudaStream_t s, int minb) {
   dim3 block(bx, by, 1);
-  dim3 grid((v.nx + bx - 1) / bx, (v.ny + by - 1) / by, v.nz);
+  const dim3 grid = tile_grid(v.nx, v.ny, (unsigned)v.nz, bx, by);
   launch_step_t<float, uint32_t, true>(v, grid, block, minb, s);
   return cudaGetLastError();
 }

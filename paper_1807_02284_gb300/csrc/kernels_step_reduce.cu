@@ -36,13 +36,13 @@ __device__ __forceinline__ void finish_cta_record(float (*swarp)[6], unsigned& d
 // partials[cta * 8 + value].  All of it in FP32 (FP64's issue rate on this part
 // is a small fraction of FP32's); the records are summed in FP64 afterwards, in a fixed
 // order.  Same populations, velocity and scalar as k_step.
-template <typename T, int MINB, bool WALLS>
+template <typename T, int MINB, bool WALLS, bool LINEAR>
 __global__ void __launch_bounds__(256, MINB) k_step_reduce(BlockView v, double* partials) {
   __shared__ float snm[8][6][32];
   __shared__ float swarp[8][6];
   __shared__ unsigned done;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int x, y;
+  const bool in = thread_column<LINEAR>(v.nx, v.ny, x, y);
   const int z = blockIdx.z;
   const int t = threadIdx.y * blockDim.x + threadIdx.x;
   const int lane = t & 31, w = t >> 5;
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(256, MINB) k_step_reduce(BlockView v, double* 
   if (t == 0) done = 0u;
   __syncthreads();                          // the counter is set before any warp counts
   const NodeMomentsOut out{&col[0][lane], 32};
-  if (x < v.nx && y < v.ny) cell_update<T, uint32_t, false, WALLS, true>(v, x, y, z, &out);
+  if (in) cell_update<T, uint32_t, false, WALLS, true>(v, x, y, z, &out);
   __syncwarp();
   float val[6];
 #pragma unroll
@@ -75,13 +75,14 @@ __global__ void __launch_bounds__(256, MINB) k_step_reduce(BlockView v, double* 
 // tree after a warp barrier only; the last warp to finish (a shared-memory counter) adds
 // the eight group sums in order.  The CTA records, and the diagnostics, are bit-identical
 // to k_step_reduce's on the same node tile, and no warp waits for the others' collision.
-template <typename T, int MINB, bool WALLS>
+template <typename T, int MINB, bool WALLS, bool LINEAR>
 __global__ void __launch_bounds__(128, MINB) k_step2_reduce(BlockView v, double* partials) {
   __shared__ float snm[8][6][32];
   __shared__ float swarp[8][6];
   __shared__ unsigned done;
-  const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int x, y;
+  const bool in = thread_column<LINEAR>(v.nx / 2, v.ny, x, y);
+  x *= 2;
   const int z = blockIdx.z;
   const int t = threadIdx.y * blockDim.x + threadIdx.x;
   const int lane = t & 31, w = t >> 5;
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(128, MINB) k_step2_reduce(BlockView v, double*
   __syncthreads();                          // the counter is set before any warp counts
   const NodeMomentsOut out0{&snm[t0 >> 5][0][t0 & 31], 32};
   const NodeMomentsOut out1{&snm[t1 >> 5][0][t1 & 31], 32};
-  if (x < v.nx && y < v.ny) {
+  if (in) {
     if constexpr (pair_corners_async<T>()) {
       __shared__ float corners[16][128];
       cell_update_pair<T, uint32_t, WALLS, true>(v, x, y, z, &corners[0][t], 128, &out0, &out1);
@@ -124,36 +125,42 @@ __global__ void __launch_bounds__(128, MINB) k_step2_reduce(BlockView v, double*
 
 // records written by one k_step_reduce launch (one per CTA)
 size_t step_reduce_ctas(const BlockView& v, int bx, int by) {
-  return (size_t)((v.nx + bx - 1) / bx) * ((v.ny + by - 1) / by) * v.nz;
+  const dim3 g = tile_grid(v.nx, v.ny, (unsigned)v.nz, bx, by);
+  return (size_t)g.x * g.y * g.z;
 }
 
-// The register bound the step's autotuner chose for the block (the diagnostics add no live
+// The register bound chosen for the block's step (the diagnostics add no live
 // values through the collision: both bounds compile without spills).
+template <typename T, int MINB, bool LINEAR>
+static void launch_step_reduce_b(const BlockView& v, dim3 grid, dim3 block, double* partials,
+                                 cudaStream_t s) {
+  if (v.walls) k_step_reduce<T, MINB, true, LINEAR><<<grid, block, 0, s>>>(v, partials);
+  else k_step_reduce<T, MINB, false, LINEAR><<<grid, block, 0, s>>>(v, partials);
+}
+
 template <typename T>
 static void launch_step_reduce_t(const BlockView& v, dim3 grid, dim3 block, int minb,
                                  double* partials, cudaStream_t s) {
-  if (step_scalar_bound(minb) >= 4) {
-    if (v.walls) k_step_reduce<T, 4, true><<<grid, block, 0, s>>>(v, partials);
-    else k_step_reduce<T, 4, false><<<grid, block, 0, s>>>(v, partials);
-  } else {
-    if (v.walls) k_step_reduce<T, 3, true><<<grid, block, 0, s>>>(v, partials);
-    else k_step_reduce<T, 3, false><<<grid, block, 0, s>>>(v, partials);
-  }
+  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_reduce_b<T, 4, true>(v, grid, block, partials, s);
+  else if (step_scalar_bound(minb) >= 4) launch_step_reduce_b<T, 4, false>(v, grid, block, partials, s);
+  else launch_step_reduce_b<T, 3, false>(v, grid, block, partials, s);
 }
 
-template <typename T, int MINB>
+template <typename T, int MINB, bool LINEAR>
 static void launch_step2_reduce_b(const BlockView& v, dim3 grid, dim3 block, double* partials,
                                   cudaStream_t s) {
-  if (v.walls) k_step2_reduce<T, MINB, true><<<grid, block, 0, s>>>(v, partials);
-  else k_step2_reduce<T, MINB, false><<<grid, block, 0, s>>>(v, partials);
+  if (v.walls) k_step2_reduce<T, MINB, true, LINEAR><<<grid, block, 0, s>>>(v, partials);
+  else k_step2_reduce<T, MINB, false, LINEAR><<<grid, block, 0, s>>>(v, partials);
 }
 
 template <typename T>
 static void launch_step2_reduce_t(const BlockView& v, dim3 grid, dim3 block, int b,
                                   double* partials, cudaStream_t s) {
-  if (b >= 6) launch_step2_reduce_b<T, 6>(v, grid, block, partials, s);
-  else if (b == 5) launch_step2_reduce_b<T, 5>(v, grid, block, partials, s);
-  else launch_step2_reduce_b<T, 4>(v, grid, block, partials, s);
+  if (tile_linear(v.nx / 2, (int)block.x, (int)block.y))
+    launch_step2_reduce_b<T, sizeof(T) == 2 ? 5 : 4, true>(v, grid, block, partials, s);
+  else if (b >= 6) launch_step2_reduce_b<T, 6, false>(v, grid, block, partials, s);
+  else if (b == 5) launch_step2_reduce_b<T, 5, false>(v, grid, block, partials, s);
+  else launch_step2_reduce_b<T, 4, false>(v, grid, block, partials, s);
 }
 
 // 32-bit indexing only (27 N < 2^32): the caller checks fits_32bit_index.  A two-node bound
@@ -164,7 +171,7 @@ cudaError_t launch_step_reduce(const BlockView& v, int storage, int bx, int by, 
   if (step_is_pair(minb) && step_pair_ok(v, storage, bx, by) && bx * by <= 256 &&
       ((bx / 2) * by) % 32 == 0) {
     dim3 block(bx / 2, by, 1);
-    dim3 grid((v.nx + bx - 1) / bx, (v.ny + by - 1) / by, v.nz);
+    const dim3 grid = tile_grid(v.nx / 2, v.ny, (unsigned)v.nz, bx / 2, by);
     if (storage == ST_FP16) launch_step2_reduce_t<__half>(v, grid, block, minb - STEP_PAIR, partials, s);
     else launch_step2_reduce_t<float>(v, grid, block, minb - STEP_PAIR, partials, s);
     const cudaError_t e = cudaGetLastError();
@@ -172,7 +179,7 @@ cudaError_t launch_step_reduce(const BlockView& v, int storage, int bx, int by, 
     return launch_reduce_columns(partials, step_reduce_ctas(v, bx, by), out, s, out5);
   }
   dim3 block(bx, by, 1);
-  dim3 grid((v.nx + bx - 1) / bx, (v.ny + by - 1) / by, v.nz);
+  const dim3 grid = tile_grid(v.nx, v.ny, (unsigned)v.nz, bx, by);
   if (storage == ST_FP16) launch_step_reduce_t<__half>(v, grid, block, minb, partials, s);
   else launch_step_reduce_t<float>(v, grid, block, minb, partials, s);
   const cudaError_t e = cudaGetLastError();

@@ -8,6 +8,25 @@
 
 namespace lbm {
 
+// The (x, y) column of a thread of a collide-stream launch over nx x ny columns: CTAs tile the
+// plane, or (LINEAR, one-row CTAs) take consecutive columns of the plane in x-fastest order,
+// running on into the next rows, so that no lane idles when nx is not a multiple of the CTA.
+// False for threads past the end.  A separate instance: the column of a linear thread comes
+// out of a division and is held (a few spills, 2 % on whole rows), a tile's is recomputed from
+// the thread index.
+template <bool LINEAR>
+__device__ __forceinline__ bool thread_column(int nx, int ny, int& x, int& y) {
+  if constexpr (LINEAR) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    y = (int)(i / (uint32_t)nx);
+    x = (int)(i - (uint32_t)y * (uint32_t)nx);
+    return y < ny;
+  }
+  x = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  y = (int)(blockIdx.y * blockDim.y + threadIdx.y);
+  return x < nx && y < ny;
+}
+
 template <typename IT>
 struct Nbr {
   IT xm, x0, xp;            // x - 1, x, x + 1 (wrapped or clamped)

@@ -88,7 +88,7 @@ struct WorkItem {
 };
 
 // ---- kernels_step.cu
-// Register-bound code of the collide-stream launch (chosen by autotuning with the tile
+// Register-bound code of the collide-stream launch (chosen by pick_tiles with the tile
 // bx x by of nodes): 3 or 4 = CTAs of bx by one-node threads per SM; STEP_PAIR + b = the
 // two-node kernel k_step2 (bx / 2 x by threads per CTA, b = 4, 5 or 6 CTAs per SM), which
 // needs an even nx and falls back to the one-node kernel (bound 4) otherwise.  Kernels
@@ -96,6 +96,13 @@ struct WorkItem {
 constexpr int STEP_PAIR = 16;
 inline bool step_is_pair(int minb) { return minb >= STEP_PAIR; }
 inline int step_scalar_bound(int minb) { return minb >= STEP_PAIR ? 4 : minb; }
+// Whether CTAs of tx x ty threads over rows of nx columns take the linear mapping of
+// thread_column (one-row CTAs that do not divide the row), and the grid over `planes` planes.
+inline bool tile_linear(int nx, int tx, int ty) { return ty == 1 && nx % tx != 0; }
+inline dim3 tile_grid(int nx, int ny, unsigned planes, int tx, int ty) {
+  if (tile_linear(nx, tx, ty)) return dim3((unsigned)(((size_t)nx * ny + tx - 1) / tx), 1, planes);
+  return dim3((unsigned)((nx + tx - 1) / tx), (unsigned)((ny + ty - 1) / ty), planes);
+}
 // Whether the two-node kernels can run this view with the node tile bx x by (even nx,
 // pair-aligned arrays, at most 128 threads).
 bool step_pair_ok(const BlockView& v, int storage, int bx, int by);

@@ -48,7 +48,6 @@ struct Block {
   RelaxParams rp;
   int bx = 128, by = 2;    // tile of the collide-stream launch
   int minb = 3;            // register bound of the collide-stream launch (CTAs per SM)
-  bool tuned = false;      // tile shape chosen by autotune_tiles
   // far-field block (h > 1, Sec. 4.2.4-4.2.5): it surrounds block `child` (s0 or the previous
   // far block), takes its nodes inside the child's interior from the child (far_in) and
   // gives the child its outer layer (far_out)
@@ -93,11 +92,6 @@ struct lbm_domain {
   long long steps = 0;
   lbm::TapeState* tape = nullptr;
   lbm::GraphCache* graphs = nullptr;
-  // launch shapes already timed, by block size class (x extent: < 64, < 128, < 256, more;
-  // nodes: < 2^20, < 2^23, more): a block of the same class (a rebuilt dynamic scale)
-  // reuses the choice
-  struct TunedShape { int nx_class, n_class, bx, by, minb; };
-  std::vector<TunedShape> tuned_shapes;
   void* batch_plan = nullptr;           // cached plans of lbm_step_batch (batch.cu)
   // scratch of lbm_reduce_batch when this domain heads the list (device and pinned host)
   void* rb_dev = nullptr;
@@ -144,7 +138,6 @@ struct lbm_domain {
   lbm_status error_status();
   lbm_status reset_error_word();
   void pick_tiles(int b);
-  lbm_status autotune_tiles(int b);
   void invalidate_graphs();
   void release_extras();
   void on_state_reset(int b);

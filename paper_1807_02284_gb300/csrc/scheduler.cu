@@ -37,13 +37,39 @@ static std::vector<int> next_levels(const std::vector<lbm::Block>& blocks, std::
 }
 }  // namespace lbm
 
+// Launch shape of a block's collide-stream kernel, from its extents and storage.  Figures: us per
+// step of fluid blocks on GB300, every shape and register bound tried at each size.
 void lbm_domain::pick_tiles(int b) {
   Block& B = blocks[b];
-  // x-contiguous tiles of 256 threads; narrow blocks use a 32-wide tile with more rows
-  B.bx = B.nx >= 128 ? 128 : B.nx >= 64 ? 64 : 32;
-  B.by = 256 / B.bx;
-  B.tuned = false;
-  B.minb = 3;
+  const bool half = desc.storage == LBM_FP16_SHIFTED;
+  if (B.nx % 2 == 0 && B.N >= (half ? (size_t)3 << 18 : (size_t)3 << 19)) {
+    // two nodes per thread once the block is bound by bandwidth or issue rather than by
+    // latency: FP32 from 1.6 M nodes (96^3 44 against 42 us with one node per thread, 196 x 98 x 98
+    // 84 against 85, 128^3 88 against 92, 256^3 658 against 702), FP16 from 0.8 M (80^3 24
+    // against 23, 96^3 40 against 41, 128^3 80 against 95, 256^3 591 against 718).  Tiles of
+    // 64 x 2 nodes on whole rows (FP16 with 128-node rows 128 x 2), one-row CTAs running on over ragged ones (224 x 250 x 190 FP32
+    // 427 us against 454 with 64 x 2 tiles).
+    const bool tiles = B.nx % 64 == 0;
+    B.bx = half && (!tiles || B.nx % 128 == 0) ? 128 : 64;
+    B.by = tiles ? 2 : 1;
+    B.minb = STEP_PAIR + (half ? 5 : 4);
+  } else if (B.nx <= 32) {
+    // latency-bound: a warp per row keeps the rows' faces in warps of their own (24^3 3.0 us
+    // against 3.8 with one-row CTAs, where most warps hold a face node and an inner one)
+    B.bx = 32;
+    B.by = 4;
+    B.minb = 3;
+  } else if (B.nx % 32 == 0) {
+    B.bx = 32;                           // 64^3 12.1 us, 96^3 42.2 (one-row CTAs: 12.2, 43.2)
+    B.by = 4;
+    B.minb = 4;
+  } else {
+    // ragged rows: no idle lanes (72 x 60 x 51 11.2 us against 13.5 with the best tile,
+    // 97 x 61 x 75 21.7 against 25.8, 196 x 98 x 98 85 against 92)
+    B.bx = 128;
+    B.by = 1;
+    B.minb = 4;
+  }
   if (const char* env = std::getenv("LBM_TILE")) {  // "bx,by[,minb]" forces a launch shape
     int bx = 0, by = 0, mb = 3;
     const int n = std::sscanf(env, "%d,%d,%d", &bx, &by, &mb);
@@ -52,63 +78,8 @@ void lbm_domain::pick_tiles(int b) {
       B.bx = bx;
       B.by = by;
       B.minb = mb;
-      B.tuned = true;
     }
   }
-}
-
-// Times candidate launch shapes of the collide-stream kernel (tile shape x register bound) on
-// the block's current state and keeps the fastest.  Candidates read the current level and write the next one without
-// advancing the clock, so tuning changes no result (every shape computes the same values).
-lbm_status lbm_domain::autotune_tiles(int b) {
-  Block& B = blocks[b];
-  if (B.tuned) return LBM_OK;
-  B.tuned = true;
-  if (B.N < (size_t)1 << 18 || B.lv.size() < 2) return LBM_OK;
-  const int nx_class = B.nx >= 256 ? 3 : B.nx >= 128 ? 2 : B.nx >= 64 ? 1 : 0;
-  const int n_class = B.N < ((size_t)1 << 20) ? 0 : B.N < ((size_t)1 << 23) ? 1 : 2;
-  for (const TunedShape& t : tuned_shapes)
-    if (t.nx_class == nx_class && t.n_class == n_class) {
-      B.bx = t.bx;
-      B.by = t.by;
-      B.minb = t.minb;
-      return LBM_OK;
-    }
-  const int cand[][2] = {{32, 8}, {64, 4}, {128, 2}, {256, 1}, {32, 4}, {64, 2}, {128, 1}};
-  // bound codes: one-node kernel at 3 or 4 CTAs of the tile per SM, then (even nx) the
-  // two-node kernel at 4, 5 or 6 CTAs of half the threads, on tiles of at least 64 x-nodes
-  const int bounds[] = {3, 4, STEP_PAIR + 4, STEP_PAIR + 5, STEP_PAIR + 6};
-  cudaEvent_t e0, e1;
-  if (cudaEventCreate(&e0) != cudaSuccess) return cuda_fail(cudaGetLastError(), "event");
-  if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return cuda_fail(cudaGetLastError(), "event"); }
-  const int to = (B.cur + 1) % (int)B.lv.size();
-  float best = 1e30f;
-  int bx = B.bx, by = B.by, minb = B.minb;
-  for (const int mb : bounds)
-  for (const auto& c : cand) {
-    if (c[0] > 32 && c[0] > B.nx + 31) continue;
-    if (step_is_pair(mb) && (B.nx % 2 != 0 || c[0] < 64 || c[0] > B.nx + 63)) continue;
-    const BlockView v = view(b, B.cur, to);
-    cudaError_t e = launch_step(v, desc.storage, c[0], c[1], stream, mb);  // warm-up
-    if (e == cudaSuccess) e = cudaEventRecord(e0, stream);
-    for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = launch_step(v, desc.storage, c[0], c[1], stream, mb);
-    if (e == cudaSuccess) e = cudaEventRecord(e1, stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-    float ms = 0.f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    if (e != cudaSuccess) {
-      cudaEventDestroy(e0); cudaEventDestroy(e1);
-      return cuda_fail(e, "tile autotuning");
-    }
-    if (ms < best) { best = ms; bx = c[0]; by = c[1]; minb = mb; }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  B.bx = bx;
-  B.by = by;
-  B.minb = minb;
-  tuned_shapes.push_back({nx_class, n_class, bx, by, minb});
-  return LBM_OK;
 }
 
 void lbm_domain::invalidate_graphs() {
@@ -292,14 +263,6 @@ lbm_status lbm_domain::advance_single(int m) {
 }
 
 lbm_status lbm_domain::advance(int n) {
-  if (n > 0) {
-    for (size_t b = 0; b < blocks.size(); ++b) {
-      const bool was = blocks[b].tuned;
-      lbm_status st = autotune_tiles((int)b);
-      if (st != LBM_OK) return st;
-      if (!was) invalidate_graphs();
-    }
-  }
   if (blocks.size() > 1) {  // stream and events of the fork/join schedule exist before capture
     cudaStream_t a = nullptr;
     lbm_status st = aux(&a);
@@ -381,7 +344,6 @@ static lbm_status enqueue_step_reduce(lbm_domain* dom, int32_t n, double* out5) 
     return e == cudaSuccess ? LBM_OK : dom->cuda_fail(e, "reduce");
   }
   lbm_status st = dom->advance(n - 1);
-  if (st == LBM_OK) st = dom->autotune_tiles(0);
   if (st == LBM_OK) st = tape_before_step(dom);
   if (st != LBM_OK) return st;
   const int nxt = B.cur ^ 1;

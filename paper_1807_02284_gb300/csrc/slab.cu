@@ -127,11 +127,9 @@ extern "C" lbm_status lbm_step_slab(lbm_domain* dom, int32_t lo, int32_t hi, voi
   if ((lo && bad(send_lo)) || (hi && bad(send_hi)))
     return dom->fail(LBM_ERR_INVALID_ARG, "send buffer null or not 16-byte aligned");
   if (*dom->h_err & 1) return dom->fail(LBM_ERR_DIVERGED, "divergence recorded by an earlier step");
-  lbm_status st = dom->autotune_tiles(0);
-  if (st != LBM_OK) return st;
   cudaStream_t ps = static_cast<cudaStream_t>(pack_stream);
   if (!ps) {
-    st = dom->aux(&ps);
+    const lbm_status st = dom->aux(&ps);
     if (st != LBM_OK) return st;
   }
   cudaEvent_t ev = dom->event(7);

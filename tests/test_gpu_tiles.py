@@ -1,0 +1,42 @@
+"""Launch shapes of the collide-stream step: CTAs of one row walk a plane's nodes in x-fastest
+order and run on over the ends of rows; every shape computes the same values."""
+import numpy as np
+import pytest
+
+import synth
+from tests.helpers import gpu_domain
+
+pytestmark = pytest.mark.gpu
+
+
+def _state(monkeypatch, tile, sc, storage, walls):
+    from paper_1807_02284_gb300 import lbm
+    if tile:
+        monkeypatch.setenv("LBM_TILE", tile)
+    else:
+        monkeypatch.delenv("LBM_TILE", raising=False)
+    d = gpu_domain(sc, storage)
+    if walls:
+        d.set_walls((0, 0, 1, 1, 0, 0), obstacles=True)
+    d.step(3)
+    diag = d.step_reduce(1)
+    out = [d.read_field(f, lbm.LBM_F32) for f in (lbm.LBM_FIELD_F, lbm.LBM_FIELD_U, lbm.LBM_FIELD_SCALAR)]
+    d.close()
+    return out, diag
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (2, 3, 2), (31, 5, 3), (33, 4, 3), (34, 7, 5), (65, 9, 4),
+                                  (96, 3, 2), (130, 6, 3)])
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+@pytest.mark.parametrize("walls", [False, True])
+def test_one_row_ctas_equal_tiles(lib, monkeypatch, dims, storage, walls):
+    """The chosen shape and one-row CTAs of both kernels against 32 x 8 tiles: equal bits; the
+    diagnostics to FP32 rounding of their partial sums (2^-24 times the 256 terms of a CTA)."""
+    spheres = [(dims[0] / 2, dims[1] / 2, dims[2] / 2, 1.2)] if min(dims) > 2 else ()
+    sc = synth.random_scene(dims=dims, seed=31, periodic=(False, False, True), nu=0.01, spheres=spheres)
+    ref, dref = _state(monkeypatch, "32,8,3", sc, storage, walls)
+    for tile in ("", "32,1,3", "64,1,4", "128,1,4", "256,1,3", "64,1,20", "128,1,21", "256,1,22"):
+        got, d = _state(monkeypatch, tile, sc, storage, walls)
+        for a, b in zip(ref, got):
+            assert np.array_equal(a, b), tile
+        assert np.abs(d - dref).max() <= 256 * 2.0 ** -24 * np.abs(dref).max()
