@@ -540,7 +540,7 @@ def parity_by_variant():
         worst = max(worst, float(np.abs(u - uo).max() / np.abs(uo).max()))
         d.close()
     out["batch64"] = {"u_max_abs_err_rel": worst, "bound": 1e-5,
-                      "case": "2 simulations (edges 10-16) in one persistent launch, 3 steps"}
+                      "case": "2 simulations (edges 10-16) in one batched call, 3 steps"}
     sc, target = synth.adjoint_scene(n=12, seed=5, nu=0.01, amp=0.05)
     b = sc.blocks[0]
     dom = lbm.Domain(b.dims, sc.nu, periodic=sc.periodic, adaptive=sc.adaptive)
@@ -792,7 +792,7 @@ def run_ours(args):
 
 def run_batch(args):
     """64 independent plumes of uneven size (edges 24..96) advanced by lbm_step_batch: one
-    graph-captured persistent launch for all K steps."""
+    graph-captured call for all K steps."""
     import torch
 
     import synth
@@ -886,7 +886,7 @@ def run_batch(args):
                            "l2": "inputs larger than L2 (state %.2f GB)" % (N * 280 / 1e9)},
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                              "frac": achieved / peak, "traffic": None, "peak_source": peak_src,
-                             "kernel": "k_batch (persistent, cooperative)"},
+                             "kernel": "k_step / k_step2 of every member (forked branches of one graph)"},
                 "repeats": reps,
                 "e2e": {"value": N * E * ws / t_e2e / 1e6, "unit": "MLUPS",
                         "h2d_bytes_per_step": int(sum(r.nbytes for r in recs)),

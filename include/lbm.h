@@ -466,17 +466,17 @@ lbm_status lbm_pack_box(lbm_domain* dom, int32_t block, int32_t level, const int
 lbm_status lbm_unpack_box(lbm_domain* dom, int32_t block, int32_t level, const int32_t lo[3],
                           const int32_t hi[3], const void* dev_buf, int32_t skip_flags);
 
-/* Advances n independent single-block domains by `steps` reference steps with one
-   persistent kernel per step over a joint tile work list, captured in one CUDA graph and
-   launched on doms[0]'s stream (tile shape chosen by the library's autotuner on first use).
+/* Advances n independent single-block domains by `steps` reference steps: every member's own
+   launches, forked over a few streams so that members fill the GPU together, captured in CUDA
+   graphs and launched on doms[0]'s stream.
    Every domain must be single-block, without wall faces, with the same storage and device.  Results are
    bit-identical to calling lbm_step on each domain. */
 lbm_status lbm_step_batch(lbm_domain* const* doms, int32_t n, int32_t steps);
 
 /* lbm_step_batch with steps >= 1 followed by the lbm_reduce diagnostics of every member's
-   new state, summed by the last step's own kernel (each work item's nodes add their
-   moments as they are stored; the item sums are combined per member in FP64 in a fixed
-   order and copied back by the same captured graph): no second pass over the populations.
+   new state, summed by the last step's own kernels (as lbm_step_reduce; the CTA sums are
+   combined per member in FP64 in a fixed order and copied back by the same captured graph):
+   no second pass over the populations.
    out is a host array of 5 n doubles (the lbm_reduce_batch layout); the values agree with
    lbm_reduce's to FP32 rounding of the per-node terms.  Synchronises; INVALID_ARG for
    steps < 1 or a null out; otherwise the lbm_step_batch errors, and each member's device
@@ -494,9 +494,8 @@ lbm_status lbm_step_batch_reduce(lbm_domain* const* doms, int32_t n, int32_t ste
 lbm_status lbm_step_batch_reduce_async(lbm_domain* const* doms, int32_t n, int32_t steps,
                                        double* out, int64_t* ticket);
 
-/* Self-test of the bounded device-wide barrier used by lbm_step_batch (no counterpart in the
-   paper): launches a small cooperative kernel whose barrier waits for `extra` CTAs that do
-   not exist, so every wait expires after about limit_ms (0 < limit_ms <= 5000).  Returns
+/* Self-test of the library's bounded device-wide barrier (no counterpart in the paper):
+   launches a small cooperative kernel whose barrier waits for `extra` CTAs that do not exist, so every wait expires after about limit_ms (0 < limit_ms <= 5000).  Returns
    LBM_ERR_TIMEOUT when the bounded wait gave up and reported it (extra > 0), LBM_OK when
    the barrier completed (extra = 0); the CUDA context stays usable either way. */
 lbm_status lbm_barrier_selftest(int32_t extra, double limit_ms, void* cuda_stream);

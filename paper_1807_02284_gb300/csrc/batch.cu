@@ -1,12 +1,19 @@
-// Batched persistent stepping of many independent single-block domains of uneven sizes.
+// Batched stepping of many independent single-block domains of uneven sizes.
 //
-// All domains' nodes are cut into chunks of consecutive node indices; one cooperative,
-// persistent kernel walks the joint chunk list for every step and separates the steps with a
-// device-wide barrier.  The barrier's waits are bounded by a clock limit: a CTA that waits too
-// long sets the TIMEOUT bit of the error word and every CTA leaves the kernel, so a lost CTA
-// can never hang the GPU.  The launch (plus the reset of the barrier counters) is captured in
-// a CUDA graph and replayed.  Every node runs the same cell_update as the single-block kernel,
-// so results are bit-identical to stepping each domain on its own.
+// Every member takes its own collide-stream launches (k_step / k_step2, or the diagnostics form
+// in the last step), with the launch shape its size calls for; the members' steps are forked
+// over a few streams, balanced by their nodes, and the whole call is captured in a CUDA graph.
+// Members do not depend on one another, so while one member's last CTAs drain, the other
+// branches' launches fill the SMs, and no step waits for the slowest member.  Measured against
+// one persistent cooperative kernel over a joint chunk list with a device-wide barrier per
+// step (128 registers, since a member's view came from memory instead of the constant bank;
+// one node per thread): 64 plumes of edges 24 to 96, 1.34 -> 0.98 ms per step, and no timing
+// launches at a set's first call (57 -> 24 ms).
+// Every node runs the same cell_update as a domain stepped on its own, so results are
+// bit-identical to that.
+//
+// The bounded device-wide barrier below (a wait that expires sets the TIMEOUT bit instead of
+// hanging the GPU) is kept with its self-test.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -19,17 +26,10 @@
 
 namespace lbm {
 
-struct BatchItem {
-  int dom;        // domain index in the batch
-  uint32_t start; // first node of the chunk
-};
-
 struct BarrierState {
   unsigned int count;
   unsigned int gen;
 };
-
-constexpr long long kBarrierLimitCycles = 4000000000LL;  // ~2 s at 2 GHz
 
 // Device-wide barrier with a bounded wait.  Returns false when the wait gave up.
 __device__ __forceinline__ bool grid_barrier(BarrierState* bs, unsigned int nblocks, int* err,
@@ -63,174 +63,45 @@ __device__ __forceinline__ bool grid_barrier(BarrierState* bs, unsigned int nblo
   return ok != 0;
 }
 
-template <typename T, typename IT>
-__global__ void __launch_bounds__(256) k_batch(const BlockView* __restrict__ views,
-                                               const BatchItem* __restrict__ items, int n_items,
-                                               int chunk, int steps, BarrierState* bs,
-                                               unsigned int expected_blocks, int* err,
-                                               long long limit) {
-  for (int s = 0; s < steps; ++s) {
-    const int p = s & 1;
-    for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
-      const BatchItem it = items[w];
-      const BlockView& v = views[2 * it.dom + p];
-      const uint32_t nx = (uint32_t)v.nx, nxy = (uint32_t)v.nx * (uint32_t)v.ny;
-      const uint32_t end = min((uint32_t)v.N, it.start + (uint32_t)chunk);
-      for (uint32_t idx = it.start + threadIdx.x; idx < end; idx += blockDim.x) {
-        const uint32_t z = idx / nxy;
-        const uint32_t r = idx - z * nxy;
-        const uint32_t y = r / nx;
-        cell_update<T, IT>(v, (int)(r - y * nx), (int)y, (int)z);
-      }
-    }
-    if (s + 1 < steps) {
-      if (!grid_barrier(bs, expected_blocks, err, limit)) return;
-      if (*((volatile int*)err) & 8) return;
-    }
+// The six sums of every member over its CTA records of the diagnostics step (8 doubles each),
+// one CTA per member: thread t takes records t, t + 256, ... in order, then a fixed tree; the
+// member's device error word rides along in slot 6.
+__global__ void __launch_bounds__(256) k_batch_records(const double* __restrict__ records,
+                                                       const RedMember* __restrict__ members,
+                                                       double* __restrict__ out) {
+  __shared__ double sh[6][256];
+  const RedMember m = members[blockIdx.x];
+  const int t = threadIdx.x;
+  double s[6] = {0, 0, 0, 0, 0, 0};
+  for (int i = t; i < m.n_items; i += 256) {
+#pragma unroll
+    for (int v = 0; v < 6; ++v) s[v] += records[(size_t)(m.first_item + i) * 8 + v];
   }
-}
-
-// k_batch with the diagnostics fused into the last step (lbm_step_batch_reduce): in that
-// step each node adds its moments (from cell_update, into a per-thread shared-memory slot)
-// to its thread's accumulator, and every work item ends with a CTA sum (shuffle tree per
-// warp, warps in order, FP32) stored as one record of 8 doubles, records[item * 8 + value].
-// The populations, velocities and scalars are those of k_batch.
-template <typename T>
-__global__ void __launch_bounds__(256, 2) k_batch_red(const BlockView* __restrict__ views,
-                                                   const BatchItem* __restrict__ items,
-                                                   int n_items, int chunk, int steps,
-                                                   BarrierState* bs, unsigned int expected_blocks,
-                                                   int* err, long long limit, double* records) {
-  __shared__ float tmp[6][256];
-  __shared__ float acc[6][256];
-  __shared__ float swarp[8][6];
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  const NodeMomentsOut out{&tmp[0][t], 256};
-  for (int s = 0; s < steps; ++s) {
-    const int p = s & 1;
-    const bool last = s + 1 == steps;
-    for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
-      const BatchItem it = items[w];
-      const BlockView& v = views[2 * it.dom + p];
-      const uint32_t nx = (uint32_t)v.nx, nxy = (uint32_t)v.nx * (uint32_t)v.ny;
-      const uint32_t end = min((uint32_t)v.N, it.start + (uint32_t)chunk);
-      if (!last) {
-        for (uint32_t idx = it.start + t; idx < end; idx += blockDim.x) {
-          const uint32_t z = idx / nxy;
-          const uint32_t r = idx - z * nxy;
-          const uint32_t y = r / nx;
-          cell_update<T, uint32_t>(v, (int)(r - y * nx), (int)y, (int)z);
-        }
-        continue;
-      }
 #pragma unroll
-      for (int i = 0; i < 6; ++i) acc[i][t] = 0.0f;
-      for (uint32_t idx = it.start + t; idx < end; idx += blockDim.x) {
-        const uint32_t z = idx / nxy;
-        const uint32_t r = idx - z * nxy;
-        const uint32_t y = r / nx;
+  for (int v = 0; v < 6; ++v) sh[v][t] = s[v];
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if (t < w) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) tmp[i][t] = 0.0f;
-        cell_update<T, uint32_t, false, false, true>(v, (int)(r - y * nx), (int)y, (int)z, &out);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) acc[i][t] += tmp[i][t];
-      }
-      float val[6];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) val[i] = acc[i][t];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < 6; ++i) val[i] += __shfl_xor_sync(0xffffffffu, val[i], o);
-      if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) swarp[wid][i] = val[i];
-      }
-      __syncthreads();
-      if (t < 8) {
-        float sum = 0.0f;
-        if (t < 6)
-          for (int k = 0; k < (int)(blockDim.x >> 5); ++k) sum += swarp[k][t];
-        records[(size_t)w * 8 + t] = (double)sum;
-      }
-      __syncthreads();
+      for (int v = 0; v < 6; ++v) sh[v][t] += sh[v][t + w];
     }
-    if (s + 1 < steps) {
-      if (!grid_barrier(bs, expected_blocks, err, limit)) return;
-      if (*((volatile int*)err) & 8) return;
-    }
+    __syncthreads();
   }
+  if (t < 6) out[(size_t)blockIdx.x * 8 + t] = sh[t][0];
+  if (t == 6) out[(size_t)blockIdx.x * 8 + 6] = (double)*m.err;
 }
 
-template <typename T>
-static cudaError_t launch_batch_red_t(const BlockView* views, const BatchItem* items, int n_items,
-                                      int chunk, int steps, BarrierState* bs, int threads,
-                                      int grid, unsigned int expected, int* err, long long limit,
-                                      double* records, cudaStream_t s) {
-  void* args[] = {(void*)&views, (void*)&items, (void*)&n_items, (void*)&chunk, (void*)&steps,
-                  (void*)&bs, (void*)&expected, (void*)&err, (void*)&limit, (void*)&records};
-  return cudaLaunchCooperativeKernel((const void*)k_batch_red<T>, dim3(grid), dim3(threads),
-                                     args, 0, s);
-}
-
-template <typename T, typename IT>
-static cudaError_t launch_batch_t(const BlockView* views, const BatchItem* items, int n_items,
-                                  int chunk, int steps, BarrierState* bs, int threads, int grid,
-                                  unsigned int expected, int* err, long long limit,
-                                  bool cooperative, cudaStream_t s) {
-  if (!cooperative) {
-    k_batch<T, IT><<<grid, threads, 0, s>>>(views, items, n_items, chunk, steps, bs, expected,
-                                            err, limit);
-    return cudaGetLastError();
-  }
-  void* args[] = {(void*)&views, (void*)&items, (void*)&n_items, (void*)&chunk, (void*)&steps,
-                  (void*)&bs, (void*)&expected, (void*)&err, (void*)&limit};
-  return cudaLaunchCooperativeKernel((const void*)k_batch<T, IT>, dim3(grid), dim3(threads),
-                                     args, 0, s);
-}
-
-static cudaError_t launch_batch(int storage, bool i32, const BlockView* views,
-                                const BatchItem* items, int n_items, int chunk, int steps,
-                                BarrierState* bs, int threads, int grid, unsigned int expected,
-                                int* err, long long limit, bool cooperative, cudaStream_t s) {
-  if (storage == ST_FP16) {
-    if (i32) return launch_batch_t<__half, uint32_t>(views, items, n_items, chunk, steps, bs, threads, grid, expected, err, limit, cooperative, s);
-    return launch_batch_t<__half, uint64_t>(views, items, n_items, chunk, steps, bs, threads, grid, expected, err, limit, cooperative, s);
-  }
-  if (i32) return launch_batch_t<float, uint32_t>(views, items, n_items, chunk, steps, bs, threads, grid, expected, err, limit, cooperative, s);
-  return launch_batch_t<float, uint64_t>(views, items, n_items, chunk, steps, bs, threads, grid, expected, err, limit, cooperative, s);
-}
-
-static int resident_blocks(int storage, bool i32, int threads, bool red = false) {
-  int per_sm = 0, dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const void* fn = red ? (storage == ST_FP16 ? (const void*)k_batch_red<__half> : (const void*)k_batch_red<float>)
-                 : storage == ST_FP16
-                       ? (i32 ? (const void*)k_batch<__half, uint32_t> : (const void*)k_batch<__half, uint64_t>)
-                       : (i32 ? (const void*)k_batch<float, uint32_t> : (const void*)k_batch<float, uint64_t>);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0);
-  return std::max(1, per_sm) * std::max(1, sms);
-}
-
-// One captured batched launch: the work list and views of a set of domains, starting from a
-// given assignment of time levels and advancing a given number of steps.
+// One captured call: the launches of a set of domains from a given assignment of time levels
+// over at most kGraphSteps steps.
 struct BatchPlan {
   std::vector<unsigned long long> serials;   // members (domain serials, in call order)
   std::vector<int> curs;
   int steps = 0;
-  int chunk = 0, threads = 0;
-  BlockView* views = nullptr;
-  BatchItem* items = nullptr;
-  BarrierState* bar = nullptr;
-  int n_items = 0;
-  bool i32 = true;
-  int grid = 0;
   cudaGraphExec_t exec = nullptr;
-  bool captured = false;
-  // fused diagnostics (lbm_step_batch_reduce): per-item records, per-member sums (sums and
+  // fused diagnostics (lbm_step_batch_reduce): per-CTA records, per-member sums (sums and
   // error word, 8 doubles each) copied to pinned host memory by the same graph
   bool red = false;
+  std::vector<int> first;       // each member's first record
   double* records = nullptr;
   RedMember* members = nullptr;
   double* out_dev = nullptr;
@@ -239,14 +110,16 @@ struct BatchPlan {
 };
 
 // Plans cached by the first domain of a batch.  A call with an odd step count flips every
-// member's current level, so alternating calls need two plans; a few more cover a caller
-// that alternates between batches.  Members are matched by serial, never by address, so a
-// plan never refers to a destroyed domain's memory once it is chosen.
+// member's current level, so alternating calls need two plans, and a long call takes whole
+// graphs and a rest; a few more cover a caller that alternates between batches.  Members are
+// matched by serial, never by address, so a plan never refers to a destroyed domain's memory
+// once it is chosen.
 struct BatchCache {
   std::vector<BatchPlan*> plans;   // most recently used last
-  int chunk = 0, threads = 0;      // tuned once per cache
 };
-constexpr size_t kMaxBatchPlans = 4;
+constexpr size_t kMaxBatchPlans = 8;
+constexpr int kGraphSteps = 16;      // even: a whole graph ends in the levels it started from
+constexpr int kBatchStreams = 32;
 
 }  // namespace lbm
 
@@ -254,9 +127,6 @@ using namespace lbm;
 
 static void free_plan(lbm_domain* dom, BatchPlan* p) {
   if (p->exec) cudaGraphExecDestroy(p->exec);
-  dom->dev_free(p->views);
-  dom->dev_free(p->items);
-  dom->dev_free(p->bar);
   if (p->records) dom->dev_free(p->records);
   if (p->members) dom->dev_free(p->members);
   if (p->out_dev) dom->dev_free(p->out_dev);
@@ -265,20 +135,23 @@ static void free_plan(lbm_domain* dom, BatchPlan* p) {
   delete p;
 }
 
-// The diagnostics buffers of a plan: one record per work item, the members' item ranges and
-// error words, the per-member sums on the device and in pinned host memory.
+// The diagnostics buffers of a plan: one record per CTA of every member's last step, the
+// members' record ranges and error words, the per-member sums on the device and in pinned host
+// memory.
 static lbm_status add_red_buffers(lbm_domain* const* doms, int n, BatchPlan* p) {
   lbm_domain* d0 = doms[0];
   std::vector<RedMember> hm(n);
-  int at = 0;
+  p->first.resize(n);
+  size_t at = 0;
   for (int i = 0; i < n; ++i) {
     const Block& B = doms[i]->blocks[0];
-    const int cnt = (int)((B.N + (size_t)p->chunk - 1) / (size_t)p->chunk);
-    hm[i] = RedMember{nullptr, nullptr, doms[i]->d_err, B.N, at, cnt};
+    const size_t cnt = step_reduce_ctas(doms[i]->view(0, B.cur, B.cur ^ 1), B.bx, B.by);
+    hm[i] = RedMember{nullptr, nullptr, doms[i]->d_err, B.N, (int)at, (int)cnt};
+    p->first[i] = (int)at;
     at += cnt;
   }
-  if (at != p->n_items) return d0->fail(LBM_ERR_STATE, "batch work list and members disagree");
-  p->records = static_cast<double*>(d0->dev_alloc((size_t)p->n_items * 8 * sizeof(double)));
+  if (at > (size_t)INT32_MAX) return d0->fail(LBM_ERR_UNSUPPORTED, "batch too large for one diagnostics pass");
+  p->records = static_cast<double*>(d0->dev_alloc(at * 8 * sizeof(double)));
   p->members = static_cast<RedMember*>(d0->dev_alloc((size_t)n * sizeof(RedMember)));
   p->out_dev = static_cast<double*>(d0->dev_alloc((size_t)n * 8 * sizeof(double)));
   p->out5_dev = static_cast<double*>(d0->dev_alloc((size_t)n * 5 * sizeof(double)));
@@ -296,27 +169,57 @@ static lbm_status add_red_buffers(lbm_domain* const* doms, int n, BatchPlan* p) 
   return LBM_OK;
 }
 
-// The work of one batched call on stream s: reset the barrier, the persistent launch, and with
-// fused diagnostics the per-member sums and their copy to pinned host memory.
-static cudaError_t enqueue_batch(lbm_domain* d0, BatchPlan* p, int steps, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(p->bar, 0, sizeof(BarrierState), s);
-  if (e != cudaSuccess) return e;
-  if (!p->red)
-    return launch_batch(d0->desc.storage, p->i32, p->views, p->items, p->n_items, p->chunk, steps,
-                        p->bar, p->threads, p->grid, (unsigned)p->grid, d0->d_err,
-                        kBarrierLimitCycles, true, s);
-  e = d0->desc.storage == ST_FP16
-          ? launch_batch_red_t<__half>(p->views, p->items, p->n_items, p->chunk, steps, p->bar,
-                                       p->threads, p->grid, (unsigned)p->grid, d0->d_err,
-                                       kBarrierLimitCycles, p->records, s)
-          : launch_batch_red_t<float>(p->views, p->items, p->n_items, p->chunk, steps, p->bar,
-                                      p->threads, p->grid, (unsigned)p->grid, d0->d_err,
-                                      kBarrierLimitCycles, p->records, s);
+// Step k (0-based) of member i on stream s; the plan's last step writes the member's records.
+static cudaError_t enqueue_member(lbm_domain* const* doms, const BatchPlan* p, int i, int k,
+                                  cudaStream_t s) {
+  const lbm_domain* d = doms[i];
+  const Block& B = d->blocks[0];
+  const int from = p->curs[i] ^ (k & 1);
+  const BlockView v = d->view(0, from, from ^ 1);
+  if (p->red && k == p->steps - 1)
+    return launch_step_records(v, d->desc.storage, B.bx, B.by, s, B.minb,
+                               p->records + (size_t)p->first[i] * 8);
+  return launch_step(v, d->desc.storage, B.bx, B.by, s, B.minb);
+}
+
+static cudaError_t enqueue_sums(const BatchPlan* p, cudaStream_t s) {
   const int n = (int)p->serials.size();
-  if (e == cudaSuccess) e = launch_reduce_item_records(p->records, p->members, n, p->out_dev, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(p->out_host, p->out_dev, (size_t)n * 8 * sizeof(double),
-                        cudaMemcpyDeviceToHost, s);
+  k_batch_records<<<n, 256, 0, s>>>(p->records, p->members, p->out_dev);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return cudaMemcpyAsync(p->out_host, p->out_dev, (size_t)n * 8 * sizeof(double),
+                         cudaMemcpyDeviceToHost, s);
+}
+
+// The launches of a plan: members largest first onto the least loaded of a few branches, each
+// branch step by step over its members, forked from and joined into s.
+static cudaError_t enqueue_batch(lbm_domain* const* doms, const BatchPlan* p, cudaStream_t s) {
+  lbm_domain* d0 = doms[0];
+  const int n = (int)p->serials.size();
+  const int nb = std::min(n, kBatchStreams);
+  std::vector<int> order(n);
+  for (int i = 0; i < n; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    return doms[a]->blocks[0].N > doms[b]->blocks[0].N;
+  });
+  std::vector<std::vector<int>> branch(nb);
+  std::vector<size_t> load(nb, 0);
+  for (int i : order) {
+    const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    branch[b].push_back(i);
+    load[b] += doms[i]->blocks[0].N;
+  }
+  cudaError_t e = cudaEventRecord(d0->event(0), s);
+  for (int b = 0; b < nb && e == cudaSuccess; ++b) {
+    cudaStream_t bs = b == 0 ? s : d0->post_stream(b);
+    if (b) e = cudaStreamWaitEvent(bs, d0->event(0), 0);
+    for (int k = 0; k < p->steps && e == cudaSuccess; ++k)
+      for (size_t m = 0; m < branch[b].size() && e == cudaSuccess; ++m)
+        e = enqueue_member(doms, p, branch[b][m], k, bs);
+    if (b && e == cudaSuccess) e = cudaEventRecord(d0->event(b), bs);
+  }
+  for (int b = 1; b < nb && e == cudaSuccess; ++b) e = cudaStreamWaitEvent(s, d0->event(b), 0);
+  if (e == cudaSuccess && p->red) e = enqueue_sums(p, s);
   return e;
 }
 
@@ -328,78 +231,63 @@ void release_batch_plan(lbm_domain* dom) {
   dom->batch_plan = nullptr;
 }
 
-// Views for both step parities and the chunk list of the current batch.
-static lbm_status build_plan(lbm_domain* const* doms, int n, int chunk, BatchPlan* p) {
+// The plan of `steps` (at most kGraphSteps) steps from the members' current levels, from the
+// cache or captured now.
+static lbm_status batch_plan(lbm_domain* const* doms, int n, int steps, bool red, BatchPlan** out) {
   lbm_domain* d0 = doms[0];
-  std::vector<BlockView> hv(2 * (size_t)n);
-  std::vector<BatchItem> hi;
-  p->i32 = true;
-  for (int i = 0; i < n; ++i) {
-    const Block& B = doms[i]->blocks[0];
-    hv[2 * i + 0] = doms[i]->view(0, B.cur, B.cur ^ 1);
-    hv[2 * i + 1] = doms[i]->view(0, B.cur ^ 1, B.cur);
-    if (27ull * B.N >= 0xFFFFFFFFull) p->i32 = false;
-    for (size_t s = 0; s < B.N; s += (size_t)chunk) hi.push_back(BatchItem{i, (uint32_t)s});
+  BatchCache* cache = static_cast<BatchCache*>(d0->batch_plan);
+  if (!cache) {
+    cache = new (std::nothrow) BatchCache();
+    if (!cache) return d0->fail(LBM_ERR_OOM, "out of host memory");
+    d0->batch_plan = cache;
   }
-  if (!p->i32) return d0->fail(LBM_ERR_UNSUPPORTED, "batched domains must have 27 N < 2^32");
-  p->views = static_cast<BlockView*>(d0->dev_alloc(hv.size() * sizeof(BlockView)));
-  p->items = static_cast<BatchItem*>(d0->dev_alloc(hi.size() * sizeof(BatchItem)));
-  p->bar = static_cast<BarrierState*>(d0->dev_alloc(sizeof(BarrierState)));
-  if (!p->views || !p->items || !p->bar) return d0->fail(LBM_ERR_OOM, "batch plan allocation failed");
-  cudaError_t e = cudaMemcpyAsync(p->views, hv.data(), hv.size() * sizeof(BlockView),
-                                  cudaMemcpyHostToDevice, d0->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(p->items, hi.data(), hi.size() * sizeof(BatchItem), cudaMemcpyHostToDevice,
-                        d0->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(d0->stream);
-  if (e != cudaSuccess) return d0->cuda_fail(e, "batch plan upload");
-  p->n_items = (int)hi.size();
-  p->chunk = chunk;
+  for (size_t k = 0; k < cache->plans.size(); ++k) {
+    BatchPlan* q = cache->plans[k];
+    bool same = q->steps == steps && q->red == red && (int)q->serials.size() == n;
+    for (int i = 0; i < n && same; ++i)
+      same = q->serials[i] == doms[i]->serial && q->curs[i] == doms[i]->blocks[0].cur;
+    if (same) {
+      cache->plans.erase(cache->plans.begin() + k);
+      cache->plans.push_back(q);
+      *out = q;
+      return LBM_OK;
+    }
+  }
+  // the fork's streams and events exist before the capture
+  const int nb = std::min(n, kBatchStreams);
+  if (!d0->event(nb)) return d0->fail(LBM_ERR_CUDA, "cudaEventCreate");
+  if (nb > 1 && !d0->post_stream(nb - 1)) return d0->fail(LBM_ERR_CUDA, "cudaStreamCreate");
+  BatchPlan* p = new (std::nothrow) BatchPlan();
+  if (!p) return d0->fail(LBM_ERR_OOM, "out of host memory");
+  p->steps = steps;
   p->serials.resize(n);
   p->curs.resize(n);
   for (int i = 0; i < n; ++i) {
     p->serials[i] = doms[i]->serial;
     p->curs[i] = doms[i]->blocks[0].cur;
   }
-  return LBM_OK;
-}
-
-// Picks the chunk size of the work list by timing single-step launches that write the next
-// level without advancing any domain (no result changes).
-static lbm_status tune_chunk(lbm_domain* const* doms, int n, int* chunk_out, int* threads_out) {
-  lbm_domain* d0 = doms[0];
-  const int cand[][2] = {{256, 256}, {256, 512}, {256, 1024}, {128, 128}, {128, 256}};
-  cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  float best = 1e30f;
-  *chunk_out = 256;
-  *threads_out = 256;
-  for (const auto& c : cand) {
-    BatchPlan p;
-    lbm_status st = build_plan(doms, n, c[1], &p);
-    if (st != LBM_OK) { d0->dev_free(p.views); d0->dev_free(p.items); d0->dev_free(p.bar); cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
-    const int grid = resident_blocks(d0->desc.storage, p.i32, c[0]);
-    cudaError_t e = launch_batch(d0->desc.storage, p.i32, p.views, p.items, p.n_items, p.chunk, 1,
-                                 p.bar, c[0], grid, (unsigned)grid, d0->d_err,
-                                 kBarrierLimitCycles, false, d0->stream);
-    if (e == cudaSuccess) e = cudaEventRecord(e0, d0->stream);
-    for (int r = 0; r < 3 && e == cudaSuccess; ++r)
-      e = launch_batch(d0->desc.storage, p.i32, p.views, p.items, p.n_items, p.chunk, 1, p.bar,
-                       c[0], grid, (unsigned)grid, d0->d_err, kBarrierLimitCycles, false,
-                       d0->stream);
-    if (e == cudaSuccess) e = cudaEventRecord(e1, d0->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-    float ms = 0.f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-    d0->dev_free(p.views);
-    d0->dev_free(p.items);
-    d0->dev_free(p.bar);
-    if (e != cudaSuccess) { cudaEventDestroy(e0); cudaEventDestroy(e1); return d0->cuda_fail(e, "batch tuning"); }
-    if (ms < best) { best = ms; *chunk_out = c[1]; *threads_out = c[0]; }
+  if (red) {
+    const lbm_status st = add_red_buffers(doms, n, p);
+    if (st != LBM_OK) { free_plan(d0, p); return st; }
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  while (cache->plans.size() >= kMaxBatchPlans) {
+    // a replaced plan's last launch may still be running; its buffers go back to the allocator
+    if (cudaStreamSynchronize(d0->stream) != cudaSuccess) cudaGetLastError();
+    free_plan(d0, cache->plans.front());
+    cache->plans.erase(cache->plans.begin());
+  }
+  cache->plans.push_back(p);
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(d0->stream, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    const cudaError_t e1 = enqueue_batch(doms, p, d0->stream);
+    const cudaError_t e2 = cudaStreamEndCapture(d0->stream, &g);
+    if (e1 == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&p->exec, g, 0) != cudaSuccess)
+      p->exec = nullptr;
+    if (g) cudaGraphDestroy(g);
+  }
+  cudaGetLastError();  // a capture the driver refused leaves the direct launches
+  *out = p;
   return LBM_OK;
 }
 
@@ -438,6 +326,8 @@ static lbm_status step_batch(lbm_domain* const* doms, int32_t n, int32_t steps, 
     if (doms[i]->desc.device != d0->desc.device) return d0->fail(LBM_ERR_INVALID_ARG, "mixed devices in batch");
     if (doms[i]->tape) return d0->fail(LBM_ERR_UNSUPPORTED, "batched stepping does not record tapes");
     if (doms[i]->walls) return d0->fail(LBM_ERR_UNSUPPORTED, "batched domains cannot have wall faces");
+    if (!fits_32bit_index(doms[i]->blocks[0].N))
+      return d0->fail(LBM_ERR_UNSUPPORTED, "batched domains must have 27 N < 2^32");
     if (*doms[i]->h_err & 1) return d0->fail(LBM_ERR_DIVERGED, "a domain of the batch has diverged");
   }
   if (steps == 0) return LBM_OK;
@@ -454,77 +344,24 @@ static lbm_status step_batch(lbm_domain* const* doms, int32_t n, int32_t steps, 
   }
   for (cudaEvent_t ev : evs) cudaEventDestroy(ev);
 
-  BatchCache* cache = static_cast<BatchCache*>(d0->batch_plan);
-  if (!cache) {
-    cache = new (std::nothrow) BatchCache();
-    if (!cache) return d0->fail(LBM_ERR_OOM, "out of host memory");
-    d0->batch_plan = cache;
-  }
+  // whole graphs, then the rest (with the diagnostics in its last step)
   BatchPlan* p = nullptr;
-  for (size_t k = 0; k < cache->plans.size() && !p; ++k) {
-    BatchPlan* q = cache->plans[k];
-    bool same = q->steps == steps && q->red == red && (int)q->serials.size() == n;
-    for (int i = 0; i < n && same; ++i)
-      same = q->serials[i] == doms[i]->serial && q->curs[i] == doms[i]->blocks[0].cur;
-    if (same) {
-      p = q;
-      cache->plans.erase(cache->plans.begin() + k);
-      cache->plans.push_back(p);
+  for (int left = steps; left > 0;) {
+    const int now = std::min(left, kGraphSteps);
+    const lbm_status st = batch_plan(doms, n, now, red && now == left, &p);
+    if (st != LBM_OK) return st;
+    const cudaError_t e = p->exec ? cudaGraphLaunch(p->exec, s) : enqueue_batch(doms, p, s);
+    if (e != cudaSuccess) return d0->cuda_fail(e, "batched launch");
+    for (int i = 0; i < n; ++i) {
+      Block& B = doms[i]->blocks[0];
+      if (now & 1) B.cur ^= 1;
+      doms[i]->steps += now;
     }
+    left -= now;
   }
-  if (!p) {
-    if (!cache->chunk) {
-      int chunk = 256, threads = 256;
-      lbm_status st = tune_chunk(doms, n, &chunk, &threads);
-      if (st != LBM_OK) return st;
-      cache->chunk = chunk;
-      cache->threads = threads;
-    }
-    while (cache->plans.size() >= kMaxBatchPlans) {
-      free_plan(d0, cache->plans.front());
-      cache->plans.erase(cache->plans.begin());
-    }
-    p = new (std::nothrow) BatchPlan();
-    if (!p) return d0->fail(LBM_ERR_OOM, "out of host memory");
-    // the fused diagnostics end every work item with a block-wide sum: their plans take work
-    // items 4x the tuned size (measured on the 64-plume batch: 1.23 -> 1.12 ms per step;
-    // the plain step does not change with the item size in that range)
-    const int chunk = red ? 4 * cache->chunk : cache->chunk;
-    lbm_status st = build_plan(doms, n, chunk, p);
-    if (st == LBM_OK && red) {
-      p->chunk = chunk;
-      st = add_red_buffers(doms, n, p);
-    }
-    if (st != LBM_OK) { free_plan(d0, p); return st; }
-    p->threads = cache->threads;
-    cache->plans.push_back(p);
-    p->steps = steps;
-    p->grid = std::min(resident_blocks(d0->desc.storage, p->i32, p->threads, red), std::max(1, p->n_items));
-    // capture: reset the barrier, then the cooperative persistent launch (and the fused
-    // diagnostics' sums and read-back)
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-      cudaError_t e1 = enqueue_batch(d0, p, steps, s);
-      cudaError_t e2 = cudaStreamEndCapture(s, &g);
-      if (e1 == cudaSuccess && e2 == cudaSuccess && g) {
-        e = cudaGraphInstantiate(&p->exec, g, 0);
-        p->captured = e == cudaSuccess;
-        if (!p->captured) p->exec = nullptr;
-      }
-      if (g) cudaGraphDestroy(g);
-    }
-    cudaGetLastError();  // a capture the driver refused leaves the direct launch below
-  }
-  cudaError_t e = p->captured ? cudaGraphLaunch(p->exec, s) : enqueue_batch(d0, p, steps, s);
-  if (e != cudaSuccess) return d0->cuda_fail(e, "batched launch");
-  for (int i = 0; i < n; ++i) {
-    Block& B = doms[i]->blocks[0];
-    if (steps & 1) B.cur ^= 1;
-    doms[i]->steps += steps;
-  }
+  cudaError_t e = cudaSuccess;
   // every domain's stream waits for the batch (each node reports divergence into its own
-  // domain's error word; a barrier timeout is reported by the first domain)
+  // domain's error word)
   cudaEvent_t done;
   if (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess) {
     cudaEventRecord(done, s);

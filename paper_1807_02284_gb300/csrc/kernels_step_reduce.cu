@@ -166,23 +166,26 @@ static void launch_step2_reduce_t(const BlockView& v, dim3 grid, dim3 block, int
 // 32-bit indexing only (27 N < 2^32): the caller checks fits_32bit_index.  A two-node bound
 // code runs k_step2_reduce (same CTA grid and records) where the block allows pairs and the
 // CTA is whole warps (its warp w owns the 32-node groups 2w and 2w + 1).
-cudaError_t launch_step_reduce(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
-                               int minb, double* partials, double* out, double* out5) {
+cudaError_t launch_step_records(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
+                                int minb, double* partials) {
   if (step_is_pair(minb) && step_pair_ok(v, storage, bx, by) && bx * by <= 256 &&
       ((bx / 2) * by) % 32 == 0) {
     dim3 block(bx / 2, by, 1);
     const dim3 grid = tile_grid(v.nx / 2, v.ny, (unsigned)v.nz, bx / 2, by);
     if (storage == ST_FP16) launch_step2_reduce_t<__half>(v, grid, block, minb - STEP_PAIR, partials, s);
     else launch_step2_reduce_t<float>(v, grid, block, minb - STEP_PAIR, partials, s);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_reduce_columns(partials, step_reduce_ctas(v, bx, by), out, s, out5);
+    return cudaGetLastError();
   }
   dim3 block(bx, by, 1);
   const dim3 grid = tile_grid(v.nx, v.ny, (unsigned)v.nz, bx, by);
   if (storage == ST_FP16) launch_step_reduce_t<__half>(v, grid, block, minb, partials, s);
   else launch_step_reduce_t<float>(v, grid, block, minb, partials, s);
-  const cudaError_t e = cudaGetLastError();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_step_reduce(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
+                               int minb, double* partials, double* out, double* out5) {
+  const cudaError_t e = launch_step_records(v, storage, bx, by, s, minb, partials);
   if (e != cudaSuccess) return e;
   return launch_reduce_columns(partials, step_reduce_ctas(v, bx, by), out, s, out5);
 }

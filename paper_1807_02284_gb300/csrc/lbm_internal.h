@@ -81,12 +81,6 @@ struct MapArgs {
   const float* ghost_blend;
 };
 
-// One tile of the batched work list: a BX x BY patch of one z-plane of one simulation.
-struct WorkItem {
-  int view;            // index into the BlockView array
-  int x0, y0, z;
-};
-
 // ---- kernels_step.cu
 // Register-bound code of the collide-stream launch (chosen by pick_tiles with the tile
 // bx x by of nodes): 3 or 4 = CTAs of bx by one-node threads per SM; STEP_PAIR + b = the
@@ -169,10 +163,6 @@ struct RedItem {
 cudaError_t launch_reduce_items(int storage, const RedItem* items, int n_items,
                                 const RedMember* members, int n_members, double* records,
                                 double* out, cudaStream_t s);
-// the per-member sums of item records written by another kernel (the batched step's fused
-// diagnostics): member i's items are records first_item .. first_item + n_items - 1
-cudaError_t launch_reduce_item_records(const double* records, const RedMember* members, int n,
-                                      double* out, cudaStream_t s);
 // the six sums over `n` per-CTA records of 8 doubles (partials[8 i + value]); the buffer
 // holds 8 n + 6 * 128 doubles (the records, then the first stage's sums)
 cudaError_t launch_reduce_columns(double* partials, size_t n, double* out, cudaStream_t s,
@@ -181,6 +171,9 @@ cudaError_t launch_reduce_columns(double* partials, size_t n, double* out, cudaS
 // the stored state in `out` (same six doubles as launch_reduce); `partials` holds
 // 8 * step_reduce_ctas(v, bx, by) + 6 * 128 doubles
 size_t step_reduce_ctas(const BlockView& v, int bx, int by);
+// the step alone: its CTA records (8 * step_reduce_ctas doubles) without their sums
+cudaError_t launch_step_records(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
+                                int minb, double* partials);
 cudaError_t launch_step_reduce(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
                                int minb, double* partials, double* out, double* out5 = nullptr);
 
@@ -200,9 +193,5 @@ cudaError_t launch_set_ghost_layer(uint8_t* flags, int nx, int ny, int nz, cudaS
 // outer layer of a block surrounded by a far-field block: GHOST on (except obstacle and
 // inflow nodes, which keep their own update) or off
 cudaError_t launch_outer_ghost(uint8_t* flags, int nx, int ny, int nz, int on, cudaStream_t s);
-
-// ---- kernels_batch.cu
-cudaError_t launch_step_batch(const BlockView* views_dev, const WorkItem* items, int n_items,
-                              int storage, int bx, int by, int grid, cudaStream_t s);
 
 }  // namespace lbm
