@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "lbm_cell.cuh"
+#include "reduce_util.cuh"
 #include "runtime.h"
 
 namespace lbm {
@@ -63,32 +64,21 @@ __device__ __forceinline__ bool grid_barrier(BarrierState* bs, unsigned int nblo
   return ok != 0;
 }
 
-// The six sums of every member over its CTA records of the diagnostics step (8 doubles each),
-// one CTA per member: thread t takes records t, t + 256, ... in order, then a fixed tree; the
-// member's device error word rides along in slot 6.
-__global__ void __launch_bounds__(256) k_batch_records(const double* __restrict__ records,
+// The six sums of every member over its CTA records of the diagnostics step (8 floats each),
+// one CTA per member, one warp per value: lane l takes records l, l + 32, ... in order, then the
+// shuffle tree; the member's device error word rides along in slot 6.
+__global__ void __launch_bounds__(192) k_batch_records(const float* __restrict__ records,
                                                        const RedMember* __restrict__ members,
                                                        double* __restrict__ out) {
-  __shared__ double sh[6][256];
   const RedMember m = members[blockIdx.x];
-  const int t = threadIdx.x;
-  double s[6] = {0, 0, 0, 0, 0, 0};
-  for (int i = t; i < m.n_items; i += 256) {
-#pragma unroll
-    for (int v = 0; v < 6; ++v) s[v] += records[(size_t)(m.first_item + i) * 8 + v];
-  }
-#pragma unroll
-  for (int v = 0; v < 6; ++v) sh[v][t] = s[v];
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (t < w) {
-#pragma unroll
-      for (int v = 0; v < 6; ++v) sh[v][t] += sh[v][t + w];
-    }
-    __syncthreads();
-  }
-  if (t < 6) out[(size_t)blockIdx.x * 8 + t] = sh[t][0];
-  if (t == 6) out[(size_t)blockIdx.x * 8 + 6] = (double)*m.err;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const float* rec = records + (size_t)m.first_item * 8 + w;
+  double s = 0;
+#pragma unroll 8
+  for (int i = lane; i < m.n_items; i += 32) s += (double)__ldg(rec + (size_t)i * 8);
+  s = warp_sum(s);
+  if (lane == 0) out[(size_t)blockIdx.x * 8 + w] = s;
+  if (threadIdx.x == 0) out[(size_t)blockIdx.x * 8 + 6] = (double)*m.err;
 }
 
 // One captured call: the launches of a set of domains from a given assignment of time levels
@@ -102,7 +92,7 @@ struct BatchPlan {
   // error word, 8 doubles each) copied to pinned host memory by the same graph
   bool red = false;
   std::vector<int> first;       // each member's first record
-  double* records = nullptr;
+  float* records = nullptr;
   RedMember* members = nullptr;
   double* out_dev = nullptr;
   double* out_host = nullptr;
@@ -151,7 +141,7 @@ static lbm_status add_red_buffers(lbm_domain* const* doms, int n, BatchPlan* p) 
     at += cnt;
   }
   if (at > (size_t)INT32_MAX) return d0->fail(LBM_ERR_UNSUPPORTED, "batch too large for one diagnostics pass");
-  p->records = static_cast<double*>(d0->dev_alloc(at * 8 * sizeof(double)));
+  p->records = static_cast<float*>(d0->dev_alloc(at * 8 * sizeof(float)));
   p->members = static_cast<RedMember*>(d0->dev_alloc((size_t)n * sizeof(RedMember)));
   p->out_dev = static_cast<double*>(d0->dev_alloc((size_t)n * 8 * sizeof(double)));
   p->out5_dev = static_cast<double*>(d0->dev_alloc((size_t)n * 5 * sizeof(double)));
@@ -184,7 +174,7 @@ static cudaError_t enqueue_member(lbm_domain* const* doms, const BatchPlan* p, i
 
 static cudaError_t enqueue_sums(const BatchPlan* p, cudaStream_t s) {
   const int n = (int)p->serials.size();
-  k_batch_records<<<n, 256, 0, s>>>(p->records, p->members, p->out_dev);
+  k_batch_records<<<n, 192, 0, s>>>(p->records, p->members, p->out_dev);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return cudaMemcpyAsync(p->out_host, p->out_dev, (size_t)n * 8 * sizeof(double),

@@ -56,42 +56,52 @@ __global__ void __launch_bounds__(192) k_reduce_final(const double* partials, in
   }
 }
 
-// n records of 8 doubles (6 sums + 2 unused), summed in two fixed-order stages so that many
-// SMs share the reads: CTA s of stage 1 sums slice s of the records (thread t: records
-// t, t + 256, ... of the slice, in order, then a fixed tree per value) into
-// stage[s * 6 + value]; stage 2 is k_reduce_final over those partials.
-constexpr int COL_SLICES = 128;
-
-__global__ void __launch_bounds__(256) k_reduce_records(const double* rec, size_t n,
-                                                        double* stage) {
-  __shared__ double sh[6][256];
-  const int sl = blockIdx.x;
-  const size_t per = (n + COL_SLICES - 1) / COL_SLICES;
-  const size_t lo = per * sl, hi = lo + per < n ? lo + per : n;
-  double s[6] = {0, 0, 0, 0, 0, 0};
-  for (size_t i = lo + threadIdx.x; i < hi; i += 256) {
-#pragma unroll
-    for (int v = 0; v < 6; ++v) s[v] += rec[i * 8 + v];
+// n records of 8 floats (6 sums + 2 unused), summed in FP64 in a fixed order in one launch: warp v
+// of CTA s sums value v over slice s of the records (lane l: records l, l + 32, ... in order,
+// then the shuffle tree) into stage[s * 6 + v], and the last CTA to finish (a device counter,
+// which it resets) sums the slices the same way.  The FP64 adds bound it (an SM issues one for a
+// warp in about 16 cycles), so a slice has 256 records until there are RED_SLICES of them, and
+// no thread adds anything but its own lane's sum.  One launch in place of two, half the record
+// bytes, and the results and the error word go to pinned memory without a copy of their own.
+__global__ void __launch_bounds__(192) k_reduce_records(const float* __restrict__ rec, size_t n,
+                                                        RedSink k) {
+  __shared__ double sh[6];
+  __shared__ unsigned last;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const size_t per = (n + gridDim.x - 1) / gridDim.x;
+  const size_t lo = per * blockIdx.x, hi = lo + per < n ? lo + per : n;
+  double s = 0;
+#pragma unroll 8
+  for (size_t i = lo + lane; i < hi; i += 32) s += (double)__ldg(rec + (8 * i + w));
+  s = warp_sum(s);
+  if (lane == 0) {
+    k.stage[blockIdx.x * 6 + w] = s;
+    __threadfence();
   }
-#pragma unroll
-  for (int v = 0; v < 6; ++v) sh[v][threadIdx.x] = s[v];
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-#pragma unroll
-      for (int v = 0; v < 6; ++v) sh[v][threadIdx.x] += sh[v][threadIdx.x + w];
-    }
-    __syncthreads();
+  if (t == 0) last = atomicAdd(k.counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double x = 0;
+#pragma unroll 4
+  for (int i = lane; i < (int)gridDim.x; i += 32) x += __ldcg(k.stage + (i * 6 + w));
+  x = warp_sum(x);
+  if (lane == 0) {
+    sh[w] = x;
+    k.out[w] = x;
+    if (k.host6) k.host6[w] = x;
   }
-  if (threadIdx.x < 6) stage[sl * 6 + threadIdx.x] = sh[threadIdx.x][0];
+  __syncthreads();
+  if (k.out5 && t < 5) k.out5[t] = t == 0 ? sh[0] + sh[1] : sh[t + 1];
+  if (t == 32) *k.counter = 0u;
+  if (t == 64 && k.host_err) *k.host_err = *k.err;
 }
 
-// `partials` holds 8 n + 6 COL_SLICES doubles: the records, then the stage-1 sums.
-cudaError_t launch_reduce_columns(double* partials, size_t n, double* out, cudaStream_t s,
-                                  double* out5) {
-  double* stage = partials + 8 * n;
-  k_reduce_records<<<COL_SLICES, 256, 0, s>>>(partials, n, stage);
-  k_reduce_final<<<1, 192, 0, s>>>(stage, COL_SLICES, out, out5);
+cudaError_t launch_reduce_records(const float* records, size_t n, const RedSink& sink, cudaStream_t s) {
+  const size_t slices = (n + 255) / 256;
+  const unsigned g = (unsigned)(slices < 1 ? 1 : slices < RED_SLICES ? slices : RED_SLICES);
+  k_reduce_records<<<g, 192, 0, s>>>(records, n, sink);
   return cudaGetLastError();
 }
 

@@ -268,18 +268,33 @@ __device__ __forceinline__ void wall_regularize(float (&d)[27], const BlockView&
 
 // Where a node writes the moments of the state it stores, for the diagnostics fused into
 // the step (the quantities lbm_reduce sums: node count, rho - 1, j, |j|^2 / (2 rho)): six
-// floats at nm[0], nm[stride], ..., nm[5 stride] (shared memory, one column per thread).
+// floats at nm[0], nm[stride], ..., nm[5 stride] (shared memory, one column per thread; the
+// caller zeroes it first).  put adds to the column, so the two nodes of a pair share one:
+// 0 + v0 + v1 rounds once, like the first stage of the one-node kernel's shuffle tree.
 struct NodeMomentsOut {
   float* nm;
   int stride;
-  __device__ __forceinline__ void put(float drho, float jx, float jy, float jz, float inv_rho) const {
-    nm[0] = 1.0f;
-    nm[stride] = drho;
-    nm[2 * stride] = jx;
-    nm[3 * stride] = jy;
-    nm[4 * stride] = jz;
+  static __device__ __forceinline__ float energy(float jx, float jy, float jz, float inv_rho) {
     const float jj = __fmaf_rn(jz, jz, __fmaf_rn(jy, jy, __fmul_rn(jx, jx)));
-    nm[5 * stride] = __fmul_rn(__fmul_rn(0.5f, jj), inv_rho);   // explicit: one value per node
+    return __fmul_rn(__fmul_rn(0.5f, jj), inv_rho);   // explicit: one value per node
+  }
+  __device__ __forceinline__ void put(float drho, float jx, float jy, float jz, float inv_rho) const {
+    nm[0] += 1.0f;
+    nm[stride] = __fadd_rn(nm[stride], drho);
+    nm[2 * stride] = __fadd_rn(nm[2 * stride], jx);
+    nm[3 * stride] = __fadd_rn(nm[3 * stride], jy);
+    nm[4 * stride] = __fadd_rn(nm[4 * stride], jz);
+    nm[5 * stride] = __fadd_rn(nm[5 * stride], energy(jx, jy, jz, inv_rho));
+  }
+  // both nodes of a pair (the column is still zero)
+  __device__ __forceinline__ void put_pair(float2 drho, float2 jx, float2 jy, float2 jz,
+                                           float2 inv_rho) const {
+    nm[0] = 2.0f;
+    nm[stride] = __fadd_rn(drho.x, drho.y);
+    nm[2 * stride] = __fadd_rn(jx.x, jx.y);
+    nm[3 * stride] = __fadd_rn(jy.x, jy.y);
+    nm[4 * stride] = __fadd_rn(jz.x, jz.y);
+    nm[5 * stride] = __fadd_rn(energy(jx.x, jy.x, jz.x, inv_rho.x), energy(jx.y, jy.y, jz.y, inv_rho.y));
   }
 };
 
@@ -495,13 +510,12 @@ template <typename T>
 constexpr bool pair_corners_async() { return sizeof(T) == 2; }
 
 // slot: this thread's 16 shared-memory floats (slot[i * stride], i < 16) for the corners
-// when pair_corners_async<T>(), unused otherwise.  RED: the two nodes' moments go through
-// nm0 and nm1 as cell_update's RED form writes them.
+// when pair_corners_async<T>(), unused otherwise.  RED: the two nodes' moments are added to
+// the column nm.
 template <typename T, typename IT, bool WALLS, bool RED = false>
 __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int y, int z,
                                                  float* slot, int stride,
-                                                 const NodeMomentsOut* nm0 = nullptr,
-                                                 const NodeMomentsOut* nm1 = nullptr) {
+                                                 const NodeMomentsOut* nm = nullptr) {
   const IT N = (IT)v.N;
   const IT nxI = (IT)v.nx, nxyI = (IT)v.nx * (IT)v.ny;
   const IT row = nxyI * (IT)z + nxI * (IT)y;
@@ -510,8 +524,8 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
   const uint8_t fl0 = (uint8_t)(fl2 & 0xffu), fl1 = (uint8_t)(fl2 >> 8);
   constexpr uint8_t kNodeWise = F_SOLID | F_INFLOW | F_GHOST | F_NEAR_SOLID | F_WALL | F_OBST_WALL;
   if (!inner_yz(v, y, z) || ((fl0 | fl1) & kNodeWise)) {
-    cell_update<T, IT, false, WALLS, RED>(v, x, y, z, nm0);
-    cell_update<T, IT, false, WALLS, RED>(v, x + 1, y, z, nm1);
+    cell_update<T, IT, false, WALLS, RED>(v, x, y, z, nm);
+    cell_update<T, IT, false, WALLS, RED>(v, x + 1, y, z, nm);
     return;
   }
   const T* __restrict__ din = static_cast<const T*>(v.d_in);
@@ -529,11 +543,7 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
   const float2 ux = vmul(d[kap(1, 0, 0)], inv), uy = vmul(d[kap(0, 1, 0)], inv),
                uz = vmul(d[kap(0, 0, 1)], inv);
   flag_error(v.err, unphysical(drho.x, ux.x, uy.x, uz.x) || unphysical(drho.y, ux.y, uy.y, uz.y));
-  if constexpr (RED) {
-    const float2 jx = d[kap(1, 0, 0)], jy = d[kap(0, 1, 0)], jz = d[kap(0, 0, 1)];
-    nm0->put(drho.x, jx.x, jy.x, jz.x, inv.x);
-    nm1->put(drho.y, jx.y, jy.y, jz.y, inv.y);
-  }
+  if constexpr (RED) nm->put_pair(drho, d[kap(1, 0, 0)], d[kap(0, 1, 0)], d[kap(0, 0, 1)], inv);
 
   const bool src0 = (fl0 & F_SCALAR_SRC) != 0, src1 = (fl1 & F_SCALAR_SRC) != 0;
   constexpr bool kAsync = pair_corners_async<T>();

@@ -163,19 +163,30 @@ struct RedItem {
 cudaError_t launch_reduce_items(int storage, const RedItem* items, int n_items,
                                 const RedMember* members, int n_members, double* records,
                                 double* out, cudaStream_t s);
-// the six sums over `n` per-CTA records of 8 doubles (partials[8 i + value]); the buffer
-// holds 8 n + 6 * 128 doubles (the records, then the first stage's sums)
-cudaError_t launch_reduce_columns(double* partials, size_t n, double* out, cudaStream_t s,
-                                  double* out5 = nullptr);
+// Where the sums of a step's records go: the six values (device), and where given the five
+// diagnostics in the lbm_reduce layout (device), the six values and the error word in pinned
+// host memory, written by the kernel itself (visible once the stream has passed it).
+struct RedSink {
+  double* out = nullptr;
+  double* out5 = nullptr;
+  double* host6 = nullptr;
+  const int* err = nullptr;
+  int* host_err = nullptr;
+  double* stage = nullptr;        // 6 * RED_SLICES doubles of scratch
+  unsigned* counter = nullptr;    // zero between launches
+};
+constexpr int RED_SLICES = 512;
+// the six sums over `n` per-CTA records of 8 floats (records[8 i + value])
+cudaError_t launch_reduce_records(const float* records, size_t n, const RedSink& sink, cudaStream_t s);
 // one collide-stream step of a block (32-bit indexing) that also leaves the diagnostics of
-// the stored state in `out` (same six doubles as launch_reduce); `partials` holds
-// 8 * step_reduce_ctas(v, bx, by) + 6 * 128 doubles
+// the stored state in the sink (same six doubles as launch_reduce); `records` holds
+// 8 * step_reduce_ctas(v, bx, by) floats
 size_t step_reduce_ctas(const BlockView& v, int bx, int by);
-// the step alone: its CTA records (8 * step_reduce_ctas doubles) without their sums
+// the step alone: its CTA records without their sums
 cudaError_t launch_step_records(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
-                                int minb, double* partials);
+                                int minb, float* records);
 cudaError_t launch_step_reduce(const BlockView& v, int storage, int bx, int by, cudaStream_t s,
-                               int minb, double* partials, double* out, double* out5 = nullptr);
+                               int minb, float* records, const RedSink& sink);
 
 // ---- coupling.cu
 cudaError_t launch_map(const MapArgs& a, int storage, cudaStream_t s);

@@ -262,6 +262,9 @@ lbm_status lbm_create_domain(const lbm_domain_desc* desc, lbm_domain** out) {
   if (!dom->d_err || !dom->d_partials || !dom->d_red) {
     g_create_error = "allocation failed"; lbm_destroy_domain(dom); return LBM_ERR_OOM;
   }
+  // word 0: the error word; word 8: the arrival counter of the diagnostics' sums
+  e = cudaMemsetAsync(dom->d_err, 0, 64, dom->stream);
+  if (e != cudaSuccess) { g_create_error = cudaGetErrorString(e); lbm_destroy_domain(dom); return LBM_ERR_CUDA; }
 
   Block B;
   B.nx = desc->dims[0]; B.ny = desc->dims[1]; B.nz = desc->dims[2];

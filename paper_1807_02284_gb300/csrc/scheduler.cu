@@ -331,17 +331,22 @@ lbm_status lbm_domain::advance(int n) {
 // indexing) also sums the diagnostics of the state it stores, so that reading mass, momentum
 // and energy back after a step costs no second pass over the populations.  Other domains
 // take the n steps and lbm_reduce of block 0.
-// Enqueues n steps and the diagnostics of block 0's new state: the 6 sums into dom->d_red
-// and, when out5 (device) is given, the 5 combined values.  On a single-block domain with
-// 27 N < 2^32 the last step's own kernel sums them; otherwise a separate reduction follows.
-static lbm_status enqueue_step_reduce(lbm_domain* dom, int32_t n, double* out5) {
+// Enqueues n steps and the diagnostics of block 0's new state: the 6 sums into dom->d_red,
+// the 5 combined values into out5 (device, may be null), the 6 sums into h_red (`to_host`)
+// and the error word into h_err.  On a single-block domain with 27 N < 2^32 the last step's
+// own kernel sums them; otherwise a separate reduction follows.
+static lbm_status enqueue_step_reduce(lbm_domain* dom, int32_t n, double* out5, bool to_host) {
   Block& B = dom->blocks[0];
   if (dom->blocks.size() > 1 || !fits_32bit_index(B.N)) {
     lbm_status st = dom->advance(n);
     if (st != LBM_OK) return st;
-    const cudaError_t e = launch_reduce(B.lv[B.cur].f, dom->desc.storage, B.flags, B.N,
-                                        dom->d_partials, dom->d_red, dom->stream, out5);
-    return e == cudaSuccess ? LBM_OK : dom->cuda_fail(e, "reduce");
+    cudaError_t e = launch_reduce(B.lv[B.cur].f, dom->desc.storage, B.flags, B.N,
+                                  dom->d_partials, dom->d_red, dom->stream, out5);
+    if (e == cudaSuccess && to_host)
+      e = cudaMemcpyAsync(dom->h_red, dom->d_red, 6 * sizeof(double), cudaMemcpyDeviceToHost, dom->stream);
+    if (e != cudaSuccess) return dom->cuda_fail(e, "reduce");
+    dom->post_error_probe();
+    return LBM_OK;
   }
   lbm_status st = dom->advance(n - 1);
   if (st == LBM_OK) st = tape_before_step(dom);
@@ -349,15 +354,25 @@ static lbm_status enqueue_step_reduce(lbm_domain* dom, int32_t n, double* out5) 
   const int nxt = B.cur ^ 1;
   const BlockView v = dom->view(0, B.cur, nxt);
   const size_t ctas = step_reduce_ctas(v, B.bx, B.by);
-  if (ctas > dom->step_partials_n) {
-    if (dom->d_step_partials) dom->dev_free(dom->d_step_partials);
-    dom->step_partials_n = 0;
-    dom->d_step_partials = static_cast<double*>(dom->dev_alloc((ctas * 8 + 6 * 128) * sizeof(double)));
-    if (!dom->d_step_partials) return dom->fail(LBM_ERR_OOM, "step-reduce partials");
-    dom->step_partials_n = ctas;
+  if (ctas > dom->step_records_n) {
+    if (dom->d_step_records) dom->dev_free(dom->d_step_records);
+    dom->step_records_n = 0;
+    dom->d_step_records = static_cast<float*>(
+        dom->dev_alloc(6 * RED_SLICES * sizeof(double) + ctas * 8 * sizeof(float)));
+    if (!dom->d_step_records) return dom->fail(LBM_ERR_OOM, "step-reduce records");
+    dom->step_records_n = ctas;
   }
+  RedSink sink;
+  sink.out = dom->d_red;
+  sink.out5 = out5;
+  sink.host6 = to_host ? dom->h_red : nullptr;
+  sink.err = dom->d_err;
+  sink.host_err = dom->h_err;
+  sink.stage = reinterpret_cast<double*>(dom->d_step_records);
+  sink.counter = reinterpret_cast<unsigned*>(dom->d_err + 8);
+  float* records = dom->d_step_records + 2 * 6 * RED_SLICES;
   const cudaError_t e = launch_step_reduce(v, dom->desc.storage, B.bx, B.by, dom->stream, B.minb,
-                                           dom->d_step_partials, dom->d_red, out5);
+                                           records, sink);
   if (e != cudaSuccess) return dom->cuda_fail(e, "collide-stream launch");
   B.cur = nxt;
   ++dom->steps;
@@ -370,12 +385,11 @@ lbm_status lbm_step_reduce(lbm_domain* dom, int32_t n, double out[5]) {
   if (n < 1) return dom->fail(LBM_ERR_INVALID_ARG, "lbm_step_reduce needs at least one step");
   if (!out) return dom->fail(LBM_ERR_INVALID_ARG, "null output");
   if (*dom->h_err & 1) return dom->fail(LBM_ERR_DIVERGED, "divergence recorded by an earlier step");
-  lbm_status st = enqueue_step_reduce(dom, n, nullptr);
+  lbm_status st = enqueue_step_reduce(dom, n, nullptr, true);
   if (st != LBM_OK) return st;
-  const cudaError_t e = cudaMemcpyAsync(dom->h_red, dom->d_red, 6 * sizeof(double),
-                                        cudaMemcpyDeviceToHost, dom->stream);
-  if (e != cudaSuccess) return dom->cuda_fail(e, "reduce read-back");
-  st = dom->sync_and_check();
+  const cudaError_t e = cudaStreamSynchronize(dom->stream);
+  if (e != cudaSuccess) return dom->cuda_fail(e, "cudaStreamSynchronize");
+  st = dom->error_status();
   const double* r = dom->h_red;
   out[0] = r[0] + r[1];
   out[1] = r[2];
@@ -398,14 +412,11 @@ lbm_status lbm_step_reduce_async(lbm_domain* dom, int32_t n, double out[5], int6
     return dom->fail(LBM_ERR_CUDA, "cudaEventCreate");
   }
   double* d_out5 = dom->d_red + 8;
-  lbm_status st = enqueue_step_reduce(dom, n, d_out5);
+  lbm_status st = enqueue_step_reduce(dom, n, d_out5, false);
   if (st != LBM_OK) return st;
   cudaError_t e = cudaMemcpyAsync(out, d_out5, 5 * sizeof(double), cudaMemcpyDeviceToHost,
                                   dom->stream);
-  if (e == cudaSuccess) {
-    dom->post_error_probe();
-    e = cudaEventRecord(dom->result_ev[slot], dom->stream);
-  }
+  if (e == cudaSuccess) e = cudaEventRecord(dom->result_ev[slot], dom->stream);
   if (e != cudaSuccess) return dom->cuda_fail(e, "reduce read-back");
   *ticket = ++dom->results_issued;
   return LBM_OK;
