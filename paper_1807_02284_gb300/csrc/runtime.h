@@ -143,7 +143,7 @@ struct lbm_domain {
   void on_state_reset(int b);
   lbm_status advance(int n);            // Algorithm 1, n reference steps
   lbm_status advance_direct(int n);     // same, launched without graph capture
-  lbm_status advance_single(int m);     // m steps from one-step graphs (several blocks)
+  lbm_status advance_graph(int n, bool eager, bool* done);   // n steps as one captured graph
 };
 
 using Domain = lbm_domain;

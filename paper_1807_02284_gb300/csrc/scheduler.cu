@@ -11,14 +11,22 @@
 using namespace lbm;
 
 namespace lbm {
-// Captured step graphs, one per starting assignment of time levels (the `cur` level of every
-// block).  Each graph advances `chunk` reference steps, a multiple of the period after which
-// the level assignment repeats, so it ends in the assignment it started from.
+// Captured step graphs, keyed by the starting assignment of time levels (the `cur` level of
+// every block) and the number of reference steps: `chunk`-step graphs (a multiple of the period
+// after which the level assignment repeats, so they end in the assignment they started from),
+// one-step graphs of continuous-scale domains, and shorter runs of small single blocks.  They
+// hold level pointers and launch parameters only, so they outlive lbm_init_macro and
+// lbm_write_field; whatever changes a launch (blocks, walls, a tape) drops them.
 struct GraphCache {
-  std::vector<std::pair<std::vector<int>, cudaGraphExec_t>> exec;     // chunk-step graphs
-  std::vector<std::pair<std::vector<int>, cudaGraphExec_t>> single;   // one-step graphs
+  struct Entry {
+    std::vector<int> cur;
+    int steps;
+    cudaGraphExec_t exec;      // null: seen once, not captured yet
+  };
+  std::vector<Entry> entries;
   int chunk = 0;
 };
+constexpr size_t kMaxStepGraphs = 96;
 
 // Level assignment after one reference step (mirrors the schedule of multiscale_step).
 static std::vector<int> next_levels(const std::vector<lbm::Block>& blocks, std::vector<int> cur) {
@@ -84,10 +92,8 @@ void lbm_domain::pick_tiles(int b) {
 
 void lbm_domain::invalidate_graphs() {
   if (!graphs) return;
-  for (auto& kv : graphs->exec)
-    if (kv.second) cudaGraphExecDestroy(kv.second);
-  for (auto& kv : graphs->single)
-    if (kv.second) cudaGraphExecDestroy(kv.second);
+  for (auto& en : graphs->entries)
+    if (en.exec) cudaGraphExecDestroy(en.exec);
   delete graphs;
   graphs = nullptr;
 }
@@ -196,7 +202,6 @@ const void* lbm_domain::upload_small(const void* src, size_t bytes, lbm_status* 
 void lbm_domain::on_state_reset(int b) {
   (void)b;
   steps = 0;
-  invalidate_graphs();
   release_tape(this);
 }
 
@@ -223,45 +228,65 @@ lbm_status lbm_domain::advance_direct(int n) {
   return LBM_OK;
 }
 
-// Without a tape, steps are replayed from captured graphs of `chunk` reference steps (a
-// multiple of the level-rotation period, at least 16 steps); the remainder launches directly.
-// m reference steps of a continuous-scale domain from one-step graphs captured per level
-// assignment (the schedule of one step is 16 launches with forks and joins on several
-// streams; replaying it as one graph leaves the GPU no gaps between them).  Single-block
-// domains launch their one kernel directly.
-lbm_status lbm_domain::advance_single(int m) {
-  if (blocks.size() == 1 || !graphs) return advance_direct(m);
-  for (int i = 0; i < m; ++i) {
-    std::vector<int> key(blocks.size());
-    for (size_t b = 0; b < blocks.size(); ++b) key[b] = blocks[b].cur;
-    cudaGraphExec_t exec = nullptr;
-    for (auto& kv : graphs->single)
-      if (kv.first == key) exec = kv.second;
-    if (!exec) {
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-      const lbm_status st = multiscale_step(this);
-      cudaError_t e2 = cudaStreamEndCapture(stream, &g);
-      for (size_t b = 0; b < blocks.size(); ++b) blocks[b].cur = key[b];
-      if (st != LBM_OK || e2 != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return st != LBM_OK ? st : cuda_fail(e2, "step graph capture");
-      }
-      e = cudaGraphInstantiate(&exec, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-      graphs->single.push_back({key, exec});
-    }
-    const cudaError_t e = cudaGraphLaunch(exec, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
-    const std::vector<int> s = next_levels(blocks, key);
-    for (size_t b = 0; b < blocks.size(); ++b) blocks[b].cur = s[b];
-    ++steps;
+// n reference steps as one graph launch, captured on the first such call from this level
+// assignment (`eager`), or on the second (a run that may never come again).  *done = false:
+// nothing was launched.
+lbm_status lbm_domain::advance_graph(int n, bool eager, bool* done) {
+  *done = false;
+  std::vector<int> key(blocks.size());
+  for (size_t b = 0; b < blocks.size(); ++b) key[b] = blocks[b].cur;
+  GraphCache::Entry* en = nullptr;
+  for (auto& e : graphs->entries)
+    if (e.steps == n && e.cur == key) en = &e;
+  if (!en) {
+    if (graphs->entries.size() >= kMaxStepGraphs) return LBM_OK;
+    graphs->entries.push_back({key, n, nullptr});
+    en = &graphs->entries.back();
+    if (!eager) return LBM_OK;
   }
+  if (!en->exec) {
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
+    lbm_status st = LBM_OK;
+    for (int i = 0; i < n && st == LBM_OK; ++i) {
+      if (blocks.size() == 1) {
+        Block& B = blocks[0];
+        const cudaError_t el = launch_step(view(0, B.cur, B.cur ^ 1), desc.storage, B.bx, B.by, stream, B.minb);
+        if (el != cudaSuccess) st = cuda_fail(el, "collide-stream launch");
+        B.cur ^= 1;
+      } else {
+        st = multiscale_step(this);
+      }
+    }
+    const cudaError_t e2 = cudaStreamEndCapture(stream, &g);
+    for (size_t b = 0; b < blocks.size(); ++b) blocks[b].cur = key[b];
+    if (st != LBM_OK || e2 != cudaSuccess) {
+      if (g) cudaGraphDestroy(g);
+      return st != LBM_OK ? st : cuda_fail(e2, "step graph capture");
+    }
+    cudaGraphExec_t exec = nullptr;
+    e = cudaGraphInstantiate(&exec, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
+    en->exec = exec;
+  }
+  const cudaError_t e = cudaGraphLaunch(en->exec, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
+  std::vector<int> s = key;
+  for (int i = 0; i < n; ++i) s = next_levels(blocks, s);
+  for (size_t b = 0; b < blocks.size(); ++b) blocks[b].cur = s[b];
+  steps += n;
+  *done = true;
   return LBM_OK;
 }
 
+// Without a tape: whole chunks from chunk graphs; the rest of a continuous-scale domain step by
+// step from one-step graphs (the schedule of one step is 16 launches with forks and joins on
+// several streams; replaying it as one graph leaves the GPU no gaps between them), the rest
+// of a small single block (a step shorter than its launch takes the host: 3.8 us against
+// about 7 on a 32^3 block) from a graph of its length once it has come twice, of a larger one
+// launch by launch.
 lbm_status lbm_domain::advance(int n) {
   if (blocks.size() > 1) {  // stream and events of the fork/join schedule exist before capture
     cudaStream_t a = nullptr;
@@ -271,9 +296,9 @@ lbm_status lbm_domain::advance(int n) {
     if (!post_stream((int)blocks.size())) return fail(LBM_ERR_CUDA, "cudaStreamCreate");
   }
   if (tape != nullptr) return advance_direct(n);
-  std::vector<int> start(blocks.size());
-  for (size_t b = 0; b < blocks.size(); ++b) start[b] = blocks[b].cur;
   if (!graphs) {
+    std::vector<int> start(blocks.size());
+    for (size_t b = 0; b < blocks.size(); ++b) start[b] = blocks[b].cur;
     int period = 1;
     std::vector<int> s = next_levels(blocks, start);
     while (s != start && period < 64) { s = next_levels(blocks, s); ++period; }
@@ -282,49 +307,34 @@ lbm_status lbm_domain::advance(int n) {
     graphs->chunk = period * ((16 + period - 1) / period);
   }
   const int chunk = graphs->chunk;
-  if (n < 2 * chunk) return advance_single(n);
-  int done = 0;
-  while (n - done >= chunk) {
-    std::vector<int> key(blocks.size());
-    for (size_t b = 0; b < blocks.size(); ++b) key[b] = blocks[b].cur;
-    cudaGraphExec_t exec = nullptr;
-    for (auto& kv : graphs->exec)
-      if (kv.first == key) exec = kv.second;
-    if (!exec) {
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-      lbm_status st = LBM_OK;
-      for (int i = 0; i < chunk && st == LBM_OK; ++i) {
-        if (blocks.size() == 1) {
-          Block& B = blocks[0];
-          const cudaError_t el = launch_step(view(0, B.cur, B.cur ^ 1), desc.storage, B.bx, B.by, stream, B.minb);
-          if (el != cudaSuccess) st = cuda_fail(el, "collide-stream launch");
-          B.cur ^= 1;
-        } else {
-          st = multiscale_step(this);
-        }
-      }
-      cudaError_t e2 = cudaStreamEndCapture(stream, &g);
-      for (size_t b = 0; b < blocks.size(); ++b) blocks[b].cur = key[b];
-      if (st != LBM_OK || e2 != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return st != LBM_OK ? st : cuda_fail(e2, "step graph capture");
-      }
-      e = cudaGraphInstantiate(&exec, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-      graphs->exec.push_back({key, exec});
+  const bool multi = blocks.size() > 1;
+  bool ok = true;
+  if (n >= 2 * chunk)
+    while (n >= chunk && ok) {
+      const lbm_status st = advance_graph(chunk, true, &ok);
+      if (st != LBM_OK) return st;
+      if (ok) n -= chunk;
     }
-    cudaError_t e = cudaGraphLaunch(exec, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
-    std::vector<int> s = key;
-    for (int i = 0; i < chunk; ++i) s = next_levels(blocks, s);
-    for (size_t b = 0; b < blocks.size(); ++b) blocks[b].cur = s[b];
-    steps += chunk;
-    done += chunk;
+  if (multi) {
+    ok = true;
+    while (n > 0 && ok) {
+      const lbm_status st = advance_graph(1, true, &ok);
+      if (st != LBM_OK) return st;
+      if (ok) --n;
+    }
+  } else if (n >= 3 && blocks[0].N <= (size_t)1 << 18) {
+    // (a caller that captures the domain's stream itself gets the launches)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+      const int run = std::min(n, chunk);
+      const lbm_status st = advance_graph(run, false, &ok);
+      if (st != LBM_OK) return st;
+      if (ok) n -= run;
+    } else {
+      cudaGetLastError();
+    }
   }
-  return advance_single(n - done);
+  return advance_direct(n);
 }
 
 // lbm_step_reduce: n reference steps whose last one (on a single-block domain with 32-bit
