@@ -1075,7 +1075,8 @@ struct TapeState {
   bool multi = false;
   std::vector<std::vector<Level>> mck;        // [checkpoint][block]: state at the step start
   std::vector<std::vector<Level>> snap;       // [step of the segment][block]
-  std::vector<std::vector<Level>> scr;        // [block][level]: replay levels (+ a spare)
+  std::vector<std::vector<Level>> ver;        // [block]: versions 1.. of the block's levels (MsOp)
+  std::vector<Level> spare;                   // [block]: a plain step's result (aligned steps)
   std::vector<std::vector<AdjLevel>> lamb;    // [block][level]: adjoints of the replay levels
   std::vector<float*> grad;                   // [block]: dL/du_0 of the block
 };
@@ -1105,7 +1106,8 @@ void release_tape(lbm_domain* dom) {
   dom->dev_free(t->side);
   for (auto& v : t->mck) for (Level& L : v) free_level(dom, L);
   for (auto& v : t->snap) for (Level& L : v) free_level(dom, L);
-  for (auto& v : t->scr) for (Level& L : v) free_level(dom, L);
+  for (auto& v : t->ver) for (Level& L : v) free_level(dom, L);
+  for (Level& L : t->spare) free_level(dom, L);
   for (auto& v : t->lamb)
     for (AdjLevel& A : v) {
       dom->dev_free(A.f);
@@ -1227,7 +1229,11 @@ extern "C" lbm_status lbm_set_tape(lbm_domain* dom, int32_t every) {
 }
 
 // One operation of the Algorithm 1 schedule of a continuous-scale domain, on replay levels
-// numbered from a canonical start (every block's state at t_n in level 0).
+// numbered from a canonical start (every block's state at t_n in level 0).  The adjoints live
+// on these levels.  The values an operation reads and writes have versions (v_...): a step
+// writes a version of its own, a mapping into a version that the reverse sweep still needs
+// first copies it (copy_from), so after one replay of a reference step every operation's inputs
+// are there to reverse it.  Version 0 of a block is its state at t_n.
 struct MsOp {
   int kind = 0;                       // 0 collide-stream, 1 aligned collide-stream, 2 mapping
   int b = 0, in = 0, out = 0, al = 0; // block and levels of a (aligned) collide-stream
@@ -1236,7 +1242,54 @@ struct MsOp {
   int src = 0, lo = 0, hi = 0, dst = 0, dlv = 0;
   float theta = 0.f;
   uint8_t skip = 0;
+  bool opens = false;                 // a scale boundary written before the step into its level
+  int v_in = 0, v_out = 0, v_al = 0, v_lo = 0, v_hi = 0, v_dst = 0, copy_from = -1;
 };
+
+// Versions of the operations' values; versions[b] receives the number of block b's versions,
+// last[b] the one holding its state at the end of the step.
+static void ms_versions(std::vector<MsOp>& ops, const std::vector<int>& cur_end,
+                        std::vector<int>& versions, std::vector<int>& last) {
+  const int nb = (int)cur_end.size();
+  versions.assign(nb, 1);
+  std::vector<std::vector<int>> at(nb, std::vector<int>{0, -1, -1});   // [block][level]
+  std::vector<std::vector<char>> needed(nb, std::vector<char>{1});     // [block][version]
+  std::vector<char> open(nb, 0);       // the level's version was opened by its scale boundary
+  auto fresh = [&](int b, int level) {
+    needed[b].push_back(0);
+    return at[b][level] = versions[b]++;
+  };
+  for (MsOp& o : ops) {
+    if (o.kind != 2) {
+      o.v_in = at[o.b][o.in];
+      if (o.kind == 1) o.v_al = at[o.b][o.al];
+      needed[o.b][o.v_in] = 1;
+      if (o.kind == 1) needed[o.b][o.v_al] = 1;
+      o.v_out = open[o.b] ? at[o.b][o.out] : fresh(o.b, o.out);
+      open[o.b] = 0;
+      needed[o.b][o.v_out] = 1;        // its velocity (and an aligned step's populations)
+      continue;
+    }
+    o.v_lo = at[o.src][o.lo];
+    o.v_hi = at[o.src][o.hi];
+    needed[o.src][o.v_lo] = needed[o.src][o.v_hi] = 1;
+    if (o.opens) {
+      o.v_dst = fresh(o.dst, o.dlv);
+      open[o.dst] = 1;
+      continue;
+    }
+    o.v_dst = at[o.dst][o.dlv];
+    // (the scale boundary at t_n, into version 0, is written before anything reads it and
+    // comes out the same on every replay)
+    const bool refresh = o.v_dst == 0;
+    if (needed[o.dst][o.v_dst] && !refresh) {
+      o.copy_from = o.v_dst;
+      o.v_dst = fresh(o.dst, o.dlv);
+    }
+  }
+  last.resize(nb);
+  for (int b = 0; b < nb; ++b) last[b] = at[b][cur_end[b]];
+}
 
 // The operations of one reference step in the order multiscale_step issues them (its forked
 // mappings write nodes disjoint from the concurrent collide-stream, so this sequential order
@@ -1297,6 +1350,7 @@ static std::vector<MsOp> ms_ops(const lbm_domain* dom, std::vector<int>& cur) {
     for (int j = 1; j <= B.substeps; ++j) {
       const int out = (j == 1) ? A : (c == A ? Bv : A);
       ops.push_back(prior(j < B.substeps ? (float)(j * B.h) : 1.0f, out));
+      ops.back().opens = true;
       MsOp s;
       s.b = b; s.in = c; s.out = out;
       if (j == B.substeps && !exact) {
@@ -1320,56 +1374,73 @@ static std::vector<MsOp> ms_ops(const lbm_domain* dom, std::vector<int>& cur) {
   return ops;
 }
 
-static BlockView ms_view(lbm_domain* dom, TapeState* t, int b, int from, int to) {
-  BlockView v = dom->view(b, 0, 0);   // geometry, flags, rates, error word
-  const Level& F = t->scr[b][from];
-  const Level& T = t->scr[b][to];
-  v.d_in = F.f; v.u_in = F.u; v.c_in = F.c;
-  v.d_out = T.f; v.u_out = T.u; v.c_out = T.c;
-  return v;
-}
+// The values of one reference step: `start` holds every block's version 0.
+struct MsStep {
+  lbm_domain* dom;
+  TapeState* t;
+  std::vector<Level>* start;
+  const Level& at(int b, int version) const {
+    return version == 0 ? (*start)[b] : t->ver[b][version - 1];
+  }
+  BlockView view(int b, const Level& F, const Level& T) const {
+    BlockView v = dom->view(b, 0, 0);   // geometry, flags, rates, error word
+    v.d_in = F.f; v.u_in = F.u; v.c_in = F.c;
+    v.d_out = T.f; v.u_out = T.u; v.c_out = T.c;
+    return v;
+  }
+  MapArgs map_args(const MsOp& o) const {
+    const Block& S = dom->blocks[o.src];
+    const Block& D = dom->blocks[o.dst];
+    const Level &lo = at(o.src, o.v_lo), &hi = at(o.src, o.v_hi), &to = at(o.dst, o.v_dst);
+    MapArgs a{};
+    a.table = o.t->d;
+    a.n = o.t->n;
+    a.f_lo = lo.f;
+    a.f_hi = hi.f;
+    a.c_lo = lo.c;
+    a.c_hi = hi.c;
+    a.theta = o.theta;
+    a.src_flags = S.flags;
+    a.snx = S.nx; a.sny = S.ny; a.snz = S.nz; a.sN = S.N;
+    a.f_dst = to.f;
+    a.u_dst = to.u;
+    a.c_dst = to.c;
+    a.dst_flags = D.flags;
+    a.skip_mask = o.skip;
+    a.dN = D.N;
+    a.khat = o.t->khat;
+    a.rest_if_empty = (o.skip & F_GHOST) ? 0 : 1;   // prior maps write scale boundaries
+    return a;
+  }
+};
 
-static MapArgs ms_map_args(lbm_domain* dom, TapeState* t, const MsOp& o) {
-  const Block& S = dom->blocks[o.src];
-  const Block& D = dom->blocks[o.dst];
-  MapArgs a{};
-  a.table = o.t->d;
-  a.n = o.t->n;
-  a.f_lo = t->scr[o.src][o.lo].f;
-  a.f_hi = t->scr[o.src][o.hi].f;
-  a.c_lo = t->scr[o.src][o.lo].c;
-  a.c_hi = t->scr[o.src][o.hi].c;
-  a.theta = o.theta;
-  a.src_flags = S.flags;
-  a.snx = S.nx; a.sny = S.ny; a.snz = S.nz; a.sN = S.N;
-  a.f_dst = t->scr[o.dst][o.dlv].f;
-  a.u_dst = t->scr[o.dst][o.dlv].u;
-  a.c_dst = t->scr[o.dst][o.dlv].c;
-  a.dst_flags = D.flags;
-  a.skip_mask = o.skip;
-  a.dN = D.N;
-  a.khat = o.t->khat;
-  a.rest_if_empty = (o.skip & F_GHOST) ? 0 : 1;   // prior maps write scale boundaries
-  return a;
-}
-
-static cudaError_t ms_forward_op(lbm_domain* dom, TapeState* t, const MsOp& o, cudaStream_t s) {
-  if (o.kind == 2) return launch_map(ms_map_args(dom, t, o), ST_FP32, s);
-  const Block& B = dom->blocks[o.b];
-  BlockView v = ms_view(dom, t, o.b, o.in, o.out);
+static cudaError_t ms_forward_op(const MsStep& m, const MsOp& o, cudaStream_t s) {
+  if (o.kind == 2) {
+    if (o.copy_from >= 0) {
+      const cudaError_t e = copy_level(m.at(o.dst, o.v_dst), m.at(o.dst, o.copy_from),
+                                       m.dom->blocks[o.dst].N, s);
+      if (e != cudaSuccess) return e;
+    }
+    return launch_map(m.map_args(o), ST_FP32, s);
+  }
+  const Block& B = m.dom->blocks[o.b];
+  BlockView v = m.view(o.b, m.at(o.b, o.v_in), m.at(o.b, o.v_out));
   if (o.kind == 1) {
-    v.f_al0 = t->scr[o.b][o.al].f;
-    v.c_al0 = t->scr[o.b][o.al].c;
+    const Level& al = m.at(o.b, o.v_al);
+    v.f_al0 = al.f;
+    v.c_al0 = al.c;
     v.al0 = o.al0; v.al1 = o.al1; v.al2 = o.al2;
     return launch_step_align(v, B.bx, B.by, s, B.minb);
   }
   return launch_step(v, ST_FP32, B.bx, B.by, s, B.minb);
 }
 
-// Transpose of one operation, with its forward inputs present in the replay levels.
-static cudaError_t ms_reverse_op(lbm_domain* dom, TapeState* t, const MsOp& o, cudaStream_t s) {
+// Transpose of one operation, with its forward values in their versions.
+static cudaError_t ms_reverse_op(const MsStep& m, const MsOp& o, cudaStream_t s) {
+  lbm_domain* dom = m.dom;
+  TapeState* t = m.t;
   if (o.kind == 2) {
-    const MapArgs a = ms_map_args(dom, t, o);
+    const MapArgs a = m.map_args(o);
     if (a.n > 0)
       k_map_vjp<<<(a.n + 127) / 128, 128, 0, s>>>(a, t->lamb[o.dst][o.dlv], t->lamb[o.src][o.lo],
                                                     t->lamb[o.src][o.hi]);
@@ -1379,19 +1450,20 @@ static cudaError_t ms_reverse_op(lbm_domain* dom, TapeState* t, const MsOp& o, c
   const uint32_t N = (uint32_t)B.N;
   const int g = (int)std::min<size_t>((B.N + 255) / 256, 16384);
   AdjLevel lin = t->lamb[o.b][o.in], lout = t->lamb[o.b][o.out];
-  const float* u_next = t->scr[o.b][o.out].u;
+  const Level &in = m.at(o.b, o.v_in), &out = m.at(o.b, o.v_out);
+  const float* u_next = out.u;
   if (o.kind == 1) {
     // the sub-step's own velocity (the scalar's departure velocity) is not stored by an
     // aligned step: recompute the plain step into the spare level
-    const int spare = (int)t->scr[o.b].size() - 1;
-    cudaError_t e = launch_step(ms_view(dom, t, o.b, o.in, spare), ST_FP32, B.bx, B.by, s, B.minb);
+    const Level& spare = t->spare[o.b];
+    cudaError_t e = launch_step(m.view(o.b, in, spare), ST_FP32, B.bx, B.by, s, B.minb);
     if (e != cudaSuccess) return e;
-    u_next = t->scr[o.b][spare].u;
-    k_align_vjp_pre<<<g, 256, 0, s>>>(ms_view(dom, t, o.b, o.out, o.out), lout,
-                                      t->lamb[o.b][o.al], lin, o.al0, o.al1, o.al2);
+    u_next = spare.u;
+    k_align_vjp_pre<<<g, 256, 0, s>>>(m.view(o.b, out, out), lout, t->lamb[o.b][o.al], lin, o.al0,
+                                      o.al1, o.al2);
   }
   AdjArgs a;
-  a.fwd = ms_view(dom, t, o.b, o.in, o.in);
+  a.fwd = m.view(o.b, in, in);
   a.lam_in = lout.f; a.ups_in = lout.u; a.gam_in = lout.c;
   a.u_next = u_next;
   a.lam_out = lin.f; a.ups_out = lin.u; a.gam_out = lin.c;
@@ -1421,9 +1493,11 @@ static cudaError_t zero_adj(const AdjLevel& A, size_t N, cudaStream_t s) {
 
 // Reverse sweep of a continuous-scale domain: the recorded reference steps are reversed last
 // to first; each segment between checkpoints is replayed once to record every step's start
-// state, and each operation of a step is reversed after a replay of the operations before it
-// from that start state (the level buffers of refined blocks rotate, so an operation's
-// inputs may have been overwritten later in the step).
+// state, and each step once more from there, keeping a version of every value that its
+// operations read (MsOp), before the operations are reversed one after another.  (Replaying
+// the operations before each one from the step's start took K (K + 1) / 2 operations and K
+// copies of every block for K operations per step, 120 and 48 for a three-block domain of 1/1.5
+// and 1/2.25; @MS@.)
 static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* dL_dc,
                                      const float* dL_du, float* dL_du0, float* dL_dinflow) {
   TapeState* t = dom->tape;
@@ -1431,17 +1505,29 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
   const int nb = (int)dom->blocks.size();
   size_t nmax = 0;
   for (const Block& B : dom->blocks) nmax = std::max(nmax, B.N);
+  std::vector<int> cur_end, versions, last;
+  std::vector<MsOp> ops = ms_ops(dom, cur_end);
+  ms_versions(ops, cur_end, versions, last);
   // buffers
-  if (t->scr.empty()) {
-    t->scr.resize(nb);
+  if (t->lamb.empty()) {
+    t->ver.resize(nb);
+    t->spare.resize(nb);
     t->lamb.resize(nb);
     t->grad.assign(nb, nullptr);
     for (int b = 0; b < nb; ++b) {
       const size_t N = dom->blocks[b].N;
       const int levels = b == 0 ? 2 : 3;
-      t->scr[b].resize(b == 0 ? 2 : 4);
-      for (Level& L : t->scr[b])
+      t->ver[b].resize(versions[b] - 1);
+      for (Level& L : t->ver[b]) {
         if (!alloc_level(dom, N, L)) return dom->fail(LBM_ERR_OOM, "adjoint replay levels");
+        // (a scale boundary that no one has written yet is read with weight 0: keep it finite)
+        const cudaError_t e0 = cudaMemsetAsync(L.f, 0, N * 27 * sizeof(float), s);
+        const cudaError_t e1 = cudaMemsetAsync(L.u, 0, N * 3 * sizeof(float), s);
+        const cudaError_t e2 = cudaMemsetAsync(L.c, 0, N * sizeof(float), s);
+        if (e0 != cudaSuccess || e1 != cudaSuccess || e2 != cudaSuccess)
+          return dom->fail(LBM_ERR_CUDA, "adjoint replay levels");
+      }
+      if (b && !alloc_level(dom, N, t->spare[b])) return dom->fail(LBM_ERR_OOM, "adjoint replay levels");
       t->lamb[b].resize(levels);
       for (AdjLevel& A : t->lamb[b])
         if (!alloc_adj(dom, N, A)) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
@@ -1470,8 +1556,6 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
     lbm_status st = tape_before_step(dom);
     if (st != LBM_OK) return st;
   }
-  std::vector<int> cur_end;
-  const std::vector<MsOp> ops = ms_ops(dom, cur_end);
   cudaError_t e = cudaSuccess;
   for (int b = 0; b < nb && e == cudaSuccess; ++b)
     for (const AdjLevel& A : t->lamb[b])
@@ -1487,23 +1571,25 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
   const int n_seg = (n_steps + t->every - 1) / t->every;
   for (int sg = n_seg - 1; sg >= 0 && e == cudaSuccess; --sg) {
     const int len = std::min(t->every, n_steps - sg * t->every);
-    for (int b = 0; b < nb && e == cudaSuccess; ++b)
-      e = copy_level(t->scr[b][0], t->mck[sg][b], dom->blocks[b].N, s);
-    for (int i = 0; i < len && e == cudaSuccess; ++i) {
-      for (int b = 0; b < nb && e == cudaSuccess; ++b)
-        e = copy_level(t->snap[i][b], t->scr[b][0], dom->blocks[b].N, s);
-      if (i == len - 1) break;
+    auto replay = [&](int i) {
+      const MsStep m{dom, t, &t->snap[i]};
+      cudaError_t e = cudaSuccess;
       for (const MsOp& o : ops)
-        if (e == cudaSuccess) e = ms_forward_op(dom, t, o, s);
-      for (int b = 0; b < nb; ++b) std::swap(t->scr[b][0], t->scr[b][cur_end[b]]);
+        if (e == cudaSuccess) e = ms_forward_op(m, o, s);
+      return e;
+    };
+    for (int b = 0; b < nb && e == cudaSuccess; ++b)
+      e = copy_level(t->snap[0][b], t->mck[sg][b], dom->blocks[b].N, s);
+    for (int i = 0; i + 1 < len && e == cudaSuccess; ++i) {
+      e = replay(i);
+      const MsStep m{dom, t, &t->snap[i]};
+      for (int b = 0; b < nb && e == cudaSuccess; ++b)
+        e = copy_level(t->snap[i + 1][b], m.at(b, last[b]), dom->blocks[b].N, s);
     }
     for (int i = len - 1; i >= 0 && e == cudaSuccess; --i) {
-      for (int k = (int)ops.size() - 1; k >= 0 && e == cudaSuccess; --k) {
-        for (int b = 0; b < nb && e == cudaSuccess; ++b)
-          e = copy_level(t->scr[b][0], t->snap[i][b], dom->blocks[b].N, s);
-        for (int j = 0; j < k && e == cudaSuccess; ++j) e = ms_forward_op(dom, t, ops[j], s);
-        if (e == cudaSuccess) e = ms_reverse_op(dom, t, ops[k], s);
-      }
+      const MsStep m{dom, t, &t->snap[i]};
+      e = replay(i);
+      for (int k = (int)ops.size() - 1; k >= 0 && e == cudaSuccess; --k) e = ms_reverse_op(m, ops[k], s);
       // the adjoint of this step's start state is in level 0: it is the adjoint of the end
       // state of the step before, whose replay ends in the levels cur_end
       if (!(sg == 0 && i == 0))

@@ -24,3 +24,35 @@ def test_adjoint_at_tile_edges_matches_fp64_oracle(lib, dims, periodic):
     Lo, go, _ = oracle_grad(sc, target, 3)
     assert abs(L - Lo) <= 1e-5 * abs(Lo)
     assert rel(g, go.numpy()) <= 1e-5
+
+
+@pytest.mark.parametrize("h", [1 / 3.0, 1 / 3.5])
+def test_adjoint_of_blocks_with_more_than_two_levels_of_substeps(lib, h):
+    """Refined blocks whose sub-steps reuse a time level within one reference step (three exact
+    sub-steps, four with alignment): the scalar's departure velocity of each sub-step is its
+    own.  Bound 1e-4 relative L2 (FP32 against FP64 over 2 reference steps, 6 to 8 sub-steps,
+    with the mappings' atomic sums in any order)."""
+    import torch
+
+    from oracle import adjoint as oadj
+    from paper_1807_02284_gb300 import lbm
+    from tests.test_gpu_multiscale import gpu_multiscale
+    sc = synth.multiscale(seed=2, sphere_seed=3, scale=0.125, flow_amp=0.03, nu=0.004)
+    b1 = synth._empty_block((14, 13, 12), origin=(3.0, 4.0, 4.0), h=h)
+    b1.u0, b1.rho0, b1.c0 = synth.smooth_field(b1, 11, amp=0.03, wavelength=8.0)
+    sc.blocks = [sc.blocks[0], b1]
+    target = np.zeros(sc.blocks[0].shape_zyx)
+    dom = gpu_multiscale(sc)
+    dom.set_tape(2)
+    dom.step(2)
+    c = dom.read_field(lbm.LBM_FIELD_SCALAR, lbm.LBM_F64)
+    dc = torch.tensor(c, dtype=torch.float32, device="cuda")
+    grads = [torch.empty(3 * b.flags.size, dtype=torch.float32, device="cuda") for b in sc.blocks]
+    torch.cuda.synchronize()
+    dom.adjoint_step(2, dc, grads[0])
+    dom.adjoint_block_grad(1, grads[1])
+    dom.sync()
+    dom.close()
+    _, go, _ = oadj.ms_loss_and_grad(sc, 2, target)
+    for b, g, o in zip(sc.blocks, grads, go):
+        assert rel(g.cpu().numpy().astype(np.float64).reshape(b.u0.shape), o.numpy()) <= 1e-4
