@@ -39,7 +39,7 @@ static void launch_step2_b(const BlockView& v, dim3 grid, dim3 block, cudaStream
   else k_step2<T, IT, MINB, false, LINEAR><<<grid, block, 0, s>>>(v);
 }
 
-// linear one-row CTAs run at the bound pick_tiles takes for the storage
+// linear one-row CTAs run at the bound pick_tiles takes for them
 template <typename T, typename IT>
 static void launch_step2_t(const BlockView& v, dim3 grid, dim3 block, int b, cudaStream_t s) {
   if (tile_linear(v.nx / 2, (int)block.x, (int)block.y))
@@ -84,7 +84,7 @@ static void launch_step_b(const BlockView& v, dim3 grid, dim3 block, cudaStream_
 
 template <typename T, typename IT, bool ALIGN>
 static void launch_step_t(const BlockView& v, dim3 grid, dim3 block, int minb, cudaStream_t s) {
-  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_b<T, IT, ALIGN, 4, true>(v, grid, block, s);
+  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_b<T, IT, ALIGN, 3, true>(v, grid, block, s);
   else if (step_scalar_bound(minb) >= 4) launch_step_b<T, IT, ALIGN, 4, false>(v, grid, block, s);
   else launch_step_b<T, IT, ALIGN, 3, false>(v, grid, block, s);
 }

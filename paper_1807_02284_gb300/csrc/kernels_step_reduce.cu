@@ -130,26 +130,25 @@ static void launch_step_reduce_b(const BlockView& v, dim3 grid, dim3 block, floa
 template <typename T>
 static void launch_step_reduce_t(const BlockView& v, dim3 grid, dim3 block, int minb,
                                  float* records, cudaStream_t s) {
-  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_reduce_b<T, 4, true>(v, grid, block, records, s);
+  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_reduce_b<T, 3, true>(v, grid, block, records, s);
   else if (step_scalar_bound(minb) >= 4) launch_step_reduce_b<T, 4, false>(v, grid, block, records, s);
   else launch_step_reduce_b<T, 3, false>(v, grid, block, records, s);
 }
 
-template <typename T, int MINB, bool LINEAR>
+// 128 registers (4 CTAs per SM) for both storages: 256^3 FP16 652 us per fused step against 665
+// at 96, where the step alone is the faster one.
+template <typename T, bool LINEAR>
 static void launch_step2_reduce_b(const BlockView& v, dim3 grid, dim3 block, float* records,
                                   cudaStream_t s) {
-  if (v.walls) k_step2_reduce<T, MINB, true, LINEAR><<<grid, block, 0, s>>>(v, records);
-  else k_step2_reduce<T, MINB, false, LINEAR><<<grid, block, 0, s>>>(v, records);
+  if (v.walls) k_step2_reduce<T, 4, true, LINEAR><<<grid, block, 0, s>>>(v, records);
+  else k_step2_reduce<T, 4, false, LINEAR><<<grid, block, 0, s>>>(v, records);
 }
 
 template <typename T>
-static void launch_step2_reduce_t(const BlockView& v, dim3 grid, dim3 block, int b,
-                                  float* records, cudaStream_t s) {
-  if (tile_linear(v.nx / 2, (int)block.x, (int)block.y))
-    launch_step2_reduce_b<T, sizeof(T) == 2 ? 5 : 4, true>(v, grid, block, records, s);
-  else if (b >= 6) launch_step2_reduce_b<T, 6, false>(v, grid, block, records, s);
-  else if (b == 5) launch_step2_reduce_b<T, 5, false>(v, grid, block, records, s);
-  else launch_step2_reduce_b<T, 4, false>(v, grid, block, records, s);
+static void launch_step2_reduce_t(const BlockView& v, dim3 grid, dim3 block, float* records,
+                                  cudaStream_t s) {
+  if (tile_linear(v.nx / 2, (int)block.x, (int)block.y)) launch_step2_reduce_b<T, true>(v, grid, block, records, s);
+  else launch_step2_reduce_b<T, false>(v, grid, block, records, s);
 }
 
 // 32-bit indexing only (27 N < 2^32): the caller checks fits_32bit_index.  A two-node bound
@@ -161,8 +160,8 @@ cudaError_t launch_step_records(const BlockView& v, int storage, int bx, int by,
       ((bx / 2) * by) % 32 == 0) {
     dim3 block(bx / 2, by, 1);
     const dim3 grid = tile_grid(v.nx / 2, v.ny, (unsigned)v.nz, bx / 2, by);
-    if (storage == ST_FP16) launch_step2_reduce_t<__half>(v, grid, block, minb - STEP_PAIR, records, s);
-    else launch_step2_reduce_t<float>(v, grid, block, minb - STEP_PAIR, records, s);
+    if (storage == ST_FP16) launch_step2_reduce_t<__half>(v, grid, block, records, s);
+    else launch_step2_reduce_t<float>(v, grid, block, records, s);
     return cudaGetLastError();
   }
   dim3 block(bx, by, 1);

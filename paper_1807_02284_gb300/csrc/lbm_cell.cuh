@@ -317,8 +317,19 @@ __device__ __forceinline__ void cell_update(const BlockView& v, int x, int y, in
   const bool inner = inner_yz(v, y, z);
   const Nbr<IT> n = inner ? neighbours_inner<IT>(v, x, y, z) : neighbours<IT>(v, x, y, z);
   const IT idx = n.p0 + n.r0 + n.x0;
+  // every load that the node's index alone decides is issued before the flags are looked at:
+  // the pull, the lagged velocity neighbourhood (unused by the few nodes that take no update);
+  // waiting for the flag byte first put one more trip to DRAM into every warp's life
   const uint8_t fl = __ldg(v.flags + idx);
   float d[27];
+  const IT nxI = (IT)v.nx, nxyI = (IT)v.nx * (IT)v.ny;
+  const IT row = n.p0 + n.r0;
+  if (inner) pull_inner<T, IT>(d, din, N, nxI, nxyI, row + n.xm, idx, row + n.xp);
+  else pull_all<T, IT>(d, din, N, n);
+  float g_lag = 0.0f;
+  if (v.rp.adaptive && !v.rp.local)
+    g_lag = inner ? grad_norm_inner<IT>(v.u_in, N, nxI, nxyI, idx, row + n.xm, row + n.xp)
+                  : grad_norm<IT>(v.u_in, N, n);
 
   if (fl & (F_SOLID | F_INFLOW | F_GHOST)) {
     float ux = 0.f, uy = 0.f, uz = 0.f, cval = 0.f;
@@ -341,22 +352,12 @@ __device__ __forceinline__ void cell_update(const BlockView& v, int x, int y, in
     return;
   }
 
-  // all independent loads first: the pull and the lagged velocity neighbourhood
-  const IT nxI = (IT)v.nx, nxyI = (IT)v.nx * (IT)v.ny;
-  const IT row = n.p0 + n.r0;
-  if (inner) pull_inner<T, IT>(d, din, N, nxI, nxyI, row + n.xm, idx, row + n.xp);
-  else pull_all<T, IT>(d, din, N, n);
   // an obstacle wall node completes what comes from inside the obstacle itself
   if ((fl & F_NEAR_SOLID) && !(WALLS && (fl & F_OBST_WALL)))
     bounce_back<T, IT>(d, din, N, v.flags, n, idx);
   if constexpr (WALLS) {
     if (fl & (F_WALL | F_OBST_WALL)) wall_regularize<IT>(d, v, x, y, z, fl, n);
   }
-  float g_lag = 0.0f;
-  if (v.rp.adaptive && !v.rp.local)
-    g_lag = inner ? grad_norm_inner<IT>(v.u_in, N, nxI, nxyI, idx, row + n.xm, row + n.xp)
-                  : grad_norm<IT>(v.u_in, N, n);
-
   raw_moments(d);
   const float drho = d[kap(0, 0, 0)];
   const float inv = fast_rcp(__fadd_rn(1.0f, drho));
@@ -523,19 +524,24 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
   const unsigned fl2 = __ldg(reinterpret_cast<const unsigned short*>(v.flags + a0));
   const uint8_t fl0 = (uint8_t)(fl2 & 0xffu), fl1 = (uint8_t)(fl2 >> 8);
   constexpr uint8_t kNodeWise = F_SOLID | F_INFLOW | F_GHOST | F_NEAR_SOLID | F_WALL | F_OBST_WALL;
-  if (!inner_yz(v, y, z) || ((fl0 | fl1) & kNodeWise)) {
+  const T* __restrict__ din = static_cast<const T*>(v.d_in);
+  T* __restrict__ dout = static_cast<T*>(v.d_out);
+  // the loads of the pair path go out before the flags are looked at (256^3 FP32 658 -> 629 us,
+  // 128^3 88 -> 84; FP16, bound by issue as much as by latency, 591 -> 588)
+  const bool inner = inner_yz(v, y, z);
+  float2 d[27];
+  float2 g_lag = make_float2(0.0f, 0.0f);
+  if (inner) {
+    const IT am0 = row + (IT)nbr(x, -1, v.nx, v.per[0]);
+    const IT ap1 = row + (IT)nbr(x + 1, 1, v.nx, v.per[0]);
+    pull_pair<T, IT>(d, din, N, nxI, nxyI, am0, a0, ap1);
+    if (v.rp.adaptive && !v.rp.local) g_lag = grad_norm_pair<IT>(v.u_in, N, nxI, nxyI, a0, am0, ap1);
+  }
+  if (!inner || ((fl0 | fl1) & kNodeWise)) {
     cell_update<T, IT, false, WALLS, RED>(v, x, y, z, nm);
     cell_update<T, IT, false, WALLS, RED>(v, x + 1, y, z, nm);
     return;
   }
-  const T* __restrict__ din = static_cast<const T*>(v.d_in);
-  T* __restrict__ dout = static_cast<T*>(v.d_out);
-  const IT am0 = row + (IT)nbr(x, -1, v.nx, v.per[0]);
-  const IT ap1 = row + (IT)nbr(x + 1, 1, v.nx, v.per[0]);
-  float2 d[27];
-  pull_pair<T, IT>(d, din, N, nxI, nxyI, am0, a0, ap1);
-  float2 g_lag = make_float2(0.0f, 0.0f);
-  if (v.rp.adaptive && !v.rp.local) g_lag = grad_norm_pair<IT>(v.u_in, N, nxI, nxyI, a0, am0, ap1);
 
   raw_moments(d);
   const float2 drho = d[kap(0, 0, 0)];
