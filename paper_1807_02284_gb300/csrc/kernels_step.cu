@@ -11,7 +11,7 @@ __global__ void __launch_bounds__(256, MINB) k_step(BlockView v) {
   int x, y;
   if (!thread_column<LINEAR>(v.nx, v.ny, x, y)) return;
   const int z = blockIdx.z + v.z_first;
-  cell_update<T, IT, ALIGN, WALLS>(v, x, y, z);
+  cell_update<T, IT, ALIGN, WALLS, false, MINB == 3>(v, x, y, z);
 }
 
 // Two nodes (x, x + 1) per thread, x = 2 (thread's column): MINB CTAs of at most 128 threads
@@ -84,7 +84,7 @@ static void launch_step_b(const BlockView& v, dim3 grid, dim3 block, cudaStream_
 
 template <typename T, typename IT, bool ALIGN>
 static void launch_step_t(const BlockView& v, dim3 grid, dim3 block, int minb, cudaStream_t s) {
-  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_b<T, IT, ALIGN, 3, true>(v, grid, block, s);
+  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_b<T, IT, ALIGN, 4, true>(v, grid, block, s);
   else if (step_scalar_bound(minb) >= 4) launch_step_b<T, IT, ALIGN, 4, false>(v, grid, block, s);
   else launch_step_b<T, IT, ALIGN, 3, false>(v, grid, block, s);
 }

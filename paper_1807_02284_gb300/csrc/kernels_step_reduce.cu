@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256, MINB) k_step_reduce(BlockView v, float* r
   if (t == 0) done = 0u;
   __syncthreads();                          // the counter is set before any warp counts
   const NodeMomentsOut out{&snm[0][t], 256};
-  if (in) cell_update<T, uint32_t, false, WALLS, true>(v, x, y, z, &out);
+  if (in) cell_update<T, uint32_t, false, WALLS, true, MINB == 3>(v, x, y, z, &out);
   __syncwarp();
   float val[6];
 #pragma unroll
@@ -130,7 +130,7 @@ static void launch_step_reduce_b(const BlockView& v, dim3 grid, dim3 block, floa
 template <typename T>
 static void launch_step_reduce_t(const BlockView& v, dim3 grid, dim3 block, int minb,
                                  float* records, cudaStream_t s) {
-  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_reduce_b<T, 3, true>(v, grid, block, records, s);
+  if (tile_linear(v.nx, (int)block.x, (int)block.y)) launch_step_reduce_b<T, 4, true>(v, grid, block, records, s);
   else if (step_scalar_bound(minb) >= 4) launch_step_reduce_b<T, 4, false>(v, grid, block, records, s);
   else launch_step_reduce_b<T, 3, false>(v, grid, block, records, s);
 }

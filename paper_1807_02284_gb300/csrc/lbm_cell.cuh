@@ -308,7 +308,14 @@ struct NodeMomentsOut {
 // obstacle voxels and ghost nodes write nothing).  Collision conserves rho and j, so a fluid
 // node's are those of its pulled set, written as soon as they are known, so that nothing
 // is held through the collision.
-template <typename T, typename IT, bool ALIGN = false, bool WALLS = false, bool RED = false>
+// EARLY: the loads that the node's index alone decides (the pull, the lagged velocity
+// neighbourhood) are issued before the flags are looked at, which would put one more trip to
+// DRAM into the warp's life; it takes 80 registers, which pays on the smallest blocks (32^3 3.5
+// us per step against 3.8).  Elsewhere 64 registers and more warps are the better choice (64^3
+// 11.3 us against 11.6, 201 x 181 x 171 FP16 261 against 282, 64 uneven plumes 23.0 against
+// 23.8 ms a pass).
+template <typename T, typename IT, bool ALIGN = false, bool WALLS = false, bool RED = false,
+          bool EARLY = false>
 __device__ __forceinline__ void cell_update(const BlockView& v, int x, int y, int z,
                                             const NodeMomentsOut* nm = nullptr) {
   const IT N = (IT)v.N;
@@ -317,19 +324,23 @@ __device__ __forceinline__ void cell_update(const BlockView& v, int x, int y, in
   const bool inner = inner_yz(v, y, z);
   const Nbr<IT> n = inner ? neighbours_inner<IT>(v, x, y, z) : neighbours<IT>(v, x, y, z);
   const IT idx = n.p0 + n.r0 + n.x0;
-  // every load that the node's index alone decides is issued before the flags are looked at:
-  // the pull, the lagged velocity neighbourhood (unused by the few nodes that take no update);
-  // waiting for the flag byte first put one more trip to DRAM into every warp's life
   const uint8_t fl = __ldg(v.flags + idx);
-  float d[27];
+  float d[27], g_lag = 0.0f;
   const IT nxI = (IT)v.nx, nxyI = (IT)v.nx * (IT)v.ny;
   const IT row = n.p0 + n.r0;
-  if (inner) pull_inner<T, IT>(d, din, N, nxI, nxyI, row + n.xm, idx, row + n.xp);
-  else pull_all<T, IT>(d, din, N, n);
-  float g_lag = 0.0f;
-  if (v.rp.adaptive && !v.rp.local)
-    g_lag = inner ? grad_norm_inner<IT>(v.u_in, N, nxI, nxyI, idx, row + n.xm, row + n.xp)
-                  : grad_norm<IT>(v.u_in, N, n);
+  auto pull = [&]() {
+    if (inner) pull_inner<T, IT>(d, din, N, nxI, nxyI, row + n.xm, idx, row + n.xp);
+    else pull_all<T, IT>(d, din, N, n);
+  };
+  auto gradient = [&]() {
+    if (v.rp.adaptive && !v.rp.local)
+      g_lag = inner ? grad_norm_inner<IT>(v.u_in, N, nxI, nxyI, idx, row + n.xm, row + n.xp)
+                    : grad_norm<IT>(v.u_in, N, n);
+  };
+  if constexpr (EARLY) {
+    pull();
+    gradient();
+  }
 
   if (fl & (F_SOLID | F_INFLOW | F_GHOST)) {
     float ux = 0.f, uy = 0.f, uz = 0.f, cval = 0.f;
@@ -352,12 +363,14 @@ __device__ __forceinline__ void cell_update(const BlockView& v, int x, int y, in
     return;
   }
 
+  if constexpr (!EARLY) pull();
   // an obstacle wall node completes what comes from inside the obstacle itself
   if ((fl & F_NEAR_SOLID) && !(WALLS && (fl & F_OBST_WALL)))
     bounce_back<T, IT>(d, din, N, v.flags, n, idx);
   if constexpr (WALLS) {
     if (fl & (F_WALL | F_OBST_WALL)) wall_regularize<IT>(d, v, x, y, z, fl, n);
   }
+  if constexpr (!EARLY) gradient();
   raw_moments(d);
   const float drho = d[kap(0, 0, 0)];
   const float inv = fast_rcp(__fadd_rn(1.0f, drho));

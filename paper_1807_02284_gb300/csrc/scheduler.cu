@@ -49,32 +49,33 @@ static std::vector<int> next_levels(const std::vector<lbm::Block>& blocks, std::
 // step of fluid blocks on GB300, every shape and register bound tried at each size.
 void lbm_domain::pick_tiles(int b) {
   Block& B = blocks[b];
-  const bool half = desc.storage == LBM_FP16_SHIFTED, small = B.N <= (size_t)1 << 18;
-  if (B.nx % 2 == 0 && B.N >= (half ? (size_t)3 << 18 : (size_t)1 << 20)) {
+  const bool half = desc.storage == LBM_FP16_SHIFTED;
+  if (B.nx % 2 == 0 && B.N >= (size_t)1 << 20) {
     // two nodes per thread once the block is bound by bandwidth or issue rather than by
-    // latency: FP32 from 1 M nodes (80^3 26.8 against 26.3 us with one node per thread, 96^3 42.4
-    // against 41.6, 128^3 84 against 91, 256^3 629 against 820), FP16 from 0.8 M (80^3 24.6
-    // against 22.5, 96^3 41.1 against 41.9, 128^3 80 against 96, 256^3 592 against 790).  Tiles
-    // of 64 x 2 nodes on whole rows, one-row CTAs running on over ragged ones (224 x 250 x 190
-    // FP32 410 us against 431 with 64 x 2 tiles, FP16 386 against 428).
+    // latency: from 1 M nodes (96^3 FP32 42.5 against 40.8 us with one node per thread, FP16 41.2
+    // against 40.0; 128^3 84 against 91, FP16 80 against 96; 256^3 629 against 702, FP16 592
+    // against 718).  Tiles of 64 x 2 nodes on whole rows, one-row CTAs running on over ragged
+    // ones (224 x 250 x 190 FP32 410 us against 431 with 64 x 2 tiles, FP16 386 against 428).
     const bool tiles = B.nx % 64 == 0;
     B.bx = tiles ? 64 : 128;
     B.by = tiles ? 2 : 1;
     B.minb = STEP_PAIR + (half ? 5 : 4);
-  } else if (B.nx % 32 == 0 || B.nx < 32) {
-    // a warp per row; 80 registers hold the loads that go out before the flags are known (96^3
-    // 41.6 us, at 64 registers 46), 64 registers where the block is one or two waves of CTAs
-    // (64^3 11.7 us against 11.8); rows below a warp keep their faces in warps of their own
-    // (24^3 2.9 us against 4.0 with one-row CTAs, where most warps hold a face node)
+  } else if (B.nx <= 32) {
+    // latency-bound: a warp per row keeps the faces in warps of their own, 80 registers take
+    // cell_update's EARLY loads (24^3 2.9 us against 4.0 with one-row CTAs, 32^3 3.5 against 3.8)
     B.bx = 32;
     B.by = 4;
-    B.minb = small && B.nx > 32 ? 4 : 3;
+    B.minb = 3;
+  } else if (B.nx % 32 == 0) {
+    B.bx = 32;                           // 64^3 11.3 us, 96^3 40.8 (with EARLY loads 11.6, 41.5)
+    B.by = 4;
+    B.minb = 4;
   } else {
     // ragged rows: no idle lanes (72 x 60 x 51 10.7 us against 12.5 with the best tile,
-    // 97 x 61 x 75 21.7 against 25.8, 201 x 181 x 171 283 against 299)
-    B.bx = small ? 64 : 128;
+    // 97 x 61 x 75 21.7 against 25.8, 201 x 181 x 171 281 against 299)
+    B.bx = 128;
     B.by = 1;
-    B.minb = 3;
+    B.minb = 4;
   }
   if (const char* env = std::getenv("LBM_TILE")) {  // "bx,by[,minb]" forces a launch shape
     int bx = 0, by = 0, mb = 3;
