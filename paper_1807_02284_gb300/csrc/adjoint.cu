@@ -1086,9 +1086,9 @@ struct TapeState {
 using namespace lbm;
 
 static void free_level(lbm_domain* dom, Level& L) {
-  dom->dev_free(L.f);
-  dom->dev_free(L.u);
-  dom->dev_free(L.c);
+  dom->tape_free(L.f);
+  dom->tape_free(L.u);
+  dom->tape_free(L.c);
   L = Level();
 }
 
@@ -1098,31 +1098,31 @@ void release_tape(lbm_domain* dom) {
   for (Level& L : t->ckpt) free_level(dom, L);
   for (Level& L : t->seg) free_level(dom, L);
   for (int i = 0; i < 2; ++i) {
-    dom->dev_free(t->lam[i]);
-    dom->dev_free(t->ups[i]);
-    dom->dev_free(t->gam[i]);
+    dom->tape_free(t->lam[i]);
+    dom->tape_free(t->ups[i]);
+    dom->tape_free(t->gam[i]);
   }
-  dom->dev_free(t->ms);
-  dom->dev_free(t->side);
+  dom->tape_free(t->ms);
+  dom->tape_free(t->side);
   for (auto& v : t->mck) for (Level& L : v) free_level(dom, L);
   for (auto& v : t->snap) for (Level& L : v) free_level(dom, L);
   for (auto& v : t->ver) for (Level& L : v) free_level(dom, L);
   for (Level& L : t->spare) free_level(dom, L);
   for (auto& v : t->lamb)
     for (AdjLevel& A : v) {
-      dom->dev_free(A.f);
-      dom->dev_free(A.u);
-      dom->dev_free(A.c);
+      dom->tape_free(A.f);
+      dom->tape_free(A.u);
+      dom->tape_free(A.c);
     }
-  for (float* g : t->grad) dom->dev_free(g);
+  for (float* g : t->grad) dom->tape_free(g);
   delete t;
   dom->tape = nullptr;
 }
 
 static bool alloc_level(lbm_domain* dom, size_t N, Level& L) {
-  L.f = dom->dev_alloc(N * 27 * sizeof(float));
-  L.u = static_cast<float*>(dom->dev_alloc(N * 3 * sizeof(float)));
-  L.c = static_cast<float*>(dom->dev_alloc(N * sizeof(float)));
+  L.f = dom->tape_alloc(N * 27 * sizeof(float));
+  L.u = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
+  L.c = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
   return L.f && L.u && L.c;
 }
 
@@ -1216,7 +1216,10 @@ extern "C" lbm_status lbm_set_tape(lbm_domain* dom, int32_t every) {
   cudaSetDevice(dom->desc.device);
   if (every < 0) return dom->fail(LBM_ERR_INVALID_ARG, "checkpoint_every must be >= 0");
   release_tape(dom);
-  if (every == 0) return LBM_OK;
+  if (every == 0) {
+    dom->drop_tape_pool();
+    return LBM_OK;
+  }
   if (dom->steps != 0)
     return dom->fail(LBM_ERR_STATE, "the tape must be enabled right after lbm_init_macro");
   lbm_status st = adjoint_supported(dom);
@@ -1478,9 +1481,9 @@ static cudaError_t ms_reverse_op(const MsStep& m, const MsOp& o, cudaStream_t s)
 }
 
 static bool alloc_adj(lbm_domain* dom, size_t N, AdjLevel& A) {
-  A.f = static_cast<float*>(dom->dev_alloc(N * 27 * sizeof(float)));
-  A.u = static_cast<float*>(dom->dev_alloc(N * 3 * sizeof(float)));
-  A.c = static_cast<float*>(dom->dev_alloc(N * sizeof(float)));
+  A.f = static_cast<float*>(dom->tape_alloc(N * 27 * sizeof(float)));
+  A.u = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
+  A.c = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
   return A.f && A.u && A.c;
 }
 
@@ -1531,13 +1534,13 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
       t->lamb[b].resize(levels);
       for (AdjLevel& A : t->lamb[b])
         if (!alloc_adj(dom, N, A)) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-      t->grad[b] = static_cast<float*>(dom->dev_alloc(N * 3 * sizeof(float)));
+      t->grad[b] = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
       if (!t->grad[b]) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
     }
-    t->ms = static_cast<float*>(dom->dev_alloc(nmax * sizeof(float)));
+    t->ms = static_cast<float*>(dom->tape_alloc(nmax * sizeof(float)));
     size_t side = 0;
     for (const Block& B : dom->blocks) side = std::max(side, face_side_floats(B.nx, B.ny, B.nz));
-    t->side = static_cast<float*>(dom->dev_alloc(side * sizeof(float)));
+    t->side = static_cast<float*>(dom->tape_alloc(side * sizeof(float)));
     if (!t->ms || !t->side) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
     cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
     if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");
@@ -1645,16 +1648,16 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
   cudaStream_t s = dom->stream;
   // buffers
   for (int i = 0; i < 2; ++i) {
-    if (!t->lam[i]) t->lam[i] = static_cast<float*>(dom->dev_alloc(N * 27 * sizeof(float)));
-    if (!t->ups[i]) t->ups[i] = static_cast<float*>(dom->dev_alloc(N * 3 * sizeof(float)));
-    if (!t->gam[i]) t->gam[i] = static_cast<float*>(dom->dev_alloc(N * sizeof(float)));
+    if (!t->lam[i]) t->lam[i] = static_cast<float*>(dom->tape_alloc(N * 27 * sizeof(float)));
+    if (!t->ups[i]) t->ups[i] = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
+    if (!t->gam[i]) t->gam[i] = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
     if (!t->lam[i] || !t->ups[i] || !t->gam[i]) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
   }
-  if (!t->ms) t->ms = static_cast<float*>(dom->dev_alloc(N * sizeof(float)));
+  if (!t->ms) t->ms = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
   if (!t->ms) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
   if (!t->side) {
     const size_t side = face_side_floats(B.nx, B.ny, B.nz);
-    t->side = static_cast<float*>(dom->dev_alloc(side * sizeof(float)));
+    t->side = static_cast<float*>(dom->tape_alloc(side * sizeof(float)));
     if (!t->side) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
     cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
     if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");

@@ -56,3 +56,44 @@ def test_adjoint_of_blocks_with_more_than_two_levels_of_substeps(lib, h):
     _, go, _ = oadj.ms_loss_and_grad(sc, 2, target)
     for b, g, o in zip(sc.blocks, grads, go):
         assert rel(g.cpu().numpy().astype(np.float64).reshape(b.u0.shape), o.numpy()) <= 1e-4
+
+
+def test_tape_buffers_are_reused_and_given_back(lib):
+    """A second rollout takes the first one's tape buffers (no allocation), gives the same
+    gradient, and the first step without a tape, or lbm_set_tape(0), gives them back."""
+    import torch
+
+    from paper_1807_02284_gb300 import lbm
+    from tests.helpers import f32
+    sc, _ = synth.adjoint_scene(n=14, seed=5, nu=0.01)
+    b = sc.blocks[0]
+    d = lbm.Domain(b.dims, sc.nu, periodic=sc.periodic)
+    dc = torch.rand(b.flags.size, device="cuda")
+    grads = [torch.empty(3 * b.flags.size, device="cuda") for _ in range(3)]
+    torch.cuda.synchronize()
+
+    def rollout(g):
+        d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0))
+        d.set_tape(2)
+        d.step(5)
+        d.adjoint_step(5, dc, g)
+        d.sync()
+
+    held = torch.cuda.memory_allocated
+    d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0))
+    d.step(1)
+    d.sync()
+    bare = held()
+    rollout(grads[0])
+    with_tape = held()
+    assert with_tape > bare
+    rollout(grads[1])
+    assert held() == with_tape
+    d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0))
+    d.step(1)
+    assert held() == bare
+    rollout(grads[2])
+    d.set_tape(0)
+    assert held() == bare
+    assert torch.equal(grads[0], grads[1]) and torch.equal(grads[0], grads[2])
+    d.close()
