@@ -141,9 +141,11 @@ cudaError_t launch_step_align(const BlockView& v, int bx, int by, cudaStream_t s
 }
 
 // f_0 = f^eq(rho_0, u_0) (Algorithm 1 initialisation); obstacle voxels hold the rest state.
+// Also clears the device error word.
 template <typename T>
 __global__ void k_init(BlockView v, const float* rho, const float* u, const float* c) {
   const size_t N = v.N;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *v.err = 0;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < N;
        idx += (size_t)gridDim.x * blockDim.x) {
     T* dout = static_cast<T*>(v.d_out);
@@ -412,11 +414,19 @@ __device__ __forceinline__ void write_planes(const I (&f)[27], size_t N, size_t 
   }
 }
 
+// The error word on its way to the host: a read's kernel stores it into pinned memory itself,
+// in place of a 4-byte copy behind every read (an operation of its own costs the host about 4
+// us; visible once the stream has passed the kernel).
+__device__ __forceinline__ void report_error(const int* err, int* host_err) {
+  if (host_err && blockIdx.x == 0 && threadIdx.x == 0) *host_err = *err;
+}
+
 // HBM-bound copies (216 B per node between FP32 arrays): every load of a node before its
 // first store, one node per thread and trip.
 template <typename T, typename O>
 __global__ void __launch_bounds__(256) k_read_f(const T* __restrict__ d, size_t N,
-                                                O* __restrict__ out) {
+                                                O* __restrict__ out, const int* err, int* host_err) {
+  report_error(err, host_err);
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < N;
        idx += (size_t)gridDim.x * blockDim.x) {
     float v[27];
@@ -444,14 +454,14 @@ static int grid_for(size_t n) {
 }
 
 cudaError_t launch_read_f(const void* d, int storage, size_t N, void* out, int out_f64,
-                          cudaStream_t s) {
+                          cudaStream_t s, const int* err, int* host_err) {
   const int g = grid_for(N);
   if (storage == ST_FP16) {
-    if (out_f64) k_read_f<__half, double><<<g, 256, 0, s>>>((const __half*)d, N, (double*)out);
-    else k_read_f<__half, float><<<g, 256, 0, s>>>((const __half*)d, N, (float*)out);
+    if (out_f64) k_read_f<__half, double><<<g, 256, 0, s>>>((const __half*)d, N, (double*)out, err, host_err);
+    else k_read_f<__half, float><<<g, 256, 0, s>>>((const __half*)d, N, (float*)out, err, host_err);
   } else {
-    if (out_f64) k_read_f<float, double><<<g, 256, 0, s>>>((const float*)d, N, (double*)out);
-    else k_read_f<float, float><<<g, 256, 0, s>>>((const float*)d, N, (float*)out);
+    if (out_f64) k_read_f<float, double><<<g, 256, 0, s>>>((const float*)d, N, (double*)out, err, host_err);
+    else k_read_f<float, float><<<g, 256, 0, s>>>((const float*)d, N, (float*)out, err, host_err);
   }
   return cudaGetLastError();
 }
@@ -488,7 +498,8 @@ cudaError_t launch_read_rho(const void* d, int storage, size_t N, float* out, cu
 }
 
 template <typename I, typename O>
-__global__ void k_convert(const I* in, O* out, size_t n) {
+__global__ void k_convert(const I* in, O* out, size_t n, const int* err, int* host_err) {
+  report_error(err, host_err);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x)
     out[i] = (O)in[i];
@@ -497,7 +508,9 @@ __global__ void k_convert(const I* in, O* out, size_t n) {
 // FP32 to FP32 (the device read and write of velocity and scalar): 16 bytes per thread and
 // trip, taken when both arrays are 16-byte aligned; the last n % 4 values by one thread.
 __global__ void __launch_bounds__(256) k_copy4(const float* __restrict__ in,
-                                               float* __restrict__ out, size_t n) {
+                                               float* __restrict__ out, size_t n, const int* err,
+                                               int* host_err) {
+  report_error(err, host_err);
   const size_t n4 = n / 4;
   const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   for (size_t i = i0; i < n4; i += (size_t)gridDim.x * blockDim.x)
@@ -507,16 +520,16 @@ __global__ void __launch_bounds__(256) k_copy4(const float* __restrict__ in,
 }
 
 cudaError_t launch_convert(const void* in, int in_f64, void* out, int out_f64, size_t n,
-                           cudaStream_t s) {
+                           cudaStream_t s, const int* err, int* host_err) {
   const int g = grid_for(n);
   if (!in_f64 && !out_f64 && aligned_to(in, 16) && aligned_to(out, 16)) {
-    k_copy4<<<grid_for((n + 3) / 4), 256, 0, s>>>((const float*)in, (float*)out, n);
+    k_copy4<<<grid_for((n + 3) / 4), 256, 0, s>>>((const float*)in, (float*)out, n, err, host_err);
     return cudaGetLastError();
   }
-  if (in_f64 && out_f64) k_convert<double, double><<<g, 256, 0, s>>>((const double*)in, (double*)out, n);
-  else if (in_f64) k_convert<double, float><<<g, 256, 0, s>>>((const double*)in, (float*)out, n);
-  else if (out_f64) k_convert<float, double><<<g, 256, 0, s>>>((const float*)in, (double*)out, n);
-  else k_convert<float, float><<<g, 256, 0, s>>>((const float*)in, (float*)out, n);
+  if (in_f64 && out_f64) k_convert<double, double><<<g, 256, 0, s>>>((const double*)in, (double*)out, n, err, host_err);
+  else if (in_f64) k_convert<double, float><<<g, 256, 0, s>>>((const double*)in, (float*)out, n, err, host_err);
+  else if (out_f64) k_convert<float, double><<<g, 256, 0, s>>>((const float*)in, (double*)out, n, err, host_err);
+  else k_convert<float, float><<<g, 256, 0, s>>>((const float*)in, (float*)out, n, err, host_err);
   return cudaGetLastError();
 }
 

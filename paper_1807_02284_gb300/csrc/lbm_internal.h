@@ -127,13 +127,14 @@ cudaError_t launch_inflow_records(const void* rec, int n, uint8_t* flags, float*
                                   int n_levels, int nx, int ny, int nz, size_t N, int* err,
                                   cudaStream_t s);
 // fields: 0 = populations f (27 planes, paper order), 1 = u, 2 = scalar, 3 = rho
+// (host_err, where given: pinned host memory that the kernel stores the error word into)
 cudaError_t launch_read_f(const void* d, int storage, size_t N, void* out, int out_f64,
-                          cudaStream_t s);
+                          cudaStream_t s, const int* err = nullptr, int* host_err = nullptr);
 cudaError_t launch_write_f(void* d, int storage, size_t N, const void* in, int in_f64,
                            cudaStream_t s);
 cudaError_t launch_read_rho(const void* d, int storage, size_t N, float* out, cudaStream_t s);
 cudaError_t launch_convert(const void* in, int in_f64, void* out, int out_f64, size_t n,
-                           cudaStream_t s);
+                           cudaStream_t s, const int* err = nullptr, int* host_err = nullptr);
 // deterministic reduction of mass, momentum and kinetic energy over non-solid, non-ghost
 // nodes (per-thread compensated FP32 sums of per-node FP32 values, combined in FP64 in a
 // fixed order):

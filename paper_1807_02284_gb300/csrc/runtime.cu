@@ -402,7 +402,7 @@ lbm_status lbm_set_boundary(lbm_domain* dom, int32_t block_id, int32_t kind, con
     const int n = (int)(nbytes / sizeof(lbm_inflow_record));
     if (n == 0) return LBM_OK;
     if (!ptr) return dom->fail(LBM_ERR_INVALID_ARG, "null records");
-    const void* src = on_device ? ptr : dom->upload_small(ptr, nbytes, &st);
+    const void* src = on_device ? ptr : dom->stage_small(ptr, nbytes, &st);
     if (st != LBM_OK) return st;
     std::vector<float*> lv;
     for (auto& L : B.lv) lv.push_back(L.u);
@@ -410,7 +410,7 @@ lbm_status lbm_set_boundary(lbm_domain* dom, int32_t block_id, int32_t kind, con
     cudaError_t e = launch_inflow_records(src, n, B.flags, lv.data(), (int)lv.size(), B.nx,
                                           B.ny, B.nz, B.N, dom->d_err, dom->stream);
     if (e != cudaSuccess) return dom->cuda_fail(e, "inflow records");
-    return LBM_OK;
+    return on_device ? LBM_OK : dom->small_used();
   }
   return dom->fail(LBM_ERR_INVALID_ARG, "unknown boundary kind");
 }
@@ -451,7 +451,8 @@ lbm_status lbm_init_macro(lbm_domain* dom, int32_t block_id, const float* rho, c
     if (e != cudaSuccess) return dom->cuda_fail(e, "cudaStreamSynchronize");
   }
   dom->on_state_reset(block_id);
-  return dom->reset_error_word();
+  *dom->h_err = 0;                             // (the kernel has cleared the device's)
+  return LBM_OK;
 }
 
 lbm_status lbm_step(lbm_domain* dom, int32_t n) {
@@ -499,24 +500,29 @@ lbm_status lbm_read_field(lbm_domain* dom, int32_t block_id, int32_t field, int3
   cudaError_t e = cudaSuccess;
   const int f64 = dtype == LBM_F64;
   switch (field) {
-    case LBM_FIELD_F: e = launch_read_f(L.f, dom->desc.storage, N, out, f64, dom->stream); break;
-    case LBM_FIELD_U: e = launch_convert(L.u, 0, out, f64, 3 * N, dom->stream); break;
-    case LBM_FIELD_SCALAR: e = launch_convert(L.c, 0, out, f64, N, dom->stream); break;
+    case LBM_FIELD_F: e = launch_read_f(L.f, dom->desc.storage, N, out, f64, dom->stream, dom->d_err, dom->h_err); break;
+    case LBM_FIELD_U: e = launch_convert(L.u, 0, out, f64, 3 * N, dom->stream, dom->d_err, dom->h_err); break;
+    case LBM_FIELD_SCALAR: e = launch_convert(L.c, 0, out, f64, N, dom->stream, dom->d_err, dom->h_err); break;
     case LBM_FIELD_RHO: {
       float* tmp = static_cast<float*>(on_device ? dom->staging(N * 4) : (void*)((char*)out + bytes));
       if (!tmp) return dom->fail(LBM_ERR_OOM, "staging allocation failed");
       e = launch_read_rho(L.f, dom->desc.storage, N, tmp, dom->stream);
-      if (e == cudaSuccess) e = launch_convert(tmp, 0, out, f64, N, dom->stream);
+      if (e == cudaSuccess) e = launch_convert(tmp, 0, out, f64, N, dom->stream, dom->d_err, dom->h_err);
       break;
     }
-    case LBM_FIELD_FLAGS: e = cudaMemcpyAsync(out, B.flags, N, cudaMemcpyDeviceToDevice, dom->stream); break;
+    case LBM_FIELD_FLAGS:
+      e = cudaMemcpyAsync(out, B.flags, N, cudaMemcpyDeviceToDevice, dom->stream);
+      dom->post_error_probe();
+      break;
   }
   if (e != cudaSuccess) return dom->cuda_fail(e, "read field");
   if (!on_device) {
     e = cudaMemcpyAsync(dst, out, bytes, cudaMemcpyDeviceToHost, dom->stream);
     if (e != cudaSuccess) return dom->cuda_fail(e, "device to host copy");
   }
-  return dom->sync_and_check();
+  e = cudaStreamSynchronize(dom->stream);      // the read's kernel has stored the error word
+  if (e != cudaSuccess) return dom->cuda_fail(e, "cudaStreamSynchronize");
+  return dom->error_status();
 }
 
 lbm_status lbm_read_macro(lbm_domain* dom, int32_t block_id, int32_t what, void* dst,

@@ -79,8 +79,7 @@ struct lbm_domain {
   double* h_red = nullptr;              // pinned
   void* staging_buf = nullptr;
   size_t staging_bytes = 0;
-  void* small_host = nullptr;           // pinned bounce buffer for small uploads
-  void* small_dev = nullptr;
+  void* small_host = nullptr;           // pinned buffer of small uploads, read in place
   size_t small_bytes = 0;
   cudaEvent_t small_done = nullptr;
   // lbm_step_reduce_async: one event per ticket slot (ticket t uses slot (t - 1) % 16; a
@@ -134,7 +133,8 @@ struct lbm_domain {
   void drop_tape_pool();
   void* staging(size_t bytes);
   const void* device_source(const void* src, size_t bytes, int on_device, lbm_status* st);
-  const void* upload_small(const void* src, size_t bytes, lbm_status* st);
+  const void* stage_small(const void* src, size_t bytes, lbm_status* st);
+  lbm_status small_used();
   lbm::BlockView view(int b, int from, int to) const;
   lbm_status alloc_block_levels(lbm::Block& B, int levels);
   lbm::RelaxParams relax_params(double nu_block) const;

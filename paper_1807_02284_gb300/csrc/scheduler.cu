@@ -163,40 +163,37 @@ void lbm_domain::release_extras() {
   }
 }
 
-// Small host arrays (inflow records) go through a pinned bounce buffer so the copy is
-// asynchronous and the caller can reuse its array on return.
-const void* lbm_domain::upload_small(const void* src, size_t bytes, lbm_status* st) {
+// Small host arrays (inflow records) go through a pinned buffer that the kernel reads in place
+// (a copy to the device first was one more operation per call, 1.7 us on the GPU and about 4 of
+// host time, for at most some tens of KB), so the caller can reuse its array on return;
+// small_used() after the launch marks when the buffer is free again.
+const void* lbm_domain::stage_small(const void* src, size_t bytes, lbm_status* st) {
   *st = LBM_OK;
+  if (small_done) cudaEventSynchronize(small_done);   // the previous reader has left the buffer
   if (bytes > small_bytes) {
-    if (small_done) cudaEventSynchronize(small_done);
     if (small_host) cudaFreeHost(small_host);
     small_host = nullptr;
-    dev_free(small_dev);
-    small_dev = nullptr;
-    small_bytes = 0;       // no buffer until both allocations below succeed
+    small_bytes = 0;       // no buffer until the allocation below succeeds
     size_t cap = std::max<size_t>(bytes, 4096);
     if (cudaMallocHost(&small_host, cap) != cudaSuccess) {
       small_host = nullptr;
       *st = fail(LBM_ERR_OOM, "pinned allocation failed");
       return nullptr;
     }
-    small_dev = dev_alloc(cap);
-    if (!small_dev) { *st = fail(LBM_ERR_OOM, "device allocation failed"); return nullptr; }
     small_bytes = cap;
   }
-  if (!small_done) {
-    if (cudaEventCreateWithFlags(&small_done, cudaEventDisableTiming) != cudaSuccess) {
-      *st = fail(LBM_ERR_CUDA, "cudaEventCreate");
-      return nullptr;
-    }
-  } else {
-    cudaEventSynchronize(small_done);  // previous upload has left the bounce buffer
+  if (!small_done && cudaEventCreateWithFlags(&small_done, cudaEventDisableTiming) != cudaSuccess) {
+    small_done = nullptr;
+    *st = fail(LBM_ERR_CUDA, "cudaEventCreate");
+    return nullptr;
   }
   std::memcpy(small_host, src, bytes);
-  cudaError_t e = cudaMemcpyAsync(small_dev, small_host, bytes, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaEventRecord(small_done, stream);
-  if (e != cudaSuccess) { *st = cuda_fail(e, "small upload"); return nullptr; }
-  return small_dev;
+  return small_host;
+}
+
+lbm_status lbm_domain::small_used() {
+  const cudaError_t e = cudaEventRecord(small_done, stream);
+  return e == cudaSuccess ? LBM_OK : cuda_fail(e, "cudaEventRecord");
 }
 
 void lbm_domain::on_state_reset(int b) {
