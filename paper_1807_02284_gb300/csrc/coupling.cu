@@ -593,6 +593,7 @@ static lbm_status add_far_block(lbm_domain* dom, const double origin[3], double 
   const cudaError_t e = launch_outer_ghost(CW.flags, CW.nx, CW.ny, CW.nz, 1, dom->stream);
   if (e != cudaSuccess) return abandon(dom->cuda_fail(e, "scale-boundary flags"));
   dom->pick_tiles(id);
+  dom->pick_tiles(0);
   dom->invalidate_graphs();
   *block_id = id;
   return LBM_OK;
@@ -713,6 +714,7 @@ extern "C" lbm_status lbm_add_scale_block(lbm_domain* dom, const double origin[3
     NB.post.push_back(mt);
   }
   dom->pick_tiles(id);
+  dom->pick_tiles(0);
   dom->invalidate_graphs();
   *block_id = id;
   return LBM_OK;

@@ -459,6 +459,24 @@ __device__ __forceinline__ void pull_pair(float2 (&d)[27], const T* __restrict__
   }
 }
 
+// bounce_back for the pair's component C (0 or 1), node address a0 + C.
+template <int C, typename T, typename IT, int K = 0>
+__device__ __forceinline__ void bounce_back_pair(float2 (&d)[27], const T* __restrict__ din, IT N,
+                                                 const uint8_t* __restrict__ flags, IT nx, IT nxy,
+                                                 IT am, IT a, IT ap) {
+  if constexpr (K < 27) {
+    if constexpr (K != 13) {
+      constexpr int cx = cxk(K), cy = cyk(K), cz = czk(K);
+      const IT src = (cx > 0 ? am : cx < 0 ? ap : a) - (IT)cz * nxy - (IT)cy * nx;
+      if (__ldg(flags + src) & F_SOLID) {
+        const float b = load_pop(din + ((IT)(26 - K) * N + a));
+        if constexpr (C == 0) d[K].x = b; else d[K].y = b;
+      }
+    }
+    bounce_back_pair<C, T, IT, K + 1>(d, din, N, flags, nx, nxy, am, a, ap);
+  }
+}
+
 // grad_norm_inner of both nodes (the y and z differences as aligned pair loads).
 template <typename IT>
 __device__ __forceinline__ float2 grad_norm_pair(const float* __restrict__ U, IT N, IT nx, IT nxy,
@@ -536,7 +554,8 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
   const IT a0 = row + (IT)x;
   const unsigned fl2 = __ldg(reinterpret_cast<const unsigned short*>(v.flags + a0));
   const uint8_t fl0 = (uint8_t)(fl2 & 0xffu), fl1 = (uint8_t)(fl2 >> 8);
-  constexpr uint8_t kNodeWise = F_SOLID | F_INFLOW | F_GHOST | F_NEAR_SOLID | F_WALL | F_OBST_WALL;
+  constexpr uint8_t kNodeWise = F_INFLOW | F_WALL | F_OBST_WALL;
+  constexpr uint8_t kDead = F_SOLID | F_GHOST;
   const T* __restrict__ din = static_cast<const T*>(v.d_in);
   T* __restrict__ dout = static_cast<T*>(v.d_out);
   // the loads of the pair path go out before the flags are looked at (256^3 FP32 658 -> 629 us,
@@ -544,9 +563,9 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
   const bool inner = inner_yz(v, y, z);
   float2 d[27];
   float2 g_lag = make_float2(0.0f, 0.0f);
+  const IT am0 = row + (IT)nbr(x, -1, v.nx, v.per[0]);
+  const IT ap1 = row + (IT)nbr(x + 1, 1, v.nx, v.per[0]);
   if (inner) {
-    const IT am0 = row + (IT)nbr(x, -1, v.nx, v.per[0]);
-    const IT ap1 = row + (IT)nbr(x + 1, 1, v.nx, v.per[0]);
     pull_pair<T, IT>(d, din, N, nxI, nxyI, am0, a0, ap1);
     if (v.rp.adaptive && !v.rp.local) g_lag = grad_norm_pair<IT>(v.u_in, N, nxI, nxyI, a0, am0, ap1);
   }
@@ -555,16 +574,47 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
     cell_update<T, IT, false, WALLS, RED>(v, x + 1, y, z, nm);
     return;
   }
+  // Obstacle voxels, scale-boundary (ghost) nodes and the nodes next to an obstacle stay in the
+  // pair path: a warp that holds one of them would otherwise go through the collision three
+  // times (256^3 inside a far-field block, whose outer nodes are scale-boundary ones: 1058 ->
+  // 722 us).
+  const bool live0 = !(fl0 & kDead), live1 = !(fl1 & kDead);
+  const bool mixed = ((fl0 | fl1) & (kDead | F_NEAR_SOLID)) != 0;
+  if (mixed) {
+    if (live0 && (fl0 & F_NEAR_SOLID))
+      bounce_back_pair<0, T, IT>(d, din, N, v.flags, nxI, nxyI, am0, a0, a0 + 1);
+    if (live1 && (fl1 & F_NEAR_SOLID))
+      bounce_back_pair<1, T, IT>(d, din, N, v.flags, nxI, nxyI, a0, a0 + 1, ap1);
+    if (!live0 && !live1) {       // obstacle voxels store zeros, ghost nodes nothing
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        if (!((c ? fl1 : fl0) & F_SOLID)) continue;
+        const IT a = a0 + (IT)c;
+#pragma unroll
+        for (int k = 0; k < 27; ++k) store_pop(dout + ((IT)k * N + a), 0.0f);
+        v.u_out[a] = v.u_out[N + a] = v.u_out[2 * N + a] = 0.0f;
+        v.c_out[a] = 0.0f;
+      }
+      return;
+    }
+  }
 
   raw_moments(d);
   const float2 drho = d[kap(0, 0, 0)];
   const float2 inv = make_float2(fast_rcp(__fadd_rn(1.0f, drho.x)), fast_rcp(__fadd_rn(1.0f, drho.y)));
-  const float2 ux = vmul(d[kap(1, 0, 0)], inv), uy = vmul(d[kap(0, 1, 0)], inv),
-               uz = vmul(d[kap(0, 0, 1)], inv);
-  flag_error(v.err, unphysical(drho.x, ux.x, uy.x, uz.x) || unphysical(drho.y, ux.y, uy.y, uz.y));
-  if constexpr (RED) nm->put_pair(drho, d[kap(1, 0, 0)], d[kap(0, 1, 0)], d[kap(0, 0, 1)], inv);
+  float2 ux = vmul(d[kap(1, 0, 0)], inv), uy = vmul(d[kap(0, 1, 0)], inv),
+         uz = vmul(d[kap(0, 0, 1)], inv);
+  flag_error(v.err, (live0 && unphysical(drho.x, ux.x, uy.x, uz.x)) ||
+                        (live1 && unphysical(drho.y, ux.y, uy.y, uz.y)));
+  if constexpr (RED) {
+    const float2 jx = d[kap(1, 0, 0)], jy = d[kap(0, 1, 0)], jz = d[kap(0, 0, 1)];
+    if (live0 && live1) nm->put_pair(drho, jx, jy, jz, inv);
+    else if (live0) nm->put(drho.x, jx.x, jy.x, jz.x, inv.x);
+    else nm->put(drho.y, jx.y, jy.y, jz.y, inv.y);
+  }
 
-  const bool src0 = (fl0 & F_SCALAR_SRC) != 0, src1 = (fl1 & F_SCALAR_SRC) != 0;
+  // (a dead component's departure point is never looked up)
+  const bool src0 = !live0 || (fl0 & F_SCALAR_SRC), src1 = !live1 || (fl1 & F_SCALAR_SRC);
   constexpr bool kAsync = pair_corners_async<T>();
   ScalarCell sc0, sc1;
   if constexpr (kAsync) {
@@ -585,12 +635,33 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
   const KeepT<float2> kf = pair_keep(keep_factors(v.rp, g.x), keep_factors(v.rp, g.y));
   collide_from_central(d, drho, ux, uy, uz, kf);
 
+  const bool ghost = mixed && ((fl0 & kDead) == F_GHOST || (fl1 & kDead) == F_GHOST);
+  if (mixed && ((fl0 | fl1) & F_SOLID)) {
+    if (fl0 & F_SOLID) {
 #pragma unroll
-  for (int k = 0; k < 27; ++k) store_pop2(dout + ((IT)k * N + a0), d[k]);
-  __stcs(reinterpret_cast<float2*>(v.u_out + a0), ux);
-  __stcs(reinterpret_cast<float2*>(v.u_out + (N + a0)), uy);
-  __stcs(reinterpret_cast<float2*>(v.u_out + (2 * N + a0)), uz);
-  float c0 = v.c_src, c1 = v.c_src;
+      for (int k = 0; k < 27; ++k) d[k].x = 0.0f;
+      ux.x = uy.x = uz.x = 0.0f;
+    } else {
+#pragma unroll
+      for (int k = 0; k < 27; ++k) d[k].y = 0.0f;
+      ux.y = uy.y = uz.y = 0.0f;
+    }
+  }
+  const IT al = a0 + (IT)(live0 ? 0 : 1);        // the live node beside a ghost
+  if (!ghost) {
+#pragma unroll
+    for (int k = 0; k < 27; ++k) store_pop2(dout + ((IT)k * N + a0), d[k]);
+    __stcs(reinterpret_cast<float2*>(v.u_out + a0), ux);
+    __stcs(reinterpret_cast<float2*>(v.u_out + (N + a0)), uy);
+    __stcs(reinterpret_cast<float2*>(v.u_out + (2 * N + a0)), uz);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 27; ++k) store_pop(dout + ((IT)k * N + al), live0 ? d[k].x : d[k].y);
+    __stcs(v.u_out + al, live0 ? ux.x : ux.y);
+    __stcs(v.u_out + (N + al), live0 ? uy.x : uy.y);
+    __stcs(v.u_out + (2 * N + al), live0 ? uz.x : uz.y);
+  }
+  float c0 = (fl0 & F_SOLID) ? 0.0f : v.c_src, c1 = (fl1 & F_SOLID) ? 0.0f : v.c_src;
   if constexpr (kAsync) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (!src0) c0 = scalar_value_slots(v, x, y, z, ux.x, uy.x, uz.x, slot, stride);
@@ -599,7 +670,8 @@ __device__ __forceinline__ void cell_update_pair(const BlockView& v, int x, int 
     if (!src0) c0 = scalar_value(sc0);
     if (!src1) c1 = scalar_value(sc1);
   }
-  __stcs(reinterpret_cast<float2*>(v.c_out + a0), make_float2(c0, c1));
+  if (!ghost) __stcs(reinterpret_cast<float2*>(v.c_out + a0), make_float2(c0, c1));
+  else __stcs(v.c_out + al, live0 ? c0 : c1);
 }
 
 }  // namespace lbm

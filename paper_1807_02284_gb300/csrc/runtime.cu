@@ -393,6 +393,7 @@ lbm_status lbm_set_boundary(lbm_domain* dom, int32_t block_id, int32_t kind, con
     }
     if (e != cudaSuccess) return dom->cuda_fail(e, "wall flags");
     dom->walls = walls;
+    for (size_t i = 0; i < dom->blocks.size(); ++i) dom->pick_tiles((int)i);
     dom->invalidate_graphs();
     return LBM_OK;
   }

@@ -48,6 +48,7 @@ struct Block {
   RelaxParams rp;
   int bx = 128, by = 2;    // tile of the collide-stream launch
   int minb = 3;            // register bound of the collide-stream launch (CTAs per SM)
+  bool tile_forced = false;  // LBM_TILE chose them
   // far-field block (h > 1, Sec. 4.2.4-4.2.5): it surrounds block `child` (s0 or the previous
   // far block), takes its nodes inside the child's interior from the child (far_in) and
   // gives the child its outer layer (far_out)

@@ -49,8 +49,15 @@ static std::vector<int> next_levels(const std::vector<lbm::Block>& blocks, std::
 // step of fluid blocks on GB300, every shape and register bound tried at each size.
 void lbm_domain::pick_tiles(int b) {
   Block& B = blocks[b];
+  if (B.tile_forced) return;
   const bool half = desc.storage == LBM_FP16_SHIFTED;
-  if (B.nx % 2 == 0 && B.N >= (size_t)1 << 20) {
+  // walls and refined scales: warps with wall nodes take the node-wise path, and the step runs
+  // beside other blocks' kernels, so pairs pay only from 4 M nodes (196 x 98 x 98 with
+  // obstacle-surface walls 86 us with one node per thread, 100 with two; 128^3 under two refined
+  // scales 112 against 130; 256^3 inside a far-field block 740 against 722, with
+  // obstacle-surface walls 669 with two)
+  const size_t pairs_from = (size_t)1 << (walls || blocks.size() > 1 ? 22 : 20);
+  if (B.nx % 2 == 0 && B.N >= pairs_from) {
     // two nodes per thread once the block is bound by bandwidth or issue rather than by
     // latency: from 1 M nodes (96^3 FP32 42.5 against 40.8 us with one node per thread, FP16 41.2
     // against 40.0; 128^3 84 against 91, FP16 80 against 96; 256^3 629 against 702, FP16 592
@@ -85,6 +92,7 @@ void lbm_domain::pick_tiles(int b) {
       B.bx = bx;
       B.by = by;
       B.minb = mb;
+      B.tile_forced = true;
     }
   }
 }

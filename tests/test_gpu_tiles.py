@@ -40,3 +40,28 @@ def test_one_row_ctas_equal_tiles(lib, monkeypatch, dims, storage, walls):
         for a, b in zip(ref, got):
             assert np.array_equal(a, b), tile
         assert np.abs(d - dref).max() <= 256 * 2.0 ** -24 * np.abs(dref).max()
+
+
+@pytest.mark.parametrize("dims", [(36, 30, 28), (34, 9, 11)])
+def test_pairs_with_ghost_and_obstacle_nodes_equal_single_nodes(lib, monkeypatch, dims):
+    """A block with obstacles inside a far-field block (its outer nodes are scale-boundary
+    ones): two nodes per thread give the bits of one node per thread in every block."""
+    from paper_1807_02284_gb300 import lbm
+    from tests.test_gpu_multiscale import gpu_multiscale
+    sc = synth.random_scene(dims=dims, seed=4, periodic=(False,) * 3, nu=0.01, amp=0.04)
+    rng = np.random.default_rng(8)
+    solid = rng.random(sc.blocks[0].flags.shape) < 0.05
+    solid[:3] = solid[-3:] = False
+    solid[:, :3] = solid[:, -3:] = False
+    solid[:, :, :3] = solid[:, :, -3:] = False
+    sc.blocks[0].flags[solid] = synth.SOLID
+    sc.blocks.append(synth.far_block(sc.blocks[0], 2.0, 8.0, seed=9))
+    out = []
+    for tile in ("128,1,4", "64,2,20", "128,1,20"):
+        monkeypatch.setenv("LBM_TILE", tile)
+        dom = gpu_multiscale(sc)
+        dom.step(5)
+        out.append([dom.read_field(lbm.LBM_FIELD_F, lbm.LBM_F64, block=b) for b in (0, 1)])
+        dom.close()
+    for o in out[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(out[0], o))
