@@ -512,7 +512,8 @@ lbm_status lbm_set_tape(lbm_domain* dom, int32_t checkpoint_every);
    carried unchanged by every step, so dL_du0 at inflow nodes is the gradient with respect to
    that inflow velocity; dL_dinflow (3N floats, device, may be NULL) receives the same values
    at inflow nodes and 0 elsewhere (inflow velocities must not be changed while the tape
-   records).  Continuous-scale domains (refined blocks) are reversed through the whole
+   records; records set after its last step are the next frame's and leave this gradient as
+   it is, as do node boxes written then).  Continuous-scale domains (refined blocks) are reversed through the whole
    Algorithm 1 schedule (prior- and post-mapping, sub-steps, temporal alignment); the loss
    is a function of block 0's final state, dL_du0 is block 0's gradient and
    lbm_adjoint_block_grad returns the other blocks'.  No-slip walls (wall faces and

@@ -33,6 +33,7 @@
 // schedule further below).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "lbm_adjoint.cuh"
@@ -1099,6 +1100,7 @@ struct TapeState {
   int every = 0;
   std::vector<Level> ckpt;    // states at steps 0, every, 2 every, ...
   std::vector<Level> seg;     // recompute levels 1..every of one segment
+  std::vector<long long> changed;   // step counts at which the caller wrote into the live state
   float* lam[2] = {nullptr, nullptr};
   float* ups[2] = {nullptr, nullptr};
   float* gam[2] = {nullptr, nullptr};
@@ -1150,6 +1152,11 @@ void release_tape(lbm_domain* dom) {
   for (float* g : t->grad) dom->tape_free(g);
   delete t;
   dom->tape = nullptr;
+}
+
+void tape_state_changed(lbm_domain* dom) {
+  TapeState* t = dom->tape;
+  if (t && (t->changed.empty() || t->changed.back() != dom->steps)) t->changed.push_back(dom->steps);
 }
 
 static bool alloc_level(lbm_domain* dom, size_t N, Level& L) {
@@ -1755,8 +1762,20 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
     cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
     if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");
   }
-  const bool fp32 = dom->desc.storage == LBM_FP32;
-  const int seg_len = std::min(t->every, std::max(1, n_steps)) - (fp32 ? 1 : 0);
+  const int n_seg = (n_steps + t->every - 1) / t->every;
+  // Steps of segment sg that are replayed.  The last one's result is wanted for its velocity
+  // alone, which the forward kept: it is the next checkpoint's, or the domain's current one, bit
+  // for bit what the replay computes with FP32 storage.  Not where the caller has written into
+  // that state since (inflow records of the next frame, node boxes), and not with FP16 storage,
+  // whose replay follows unrounded states: there the replay's own result is taken.
+  auto replayed = [&](int sg) {
+    const int end = std::min((sg + 1) * t->every, n_steps);
+    const bool kept = dom->desc.storage == LBM_FP32 &&
+                      std::find(t->changed.begin(), t->changed.end(), (long long)end) == t->changed.end();
+    return end - sg * t->every - (kept ? 1 : 0);
+  };
+  int seg_len = 0;
+  for (int sg = 0; sg < n_seg; ++sg) seg_len = std::max(seg_len, replayed(sg));
   while ((int)t->seg.size() < seg_len) {
     Level L;
     if (!alloc_level(dom, N, L)) {
@@ -1780,18 +1799,14 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
   if (e == cudaSuccess) e = cudaMemcpyAsync(t->gam[0], dL_dc, N * sizeof(float), cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint initialisation");
 
-  const int n_seg = (n_steps + t->every - 1) / t->every;
   const bool open_faces = !dom->desc.periodic[0] || !dom->desc.periodic[1] || !dom->desc.periodic[2];
   for (int sg = n_seg - 1; sg >= 0; --sg) {
     const int s0 = sg * t->every;
     const int len = std::min(t->every, n_steps - s0);
-    // recompute the segment's states 1..n_replay from its checkpoint.  The last step's result
-    // is wanted for its velocity alone, which the forward kept: it is the next checkpoint's, or
-    // the domain's current one (bit for bit what the replay computes with FP32 storage; an FP16
-    // run's replay follows unrounded states, so its own result is taken there)
+    // recompute the segment's states 1..n_replay from its checkpoint
     auto level = [&](int i) -> const Level& { return i == 0 ? t->ckpt[sg] : t->seg[i - 1]; };
-    const int n_replay = fp32 ? len - 1 : len;
-    const float* u_end = !fp32 ? nullptr : sg == n_seg - 1 ? B.lv[B.cur].u : t->ckpt[sg + 1].u;
+    const int n_replay = replayed(sg);
+    const float* u_end = n_replay == len ? nullptr : sg == n_seg - 1 ? B.lv[B.cur].u : t->ckpt[sg + 1].u;
     for (int i = 0; i < n_replay; ++i) {
       e = launch_step(view_of(dom, level(i), level(i + 1)), ST_FP32, B.bx, B.by, s, B.minb);
       if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint recompute");

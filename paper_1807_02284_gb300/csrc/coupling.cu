@@ -1239,6 +1239,7 @@ static lbm_status box_transfer(lbm_domain* dom, int32_t block, int32_t level, co
                                        B.N, l3, d3, nb, static_cast<float*>(buf), dir, skip);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return dom->cuda_fail(e, "node box copy");
+  if (dir) tape_state_changed(dom);
   return LBM_OK;
 }
 

@@ -411,6 +411,7 @@ lbm_status lbm_set_boundary(lbm_domain* dom, int32_t block_id, int32_t kind, con
     cudaError_t e = launch_inflow_records(src, n, B.flags, lv.data(), (int)lv.size(), B.nx,
                                           B.ny, B.nz, B.N, dom->d_err, dom->stream);
     if (e != cudaSuccess) return dom->cuda_fail(e, "inflow records");
+    tape_state_changed(dom);
     return on_device ? LBM_OK : dom->small_used();
   }
   return dom->fail(LBM_ERR_INVALID_ARG, "unknown boundary kind");
@@ -805,5 +806,7 @@ lbm_status lbm_set_inflow_batch(lbm_domain* const* doms, int32_t n,
     e = launch_inflow_records_multi(g + mb, (int)total, reinterpret_cast<const int*>(g + mb + rb),
                                     reinterpret_cast<const InflowMember*>(g), d0->stream);
   if (e != cudaSuccess) return d0->cuda_fail(e, "inflow batch");
+  for (int i = 0; i < n; ++i)
+    if (counts[i]) tape_state_changed(doms[i]);
   return LBM_OK;
 }

@@ -155,3 +155,7 @@ struct lbm_domain {
 };
 
 using Domain = lbm_domain;
+
+// The caller has written into block 0's current state outside a step: a recording tape must not
+// take it for the result of the step before (adjoint.cu).
+void tape_state_changed(lbm_domain* dom);
