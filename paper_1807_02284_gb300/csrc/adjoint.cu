@@ -1127,6 +1127,26 @@ static void free_level(lbm_domain* dom, Level& L) {
   L = Level();
 }
 
+// The buffers of a continuous-scale domain's reverse sweep.
+static void free_sweep(lbm_domain* dom, TapeState* t) {
+  for (auto& v : t->ver) for (Level& L : v) free_level(dom, L);
+  for (Level& L : t->spare) free_level(dom, L);
+  for (auto& v : t->lamb)
+    for (AdjLevel& A : v) {
+      dom->tape_free(A.f);
+      dom->tape_free(A.u);
+      dom->tape_free(A.c);
+    }
+  for (float* g : t->grad) dom->tape_free(g);
+  dom->tape_free(t->ms);
+  dom->tape_free(t->side);
+  t->ver.clear();
+  t->spare.clear();
+  t->lamb.clear();
+  t->grad.clear();
+  t->ms = t->side = nullptr;
+}
+
 void release_tape(lbm_domain* dom) {
   TapeState* t = dom->tape;
   if (!t) return;
@@ -1137,19 +1157,9 @@ void release_tape(lbm_domain* dom) {
     dom->tape_free(t->ups[i]);
     dom->tape_free(t->gam[i]);
   }
-  dom->tape_free(t->ms);
-  dom->tape_free(t->side);
   for (auto& v : t->mck) for (Level& L : v) free_level(dom, L);
   for (auto& v : t->snap) for (Level& L : v) free_level(dom, L);
-  for (auto& v : t->ver) for (Level& L : v) free_level(dom, L);
-  for (Level& L : t->spare) free_level(dom, L);
-  for (auto& v : t->lamb)
-    for (AdjLevel& A : v) {
-      dom->tape_free(A.f);
-      dom->tape_free(A.u);
-      dom->tape_free(A.c);
-    }
-  for (float* g : t->grad) dom->tape_free(g);
+  free_sweep(dom, t);
   delete t;
   dom->tape = nullptr;
 }
@@ -1595,6 +1605,40 @@ static bool alloc_adj(lbm_domain* dom, size_t N, AdjLevel& A) {
   return A.f && A.u && A.c;
 }
 
+// The buffers of a reverse sweep over blocks with `versions` value versions each, all of them or
+// (a failed allocation) none.
+static lbm_status alloc_sweep(lbm_domain* dom, TapeState* t, const std::vector<int>& versions) {
+  const int nb = (int)dom->blocks.size();
+  size_t nmax = 0, side = 0;
+  bool ok = true;
+  cudaError_t e = cudaSuccess;
+  t->ver.resize(nb);
+  t->spare.resize(nb);
+  t->lamb.resize(nb);
+  t->grad.assign(nb, nullptr);
+  for (int b = 0; b < nb; ++b) {
+    const Block& B = dom->blocks[b];
+    nmax = std::max(nmax, B.N);
+    side = std::max(side, face_side_floats(B.nx, B.ny, B.nz));
+    t->ver[b].resize(versions[b] - 1);
+    for (Level& L : t->ver[b]) {
+      ok = ok && alloc_level(dom, B.N, L);
+      // (a scale boundary that no one has written yet is read with weight 0: keep it finite)
+      if (ok && e == cudaSuccess) e = copy_level(L, Level{}, B.N, dom->stream);
+    }
+    if (b) ok = ok && alloc_level(dom, B.N, t->spare[b]);
+    t->lamb[b].resize(b == 0 ? 2 : 3);
+    for (AdjLevel& A : t->lamb[b]) ok = ok && alloc_adj(dom, B.N, A);
+    if (ok) ok = (t->grad[b] = static_cast<float*>(dom->tape_alloc(B.N * 3 * sizeof(float)))) != nullptr;
+  }
+  if (ok) ok = (t->ms = static_cast<float*>(dom->tape_alloc(nmax * sizeof(float)))) != nullptr;
+  if (ok) ok = (t->side = static_cast<float*>(dom->tape_alloc(side * sizeof(float)))) != nullptr;
+  if (ok && e == cudaSuccess) e = cudaMemsetAsync(t->side, 0, side * sizeof(float), dom->stream);
+  if (ok && e == cudaSuccess) return LBM_OK;
+  free_sweep(dom, t);
+  return ok ? dom->cuda_fail(e, "adjoint buffers") : dom->fail(LBM_ERR_OOM, "adjoint buffers");
+}
+
 // Reverse sweep of a continuous-scale domain: the recorded reference steps are reversed last
 // to first; each segment between checkpoints is replayed once to record every step's start
 // state, and each step once more from there, keeping a version of every value that its
@@ -1607,41 +1651,12 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
   TapeState* t = dom->tape;
   cudaStream_t s = dom->stream;
   const int nb = (int)dom->blocks.size();
-  size_t nmax = 0;
-  for (const Block& B : dom->blocks) nmax = std::max(nmax, B.N);
   std::vector<int> cur_end, versions, last;
   std::vector<MsOp> ops = ms_ops(dom, cur_end);
   ms_versions(ops, cur_end, versions, last);
-  // buffers
   if (t->lamb.empty()) {
-    t->ver.resize(nb);
-    t->spare.resize(nb);
-    t->lamb.resize(nb);
-    t->grad.assign(nb, nullptr);
-    for (int b = 0; b < nb; ++b) {
-      const size_t N = dom->blocks[b].N;
-      const int levels = b == 0 ? 2 : 3;
-      t->ver[b].resize(versions[b] - 1);
-      for (Level& L : t->ver[b]) {
-        if (!alloc_level(dom, N, L)) return dom->fail(LBM_ERR_OOM, "adjoint replay levels");
-        // (a scale boundary that no one has written yet is read with weight 0: keep it finite)
-        if (copy_level(L, Level{}, N, s) != cudaSuccess)
-          return dom->fail(LBM_ERR_CUDA, "adjoint replay levels");
-      }
-      if (b && !alloc_level(dom, N, t->spare[b])) return dom->fail(LBM_ERR_OOM, "adjoint replay levels");
-      t->lamb[b].resize(levels);
-      for (AdjLevel& A : t->lamb[b])
-        if (!alloc_adj(dom, N, A)) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-      t->grad[b] = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
-      if (!t->grad[b]) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-    }
-    t->ms = static_cast<float*>(dom->tape_alloc(nmax * sizeof(float)));
-    size_t side = 0;
-    for (const Block& B : dom->blocks) side = std::max(side, face_side_floats(B.nx, B.ny, B.nz));
-    t->side = static_cast<float*>(dom->tape_alloc(side * sizeof(float)));
-    if (!t->ms || !t->side) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-    cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
-    if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");
+    const lbm_status st = alloc_sweep(dom, t, versions);
+    if (st != LBM_OK) return st;
   }
   const int seg_len = std::min(t->every, std::max(1, n_steps));
   while ((int)t->snap.size() < seg_len) {

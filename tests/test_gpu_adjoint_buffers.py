@@ -1,0 +1,89 @@
+"""Device buffers of the adjoint: a failed allocation leaves the tape as it was, so that the
+same call works once there is memory again."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from tests.helpers import f32
+from tests.test_gpu_adjoint import rel
+from tests.test_gpu_multiscale import gpu_multiscale
+
+pytestmark = pytest.mark.gpu
+
+
+class Allocations:
+    """Counts the library's device allocations; number `fail_at` fails (the caller's allocator
+    raises, the library gets NULL)."""
+
+    def __init__(self, monkeypatch):
+        self.count, self.fail_at = 0, -1
+        real = torch.cuda.caching_allocator_alloc
+
+        def alloc(nbytes, device=None, stream=None):
+            self.count += 1
+            if self.count - 1 == self.fail_at:
+                raise RuntimeError("no memory")
+            return real(nbytes, device, stream)
+
+        monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", alloc)
+
+
+def _scene(blocks):
+    if blocks == 1:
+        sc, _ = synth.adjoint_scene(n=12, seed=5, nu=0.01)
+        sc.periodic = (False, False, True)
+        return sc
+    sc = synth.multiscale(seed=2, sphere_seed=3, scale=0.125, flow_amp=0.03, nu=0.004)
+    sc.blocks = sc.blocks[:2]
+    return sc
+
+
+def _domain(sc):
+    from paper_1807_02284_gb300 import lbm
+    if len(sc.blocks) > 1:
+        return gpu_multiscale(sc)
+    b = sc.blocks[0]
+    d = lbm.Domain(b.dims, sc.nu, periodic=sc.periodic)
+    d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0))
+    return d
+
+
+@pytest.mark.parametrize("blocks", [1, 2])
+def test_reverse_sweep_after_a_failed_allocation(lib, monkeypatch, blocks):
+    """Every allocation of lbm_adjoint_step in turn: OOM, then the same call gives the
+    gradient.  Bound 1e-5: one block repeats its bits; the mappings' atomic sums of at most 16
+    corners come in any order, 2^-24 each, over three steps."""
+    from paper_1807_02284_gb300 import lbm
+    sc = _scene(blocks)
+    mem = Allocations(monkeypatch)
+    n = sc.blocks[0].flags.size
+    dc = torch.rand(n, device="cuda")
+    ref, fail = None, -1
+    while True:
+        d = _domain(sc)
+        d.set_tape(2)
+        d.step(3)
+        g = torch.full((3 * n,), 7.0, device="cuda")
+        torch.cuda.synchronize()
+        mem.count, mem.fail_at = 0, fail
+        failed = False
+        try:
+            d.adjoint_step(3, dc, g)
+        except lbm.LBMError as err:
+            assert err.status == lbm.LBM_ERR_OOM
+            failed = True
+            mem.fail_at = -1
+            d.adjoint_step(3, dc, g)
+        d.sync()
+        mem.fail_at = -1
+        d.close()
+        g = g.cpu().numpy().astype(np.float64)
+        if ref is None:
+            ref, total = g, mem.count
+            assert total > 0 and not failed
+        else:
+            assert failed and rel(g, ref) <= 1e-5, fail
+        fail += 1
+        if fail == total:
+            break
