@@ -1100,6 +1100,7 @@ struct TapeState {
   int every = 0;
   std::vector<Level> ckpt;    // states at steps 0, every, 2 every, ...
   std::vector<Level> seg;     // recompute levels 1..every of one segment
+  std::vector<void*> buffers;       // device memory of everything below (tape_buffer)
   std::vector<long long> changed;   // step counts at which the caller wrote into the live state
   float* lam[2] = {nullptr, nullptr};
   float* ups[2] = {nullptr, nullptr};
@@ -1120,60 +1121,53 @@ struct TapeState {
 
 using namespace lbm;
 
-static void free_level(lbm_domain* dom, Level& L) {
-  dom->tape_free(L.f);
-  dom->tape_free(L.u);
-  dom->tape_free(L.c);
-  L = Level();
-}
-
-// The buffers of a continuous-scale domain's reverse sweep.
-static void free_sweep(lbm_domain* dom, TapeState* t) {
-  for (auto& v : t->ver) for (Level& L : v) free_level(dom, L);
-  for (Level& L : t->spare) free_level(dom, L);
-  for (auto& v : t->lamb)
-    for (AdjLevel& A : v) {
-      dom->tape_free(A.f);
-      dom->tape_free(A.u);
-      dom->tape_free(A.c);
-    }
-  for (float* g : t->grad) dom->tape_free(g);
-  dom->tape_free(t->ms);
-  dom->tape_free(t->side);
-  t->ver.clear();
-  t->spare.clear();
-  t->lamb.clear();
-  t->grad.clear();
-  t->ms = t->side = nullptr;
-}
-
+// A tape's memory goes back with the tape (the next lbm_init_macro or lbm_set_tape), in few pieces: a
+// level, or all that one reverse sweep works on, is one allocation, since a call into the caller's
+// allocator takes about 2 us of host time (three arrays a level were 26 allocations and as many
+// releases per gradient of a 12-step plume, about 100 us of 1850).
 void release_tape(lbm_domain* dom) {
   TapeState* t = dom->tape;
   if (!t) return;
-  for (Level& L : t->ckpt) free_level(dom, L);
-  for (Level& L : t->seg) free_level(dom, L);
-  for (int i = 0; i < 2; ++i) {
-    dom->tape_free(t->lam[i]);
-    dom->tape_free(t->ups[i]);
-    dom->tape_free(t->gam[i]);
-  }
-  for (auto& v : t->mck) for (Level& L : v) free_level(dom, L);
-  for (auto& v : t->snap) for (Level& L : v) free_level(dom, L);
-  free_sweep(dom, t);
+  for (void* p : t->buffers) dom->dev_free(p);
   delete t;
   dom->tape = nullptr;
+}
+
+// FP32 arrays one after another in a buffer, each from a 256-byte boundary on.
+struct Carve {
+  float* base = nullptr;     // null: only adds up the size
+  size_t floats = 0;
+  float* take(size_t n) {
+    float* p = base ? base + floats : nullptr;
+    floats += (n + 63) / 64 * 64;
+    return p;
+  }
+  Level level(size_t N) {
+    Level L;
+    L.f = take(27 * N);
+    L.u = take(3 * N);
+    L.c = take(N);
+    return L;
+  }
+};
+
+// One allocation of the tape for the arrays that layout(Carve&) takes; false (and the arrays
+// null) when there is no memory.
+template <typename Layout>
+static bool tape_buffer(lbm_domain* dom, const Layout& layout) {
+  Carve size;
+  layout(size);
+  Carve place;
+  place.base = static_cast<float*>(dom->dev_alloc(size.floats * sizeof(float)));
+  if (!place.base) return false;
+  dom->tape->buffers.push_back(place.base);
+  layout(place);
+  return true;
 }
 
 void tape_state_changed(lbm_domain* dom) {
   TapeState* t = dom->tape;
   if (t && (t->changed.empty() || t->changed.back() != dom->steps)) t->changed.push_back(dom->steps);
-}
-
-static bool alloc_level(lbm_domain* dom, size_t N, Level& L) {
-  L.f = dom->tape_alloc(N * 27 * sizeof(float));
-  L.u = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
-  L.c = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
-  return L.f && L.u && L.c;
 }
 
 static BlockView view_of(lbm_domain* dom, const Level& from, const Level& to) {
@@ -1271,11 +1265,10 @@ lbm_status tape_before_step(lbm_domain* dom) {
   if (t->multi) {    // every block's state at the step start
     while (t->mck.size() <= i) {
       std::vector<Level> v(dom->blocks.size());
-      for (size_t b = 0; b < v.size(); ++b)
-        if (!alloc_level(dom, dom->blocks[b].N, v[b])) {
-          for (Level& L : v) free_level(dom, L);
-          return dom->fail(LBM_ERR_OOM, "checkpoint allocation failed");
-        }
+      if (!tape_buffer(dom, [&](Carve& m) {
+            for (size_t b = 0; b < v.size(); ++b) v[b] = m.level(dom->blocks[b].N);
+          }))
+        return dom->fail(LBM_ERR_OOM, "checkpoint allocation failed");
       t->mck.push_back(v);
     }
     PieceList list(dom->stream);
@@ -1290,10 +1283,8 @@ lbm_status tape_before_step(lbm_domain* dom) {
   Block& B = dom->blocks[0];
   while (t->ckpt.size() <= i) {
     Level L;
-    if (!alloc_level(dom, B.N, L)) {
-      free_level(dom, L);
+    if (!tape_buffer(dom, [&](Carve& m) { L = m.level(B.N); }))
       return dom->fail(LBM_ERR_OOM, "checkpoint allocation failed");
-    }
     t->ckpt.push_back(L);
   }
   const Level& S = B.lv[B.cur];
@@ -1330,10 +1321,7 @@ extern "C" lbm_status lbm_set_tape(lbm_domain* dom, int32_t every) {
   cudaSetDevice(dom->desc.device);
   if (every < 0) return dom->fail(LBM_ERR_INVALID_ARG, "checkpoint_every must be >= 0");
   release_tape(dom);
-  if (every == 0) {
-    dom->drop_tape_pool();
-    return LBM_OK;
-  }
+  if (every == 0) return LBM_OK;
   if (dom->steps != 0)
     return dom->fail(LBM_ERR_STATE, "the tape must be enabled right after lbm_init_macro");
   lbm_status st = adjoint_supported(dom);
@@ -1598,44 +1586,48 @@ static cudaError_t ms_reverse_op(const MsStep& m, const MsOp& o, cudaStream_t s)
   return cudaGetLastError();
 }
 
-static bool alloc_adj(lbm_domain* dom, size_t N, AdjLevel& A) {
-  A.f = static_cast<float*>(dom->tape_alloc(N * 27 * sizeof(float)));
-  A.u = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
-  A.c = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
-  return A.f && A.u && A.c;
-}
-
 // The buffers of a reverse sweep over blocks with `versions` value versions each, all of them or
 // (a failed allocation) none.
 static lbm_status alloc_sweep(lbm_domain* dom, TapeState* t, const std::vector<int>& versions) {
   const int nb = (int)dom->blocks.size();
   size_t nmax = 0, side = 0;
-  bool ok = true;
-  cudaError_t e = cudaSuccess;
+  for (const Block& B : dom->blocks) {
+    nmax = std::max(nmax, B.N);
+    side = std::max(side, face_side_floats(B.nx, B.ny, B.nz));
+  }
   t->ver.resize(nb);
   t->spare.resize(nb);
   t->lamb.resize(nb);
-  t->grad.assign(nb, nullptr);
+  t->grad.resize(nb);
   for (int b = 0; b < nb; ++b) {
-    const Block& B = dom->blocks[b];
-    nmax = std::max(nmax, B.N);
-    side = std::max(side, face_side_floats(B.nx, B.ny, B.nz));
     t->ver[b].resize(versions[b] - 1);
-    for (Level& L : t->ver[b]) {
-      ok = ok && alloc_level(dom, B.N, L);
-      // (a scale boundary that no one has written yet is read with weight 0: keep it finite)
-      if (ok && e == cudaSuccess) e = copy_level(L, Level{}, B.N, dom->stream);
-    }
-    if (b) ok = ok && alloc_level(dom, B.N, t->spare[b]);
     t->lamb[b].resize(b == 0 ? 2 : 3);
-    for (AdjLevel& A : t->lamb[b]) ok = ok && alloc_adj(dom, B.N, A);
-    if (ok) ok = (t->grad[b] = static_cast<float*>(dom->tape_alloc(B.N * 3 * sizeof(float)))) != nullptr;
   }
-  if (ok) ok = (t->ms = static_cast<float*>(dom->tape_alloc(nmax * sizeof(float)))) != nullptr;
-  if (ok) ok = (t->side = static_cast<float*>(dom->tape_alloc(side * sizeof(float)))) != nullptr;
-  if (ok && e == cudaSuccess) e = cudaMemsetAsync(t->side, 0, side * sizeof(float), dom->stream);
-  if (ok && e == cudaSuccess) return LBM_OK;
-  free_sweep(dom, t);
+  const bool ok = tape_buffer(dom, [&](Carve& m) {
+    for (int b = 0; b < nb; ++b) {
+      const size_t N = dom->blocks[b].N;
+      for (Level& L : t->ver[b]) L = m.level(N);
+      if (b) t->spare[b] = m.level(N);
+      for (AdjLevel& A : t->lamb[b]) A = AdjLevel{m.take(27 * N), m.take(3 * N), m.take(N)};
+      t->grad[b] = m.take(3 * N);
+    }
+    t->ms = m.take(nmax);
+    t->side = m.take(side);
+  });
+  cudaError_t e = cudaSuccess;
+  if (ok) {
+    PieceList zero(dom->stream);
+    // (a scale boundary that no one has written yet is read with weight 0: keep it finite)
+    for (int b = 0; b < nb; ++b)
+      for (Level& L : t->ver[b]) zero.level(L, Level{}, dom->blocks[b].N);
+    zero.add(t->side, nullptr, side);
+    e = zero.flush();
+    if (e == cudaSuccess) return LBM_OK;
+  }
+  t->ver.clear();
+  t->spare.clear();
+  t->lamb.clear();
+  t->grad.clear();
   return ok ? dom->cuda_fail(e, "adjoint buffers") : dom->fail(LBM_ERR_OOM, "adjoint buffers");
 }
 
@@ -1661,11 +1653,10 @@ static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* 
   const int seg_len = std::min(t->every, std::max(1, n_steps));
   while ((int)t->snap.size() < seg_len) {
     std::vector<Level> v(nb);
-    for (int b = 0; b < nb; ++b)
-      if (!alloc_level(dom, dom->blocks[b].N, v[b])) {
-        for (Level& L : v) free_level(dom, L);
-        return dom->fail(LBM_ERR_OOM, "adjoint step snapshots");
-      }
+    if (!tape_buffer(dom, [&](Carve& m) {
+          for (int b = 0; b < nb; ++b) v[b] = m.level(dom->blocks[b].N);
+        }))
+      return dom->fail(LBM_ERR_OOM, "adjoint step snapshots");
     t->snap.push_back(v);
   }
   if (t->mck.empty()) {
@@ -1762,19 +1753,19 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
   const size_t N = B.N;
   cudaStream_t s = dom->stream;
   // buffers
-  for (int i = 0; i < 2; ++i) {
-    if (!t->lam[i]) t->lam[i] = static_cast<float*>(dom->tape_alloc(N * 27 * sizeof(float)));
-    if (!t->ups[i]) t->ups[i] = static_cast<float*>(dom->tape_alloc(N * 3 * sizeof(float)));
-    if (!t->gam[i]) t->gam[i] = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
-    if (!t->lam[i] || !t->ups[i] || !t->gam[i]) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-  }
-  if (!t->ms) t->ms = static_cast<float*>(dom->tape_alloc(N * sizeof(float)));
-  if (!t->ms) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-  if (!t->side) {
+  if (!t->ms) {
     const size_t side = face_side_floats(B.nx, B.ny, B.nz);
-    t->side = static_cast<float*>(dom->tape_alloc(side * sizeof(float)));
-    if (!t->side) return dom->fail(LBM_ERR_OOM, "adjoint buffers");
-    cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
+    if (!tape_buffer(dom, [&](Carve& m) {
+          for (int i = 0; i < 2; ++i) {
+            t->lam[i] = m.take(27 * N);
+            t->ups[i] = m.take(3 * N);
+            t->gam[i] = m.take(N);
+          }
+          t->ms = m.take(N);
+          t->side = m.take(side);
+        }))
+      return dom->fail(LBM_ERR_OOM, "adjoint buffers");
+    const cudaError_t e = cudaMemsetAsync(t->side, 0, side * sizeof(float), s);
     if (e != cudaSuccess) return dom->cuda_fail(e, "adjoint buffers");
   }
   const int n_seg = (n_steps + t->every - 1) / t->every;
@@ -1791,13 +1782,15 @@ extern "C" lbm_status lbm_adjoint_step(lbm_domain* dom, int32_t n_steps, const f
   };
   int seg_len = 0;
   for (int sg = 0; sg < n_seg; ++sg) seg_len = std::max(seg_len, replayed(sg));
+  // (levels of small blocks share an allocation of at most 256 MB)
+  const size_t group = std::max<size_t>(1, ((size_t)256 << 20) / (31 * N * sizeof(float)));
   while ((int)t->seg.size() < seg_len) {
-    Level L;
-    if (!alloc_level(dom, N, L)) {
-      free_level(dom, L);
+    std::vector<Level> v(std::min(group, (size_t)seg_len - t->seg.size()));
+    if (!tape_buffer(dom, [&](Carve& m) {
+          for (Level& L : v) L = m.level(N);
+        }))
       return dom->fail(LBM_ERR_OOM, "recompute levels");
-    }
-    t->seg.push_back(L);
+    t->seg.insert(t->seg.end(), v.begin(), v.end());
   }
   if (t->ckpt.empty()) {  // no step was taken: the checkpoint of step 0 is the current state
     lbm_status st = tape_before_step(dom);

@@ -43,17 +43,11 @@ lbm_status Domain::cuda_fail(cudaError_t e, const char* what) {
 void* Domain::dev_alloc(size_t bytes) {
   if (bytes == 0) bytes = 16;
   void* p = nullptr;
-  for (int attempt = 0; attempt < 2 && !p; ++attempt) {
-    if (attempt) {
-      if (tape_pool.empty()) break;
-      drop_tape_pool();
-    }
-    if (desc.alloc.alloc) {
-      p = desc.alloc.alloc(bytes, desc.alloc.ctx);
-    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      p = nullptr;
-    }
+  if (desc.alloc.alloc) {
+    p = desc.alloc.alloc(bytes, desc.alloc.ctx);
+  } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
   }
   if (p) allocs.push_back({p, bytes});
   return p;
@@ -72,32 +66,6 @@ void Domain::dev_free(void* p) {
       return;
     }
   }
-}
-
-void* Domain::tape_alloc(size_t bytes) {
-  for (size_t i = 0; i < tape_pool.size(); ++i)
-    if (tape_pool[i].second == bytes) {
-      void* p = tape_pool[i].first;
-      tape_pool[i] = tape_pool.back();
-      tape_pool.pop_back();
-      return p;
-    }
-  return dev_alloc(bytes);
-}
-
-void Domain::tape_free(void* p) {
-  if (!p) return;
-  for (const auto& a : allocs)
-    if (a.first == p) {
-      tape_pool.push_back(a);
-      return;
-    }
-}
-
-void Domain::drop_tape_pool() {
-  std::vector<std::pair<void*, size_t>> pool;
-  pool.swap(tape_pool);
-  for (const auto& a : pool) dev_free(a.first);
 }
 
 void* Domain::staging(size_t bytes) {

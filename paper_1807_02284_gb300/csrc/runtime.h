@@ -91,10 +91,6 @@ struct lbm_domain {
   std::string last_error;
   long long steps = 0;
   lbm::TapeState* tape = nullptr;
-  // buffers of the last released tape, for the next one (a rollout and its gradient take the
-  // same sizes again after every lbm_init_macro); given back by the first step without a tape,
-  // by lbm_set_tape(0), when an allocation fails, and with the domain
-  std::vector<std::pair<void*, size_t>> tape_pool;
   lbm::GraphCache* graphs = nullptr;
   void* batch_plan = nullptr;           // cached plans of lbm_step_batch (batch.cu)
   // scratch of lbm_reduce_batch when this domain heads the list (device and pinned host)
@@ -129,9 +125,6 @@ struct lbm_domain {
   lbm_status cuda_fail(cudaError_t e, const char* what);
   void* dev_alloc(size_t bytes);
   void dev_free(void* p);
-  void* tape_alloc(size_t bytes);       // dev_alloc, or a pooled buffer of this very size
-  void tape_free(void* p);              // into the pool
-  void drop_tape_pool();
   void* staging(size_t bytes);
   const void* device_source(const void* src, size_t bytes, int on_device, lbm_status* st);
   const void* stage_small(const void* src, size_t bytes, lbm_status* st);

@@ -160,7 +160,6 @@ void lbm_domain::release_extras() {
   if (aux_stream) cudaStreamDestroy(aux_stream);
   aux_stream = nullptr;
   release_tape(this);
-  drop_tape_pool();
   if (small_host) cudaFreeHost(small_host);
   small_host = nullptr;
   if (small_done) cudaEventDestroy(small_done);
@@ -301,7 +300,6 @@ lbm_status lbm_domain::advance(int n) {
     if (!post_stream((int)blocks.size())) return fail(LBM_ERR_CUDA, "cudaStreamCreate");
   }
   if (tape != nullptr) return advance_direct(n);
-  if (!tape_pool.empty()) drop_tape_pool();
   if (!graphs) {
     std::vector<int> start(blocks.size());
     for (size_t b = 0; b < blocks.size(); ++b) start[b] = blocks[b].cur;

@@ -87,3 +87,30 @@ def test_reverse_sweep_after_a_failed_allocation(lib, monkeypatch, blocks):
         fail += 1
         if fail == total:
             break
+
+
+@pytest.mark.parametrize("blocks", [1, 2])
+def test_a_released_tape_holds_no_memory(lib, blocks):
+    """lbm_init_macro releases the tape and with it all of its memory, whatever comes next (a step,
+    a batched step, another domain's rollout): nothing but the domain's own is held then."""
+    sc = _scene(blocks)
+    held = torch.cuda.memory_allocated
+    n = sc.blocks[0].flags.size
+    dc, g = torch.rand(n, device="cuda"), torch.empty(3 * n, device="cuda")
+    torch.cuda.synchronize()
+    d = _domain(sc)
+    d.step(1)
+    d.sync()
+    bare = held()
+    for every in (2, 3, 1):
+        for i, b in enumerate(sc.blocks):
+            d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0), block=i)
+        assert held() == bare
+        d.set_tape(every)
+        d.step(5)
+        assert held() > bare
+        d.adjoint_step(5, dc, g)
+        d.sync()
+    d.init_macro(f32(sc.blocks[0].u0))
+    assert held() == bare
+    d.close()
