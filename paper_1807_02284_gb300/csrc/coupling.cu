@@ -735,6 +735,7 @@ extern "C" lbm_status lbm_remove_scale_block(lbm_domain* dom, int32_t block_id) 
   const int child = dom->blocks.back().child;
   release_block(dom, dom->blocks.back());
   dom->blocks.pop_back();
+  dom->pick_tiles(0);       // a block alone may take another launch shape than one of several
   dom->invalidate_graphs();
   if (far) {   // the child's outer layer is again an open face
     Block& C = dom->blocks[child];
