@@ -234,7 +234,8 @@ lbm_status lbm_domain::advance_direct(int n) {
 
 // n reference steps as one graph launch, captured on the first such call from this level
 // assignment (`eager`), or on the second (a run that may never come again).  *done = false:
-// nothing was launched.
+// nothing was launched (a run that needs no graph is also left to the caller's launches on a stream
+// that cannot be captured, such as the legacy default stream).
 lbm_status lbm_domain::advance_graph(int n, bool eager, bool* done) {
   *done = false;
   std::vector<int> key(blocks.size());
@@ -251,6 +252,10 @@ lbm_status lbm_domain::advance_graph(int n, bool eager, bool* done) {
   if (!en->exec) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess && !eager) {
+      cudaGetLastError();
+      return LBM_OK;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
     lbm_status st = LBM_OK;
     for (int i = 0; i < n && st == LBM_OK; ++i) {

@@ -67,3 +67,23 @@ def test_step_under_the_callers_capture(lib):
         assert np.array_equal(x, y)
     d.close()
     ref.close()
+
+
+@pytest.mark.parametrize("runs", [(4, 4, 4), (3, 1, 3, 3, 20, 20)])
+def test_short_runs_on_a_stream_that_cannot_be_captured(lib, runs):
+    """cudaStreamLegacy (handle 1): no graph can be captured on it, the steps are launched."""
+    from paper_1807_02284_gb300 import lbm
+    sc = _scene()
+    b = sc.blocks[0]
+    d = lbm.Domain(b.dims, sc.nu, periodic=sc.periodic, stream=1, torch_allocator=False)
+    d.set_flags(b.flags)
+    d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0))
+    ref = gpu_domain(sc)
+    for n in runs:
+        d.step(n)
+    for _ in range(sum(runs)):
+        ref.step(1)
+    for x, y in zip(_fields(d), _fields(ref)):
+        assert np.array_equal(x, y)
+    d.close()
+    ref.close()
