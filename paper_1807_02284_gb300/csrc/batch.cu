@@ -322,6 +322,19 @@ static lbm_status step_batch(lbm_domain* const* doms, int32_t n, int32_t steps, 
   }
   if (steps == 0) return LBM_OK;
   cudaStream_t s = d0->stream;
+  // whole graphs, then the rest (with the diagnostics in its last step).  Both plans before the
+  // first launch: a call that cannot have them leaves every domain as it was.  (A whole graph ends
+  // in the levels it started from, so one plan serves all of them and the rest starts there too.)
+  const int rest_steps = (steps - 1) % kGraphSteps + 1, n_whole = (steps - rest_steps) / kGraphSteps;
+  BatchPlan *whole = nullptr, *p = nullptr;
+  if (n_whole > 0) {
+    const lbm_status st = batch_plan(doms, n, kGraphSteps, false, &whole);
+    if (st != LBM_OK) return st;
+  }
+  {
+    const lbm_status st = batch_plan(doms, n, rest_steps, red, &p);
+    if (st != LBM_OK) return st;
+  }
   // order the batch after pending work of every domain, and every domain after the batch
   std::vector<cudaEvent_t> evs;
   for (int i = 1; i < n; ++i) {
@@ -334,22 +347,17 @@ static lbm_status step_batch(lbm_domain* const* doms, int32_t n, int32_t steps, 
   }
   for (cudaEvent_t ev : evs) cudaEventDestroy(ev);
 
-  // whole graphs, then the rest (with the diagnostics in its last step)
-  BatchPlan* p = nullptr;
-  for (int left = steps; left > 0;) {
-    const int now = std::min(left, kGraphSteps);
-    const lbm_status st = batch_plan(doms, n, now, red && now == left, &p);
-    if (st != LBM_OK) return st;
-    const cudaError_t e = p->exec ? cudaGraphLaunch(p->exec, s) : enqueue_batch(doms, p, s);
-    if (e != cudaSuccess) return d0->cuda_fail(e, "batched launch");
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k <= n_whole && e == cudaSuccess; ++k) {
+    const BatchPlan* q = k < n_whole ? whole : p;
+    e = q->exec ? cudaGraphLaunch(q->exec, s) : enqueue_batch(doms, q, s);
+    if (e != cudaSuccess) break;
     for (int i = 0; i < n; ++i) {
       Block& B = doms[i]->blocks[0];
-      if (now & 1) B.cur ^= 1;
-      doms[i]->steps += now;
+      if (q->steps & 1) B.cur ^= 1;
+      doms[i]->steps += q->steps;
     }
-    left -= now;
   }
-  cudaError_t e = cudaSuccess;
   // every domain's stream waits for the batch (each node reports divergence into its own
   // domain's error word)
   cudaEvent_t done;
@@ -359,6 +367,7 @@ static lbm_status step_batch(lbm_domain* const* doms, int32_t n, int32_t steps, 
       if (doms[i]->stream != s) cudaStreamWaitEvent(doms[i]->stream, done, 0);
     cudaEventDestroy(done);
   }
+  if (e != cudaSuccess) return d0->cuda_fail(e, "batched launch");
   if (!red) {
     d0->post_error_probe();
     return LBM_OK;
