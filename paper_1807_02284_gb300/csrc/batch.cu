@@ -221,9 +221,27 @@ void release_batch_plan(lbm_domain* dom) {
   dom->batch_plan = nullptr;
 }
 
+// Captures the plan's launches, on a stream of the library's own: the members' stream may be one
+// that cannot be captured (the legacy default stream), the graph runs on any.
+static void capture_plan(lbm_domain* const* doms, BatchPlan* p) {
+  cudaStream_t s = doms[0]->post_stream(0);
+  cudaGraph_t g = nullptr;
+  if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    const cudaError_t e1 = enqueue_batch(doms, p, s);
+    const cudaError_t e2 = cudaStreamEndCapture(s, &g);
+    if (e1 == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&p->exec, g, 0) != cudaSuccess)
+      p->exec = nullptr;
+    if (g) cudaGraphDestroy(g);
+  }
+  cudaGetLastError();  // a capture the driver refused leaves the direct launches
+}
+
 // The plan of `steps` (at most kGraphSteps) steps from the members' current levels, from the
-// cache or captured now.
-static lbm_status batch_plan(lbm_domain* const* doms, int n, int steps, bool red, BatchPlan** out) {
+// cache or captured now.  `own`: the caller is capturing the members' stream itself, where no plan
+// is captured and none is kept (a call after the capture would find it without a graph): the plan
+// is left in *own for this call alone.
+static lbm_status batch_plan(lbm_domain* const* doms, int n, int steps, bool red, BatchPlan* own,
+                             BatchPlan** out) {
   lbm_domain* d0 = doms[0];
   BatchCache* cache = static_cast<BatchCache*>(d0->batch_plan);
   if (!cache) {
@@ -243,11 +261,12 @@ static lbm_status batch_plan(lbm_domain* const* doms, int n, int steps, bool red
       return LBM_OK;
     }
   }
-  // the fork's streams and events exist before the capture
+  // the fork's streams and events exist before a capture
   const int nb = std::min(n, kBatchStreams);
   if (!d0->event(nb)) return d0->fail(LBM_ERR_CUDA, "cudaEventCreate");
-  if (nb > 1 && !d0->post_stream(nb - 1)) return d0->fail(LBM_ERR_CUDA, "cudaStreamCreate");
-  BatchPlan* p = new (std::nothrow) BatchPlan();
+  if (!d0->post_stream(nb - 1)) return d0->fail(LBM_ERR_CUDA, "cudaStreamCreate");
+  const bool keep = !own || red;
+  BatchPlan* p = keep ? new (std::nothrow) BatchPlan() : own;
   if (!p) return d0->fail(LBM_ERR_OOM, "out of host memory");
   p->steps = steps;
   p->serials.resize(n);
@@ -256,10 +275,15 @@ static lbm_status batch_plan(lbm_domain* const* doms, int n, int steps, bool red
     p->serials[i] = doms[i]->serial;
     p->curs[i] = doms[i]->blocks[0].cur;
   }
+  if (!keep) {
+    *out = p;
+    return LBM_OK;
+  }
   if (red) {
     const lbm_status st = add_red_buffers(doms, n, p);
     if (st != LBM_OK) { free_plan(d0, p); return st; }
   }
+  capture_plan(doms, p);
   while (cache->plans.size() >= kMaxBatchPlans) {
     // a replaced plan's last launch may still be running; its buffers go back to the allocator
     if (cudaStreamSynchronize(d0->stream) != cudaSuccess) cudaGetLastError();
@@ -267,16 +291,6 @@ static lbm_status batch_plan(lbm_domain* const* doms, int n, int steps, bool red
     cache->plans.erase(cache->plans.begin());
   }
   cache->plans.push_back(p);
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(d0->stream, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    const cudaError_t e1 = enqueue_batch(doms, p, d0->stream);
-    const cudaError_t e2 = cudaStreamEndCapture(d0->stream, &g);
-    if (e1 == cudaSuccess && e2 == cudaSuccess && g && cudaGraphInstantiate(&p->exec, g, 0) != cudaSuccess)
-      p->exec = nullptr;
-    if (g) cudaGraphDestroy(g);
-  }
-  cudaGetLastError();  // a capture the driver refused leaves the direct launches
   *out = p;
   return LBM_OK;
 }
@@ -326,13 +340,16 @@ static lbm_status step_batch(lbm_domain* const* doms, int32_t n, int32_t steps, 
   // first launch: a call that cannot have them leaves every domain as it was.  (A whole graph ends
   // in the levels it started from, so one plan serves all of them and the rest starts there too.)
   const int rest_steps = (steps - 1) % kGraphSteps + 1, n_whole = (steps - rest_steps) / kGraphSteps;
-  BatchPlan *whole = nullptr, *p = nullptr;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+  const bool callers = cap != cudaStreamCaptureStatusNone;
+  BatchPlan own_whole, own_rest, *whole = nullptr, *p = nullptr;
   if (n_whole > 0) {
-    const lbm_status st = batch_plan(doms, n, kGraphSteps, false, &whole);
+    const lbm_status st = batch_plan(doms, n, kGraphSteps, false, callers ? &own_whole : nullptr, &whole);
     if (st != LBM_OK) return st;
   }
   {
-    const lbm_status st = batch_plan(doms, n, rest_steps, red, &p);
+    const lbm_status st = batch_plan(doms, n, rest_steps, red, callers ? &own_rest : nullptr, &p);
     if (st != LBM_OK) return st;
   }
   // order the batch after pending work of every domain, and every domain after the batch

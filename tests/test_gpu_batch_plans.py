@@ -59,3 +59,71 @@ def test_a_call_without_its_plan_leaves_the_members(lib, monkeypatch):
     _same(a, b)
     for d in a + b:
         d.close()
+
+
+def _runtime_calls(fn):
+    """CUDA runtime calls by name made in fn()."""
+    from torch.profiler import ProfilerActivity, profile
+
+    def counts(f):
+        with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as prof:
+            f()
+            torch.cuda.synchronize()
+        return {e.key: e.count for e in prof.key_averages()}
+
+    for _ in range(3):                    # a process's first profile can come back empty
+        if counts(lambda: torch.ones(4, device="cuda").add_(1)).get("cudaLaunchKernel"):
+            return counts(fn)
+    pytest.skip("no CUDA activity records")
+
+
+def test_batch_under_the_callers_capture(lib):
+    """A batch first called while the caller captures its stream is captured as launches, replays
+    to the same bits, and leaves no plan without a graph: the next calls replay graphs."""
+    from paper_1807_02284_gb300 import lbm
+    st = torch.cuda.Stream()
+    a, b = _members(5, [st]), _members(5, [st])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(st):
+        g.capture_begin(capture_error_mode="thread_local")
+        lbm.step_batch(a, 4)
+        g.capture_end()
+        for _ in range(2):
+            g.replay()
+    st.synchronize()
+    for d in b:
+        d.step(8)
+    _same(a, b)
+    lbm.step_batch(a, 4)                  # (a plan is captured here at the latest)
+    calls = _runtime_calls(lambda: lbm.step_batch(a, 4))
+    assert calls.get("cudaGraphLaunch", 0) == 1, calls
+    for d in b:
+        d.step(8)
+    _same(a, b)
+    for d in a + b:
+        d.close()
+
+
+def test_batch_on_a_stream_that_cannot_be_captured(lib):
+    """Members on cudaStreamLegacy (handle 1): their plan is a graph all the same."""
+    from paper_1807_02284_gb300 import lbm
+    scenes = synth.batch(count=3, seed=41, lo=8, hi=20, nu=2e-3)
+    a, b = [], [gpu_domain(s) for s in scenes]
+    for s in scenes:
+        k = s.blocks[0]
+        d = lbm.Domain(k.dims, s.nu, periodic=s.periodic, adaptive=s.adaptive, c_src=s.c_src,
+                       stream=1, torch_allocator=False)
+        d.set_flags(k.flags)
+        d.init_macro(f32(k.u0), rho=f32(k.rho0), c=f32(k.c0))
+        a.append(d)
+    lbm.step_batch(a, 4)
+    calls = _runtime_calls(lambda: lbm.step_batch(a, 4))
+    assert calls.get("cudaGraphLaunch", 0) == 1, calls
+    r = lbm.step_batch_reduce(a, 3)
+    for d in b:
+        d.step(11)
+    _same(a, b)
+    for x, d in zip(r, b):
+        assert abs(x[0] - d.reduce()[0]) <= 1e-6 * x[0]
+    for d in a + b:
+        d.close()
