@@ -336,54 +336,65 @@ cudaError_t launch_inflow_records(const void* rec, int n, uint8_t* flags, float*
 
 // ---- field conversion ------------------------------------------------------------------
 
-// Conversion between the stored deviation d = f - w and the population f.  With FP32 on the
-// caller's side the sum w + d is formed in float pairs (w = wh + wl to 48 bits, the exact
-// rounding error of wh + d added back with wl), which gives the nearest float of the exact
-// sum up to ties.  An FP64 add with its two conversions per value made these copies
-// 4.6 times slower than HBM: GB300's FP64 issue rate is a small fraction of FP32's
-// (reading a 256^3 state, 4.2 GB of populations, velocity and scalar: 2604 us with FP64 adds,
-// 614 us now; writing and reading 128^3 populations: 624 us before, 120 us now).
+// Conversion between the stored deviation d = f - w and the population f.  FP64 on the caller's
+// side takes an FP64 add.  FP32 on the caller's side gives the bits of the FP64 add rounded to
+// FP32, but forms the sum in floats: w = wh + wl exactly, s + e = wh + d exactly (two_sum), and
+// s + (e + wl) is rounded once.  What can still round the other way is a sum within the rounding
+// error of e + wl, or of FP64 itself, of a tie (nearest_sum): a node with such a value, one in
+// about 10^6, is converted again in FP64, out of line (as an inlined branch per value the
+// compiler evaluates the FP64 add for all).  FP64 for every value bounds the copies, not HBM:
+// GB300's FP64 issue rate is a small fraction of FP32's.
 template <int K>
 struct WeightPair {
   static constexpr float hi = (float)wkd(K);
   static constexpr float lo = (float)(wkd(K) - (double)hi);
+  static_assert((double)hi + (double)lo == wkd(K), "the pair holds the weight exactly");
 };
 
-// a + b = s + e exactly (Knuth's two-sum); e = 0 where s is infinite or NaN
+// a + b = s + e exactly (Knuth's two-sum; e is NaN where s is infinite or NaN)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  if (!(e == e)) e = 0.0f;
 }
 
+// The float nearest to the FP64 sum of s + e and the low part of w, t being e plus that part in
+// FP32: true when every sum within the margin of s + t rounds to it.  The margin covers the
+// rounding of t (2^-24 of it) and of the FP64 sum (2^-53 of s); with e = 0 neither rounds.
+__device__ __forceinline__ bool nearest_sum(float s, float e, float t, float& r) {
+  const float m = e == 0.0f ? 0.0f : __fmaf_rn(fabsf(t), 0x1p-22f, fabsf(s) * 0x1p-51f);
+  r = __fadd_rn(s, __fadd_rn(t, m));
+  return r == __fadd_rn(s, __fsub_rn(t, m));
+}
+
+// (`sure` is cleared where the value has to be formed in FP64)
 template <int K, typename O>
-__device__ __forceinline__ O population(float d) {
+__device__ __forceinline__ O population(float d, bool& sure) {
   if constexpr (sizeof(O) == 8) {
     return wkd(K) + (double)d;
   } else {
-    float s, e;
+    float s, e, r;
     two_sum(WeightPair<K>::hi, d, s, e);
-    return __fadd_rn(s, __fadd_rn(e, WeightPair<K>::lo));
+    sure &= nearest_sum(s, e, __fadd_rn(e, WeightPair<K>::lo), r);
+    return r;
   }
 }
 
-__device__ __forceinline__ void store_deviation(float* p, float s, float t) { *p = __fadd_rn(s, t); }
-// Half storage rounds s + t once: the float sum is rounded to odd first, so that the second
-// rounding sees on which side of a tie the exact sum lies.
-__device__ __forceinline__ void store_deviation(__half* p, float s, float t) {
+// Half storage rounds s + t once: the float sum is rounded to odd first (Boldo and Melquiond),
+// so that the second rounding sees on which side of a tie the exact sum lies.
+__device__ __forceinline__ __half half_sum(float s, float t) {
   float r, e;
   two_sum(s, t, r, e);
-  if (e != 0.0f && r != 0.0f) {
+  if (e != 0.0f && e == e && r != 0.0f) {
     int b = __float_as_int(r);
     if ((e > 0.0f) != (r > 0.0f)) b -= 1;     // r was rounded away from zero: truncate
     r = __int_as_float(b | 1);
   }
-  *p = __float2half_rn(r);
+  return __float2half_rn(r);
 }
 
 template <int K, typename T, typename I>
-__device__ __forceinline__ void put_deviation(T* p, I f) {
+__device__ __forceinline__ void put_deviation(T* p, I f, bool& sure) {
   if constexpr (sizeof(I) == 8) {
     const double dev = f - wkd(K);
     if constexpr (sizeof(T) == 2) *p = __double2half(dev);
@@ -391,26 +402,53 @@ __device__ __forceinline__ void put_deviation(T* p, I f) {
   } else {
     float s, e;
     two_sum(f, -WeightPair<K>::hi, s, e);
-    store_deviation(p, s, __fsub_rn(e, WeightPair<K>::lo));
+    if constexpr (sizeof(T) == 2) {
+      if (!(e == e)) e = 0.0f;                // infinities and NaN pass through s
+      *p = half_sum(s, __fsub_rn(e, WeightPair<K>::lo));
+    } else {
+      float r;
+      sure &= nearest_sum(s, e, __fsub_rn(e, WeightPair<K>::lo), r);
+      *p = r;
+    }
   }
 }
 
 // The 27 planes of one node, Q the caller's (paper) velocity index.
 template <int Q, typename T, typename O>
-__device__ __forceinline__ void read_planes(const float (&d)[27], size_t N, size_t idx, O* out) {
+__device__ __forceinline__ void read_planes(const float (&d)[27], size_t N, size_t idx, O* out,
+                                            bool& sure) {
   if constexpr (Q < 27) {
     constexpr int k = paper_to_cube(Q);
-    out[(size_t)Q * N + idx] = population<k, O>(d[k]);
-    read_planes<Q + 1, T, O>(d, N, idx, out);
+    out[(size_t)Q * N + idx] = population<k, O>(d[k], sure);
+    read_planes<Q + 1, T, O>(d, N, idx, out, sure);
   }
 }
 
 template <int Q, typename T, typename I>
-__device__ __forceinline__ void write_planes(const I (&f)[27], size_t N, size_t idx, T* d) {
+__device__ __forceinline__ void write_planes(const I (&f)[27], size_t N, size_t idx, T* d,
+                                             bool& sure) {
   if constexpr (Q < 27) {
     constexpr int k = paper_to_cube(Q);
-    put_deviation<k>(d + (size_t)k * N + idx, f[Q]);
-    write_planes<Q + 1, T, I>(f, N, idx, d);
+    put_deviation<k>(d + (size_t)k * N + idx, f[Q], sure);
+    write_planes<Q + 1, T, I>(f, N, idx, d, sure);
+  }
+}
+
+// One node again with FP64 adds.
+template <typename T>
+__device__ __noinline__ void read_node_f64(const T* d, size_t N, size_t idx, float* out) {
+#pragma unroll 1
+  for (int q = 0; q < 27; ++q) {
+    const int k = paper_to_cube(q);
+    out[(size_t)q * N + idx] = (float)(wkd(k) + (double)load_pop(d + (size_t)k * N + idx));
+  }
+}
+
+__device__ __noinline__ void write_node_f64(const float* in, size_t N, size_t idx, float* d) {
+#pragma unroll 1
+  for (int q = 0; q < 27; ++q) {
+    const int k = paper_to_cube(q);
+    d[(size_t)k * N + idx] = (float)((double)in[(size_t)q * N + idx] - wkd(k));
   }
 }
 
@@ -432,7 +470,10 @@ __global__ void __launch_bounds__(256) k_read_f(const T* __restrict__ d, size_t 
     float v[27];
 #pragma unroll
     for (int k = 0; k < 27; ++k) v[k] = load_pop(d + (size_t)k * N + idx);
-    read_planes<0, T, O>(v, N, idx, out);
+    bool sure = true;
+    read_planes<0, T, O>(v, N, idx, out, sure);
+    if constexpr (sizeof(O) == 4)
+      if (!sure) read_node_f64(d, N, idx, out);
   }
 }
 
@@ -444,7 +485,10 @@ __global__ void __launch_bounds__(256) k_write_f(T* __restrict__ d, size_t N,
     I v[27];
 #pragma unroll
     for (int q = 0; q < 27; ++q) v[q] = __ldg(in + (size_t)q * N + idx);
-    write_planes<0, T, I>(v, N, idx, d);
+    bool sure = true;
+    write_planes<0, T, I>(v, N, idx, d, sure);
+    if constexpr (sizeof(I) == 4 && sizeof(T) == 4)
+      if (!sure) write_node_f64(in, N, idx, d);
   }
 }
 

@@ -69,3 +69,67 @@ def test_velocity_and_scalar_copies(lib, dims, offset):
     d.read_field(lbm.LBM_FIELD_U, lbm.LBM_F32, out=out[offset:offset + 3 * n])
     assert torch.equal(out[offset:offset + 3 * n], src) and out[-1] == 0
     d.close()
+
+
+def _ties(read):
+    """Per weight, the values whose sum with (read) or difference from it lies next to a tie of
+    FP32, five floats to either side, over magnitudes around the weight; padded to one length."""
+    w = np.where(np.arange(27) == 0, 8 / 27, np.where(np.arange(27) < 7, 2 / 27,
+                 np.where(np.arange(27) < 19, 1 / 54, 1 / 216)))
+    rows = []
+    for q in range(27):
+        lo = w[q] - np.float64(np.float32(w[q]))
+        out = []
+        for ex in range(-10, 11):
+            u = np.float64(np.spacing(np.float32(w[q] * 2.0 ** ex)))
+            for x in list(u * np.arange(-3, 4)) + [w[q] * 2.0 ** ex, -w[q] * 2.0 ** ex]:
+                for h in (u / 2, -u / 2, u / 4, -u / 4):
+                    v = np.float32(x + h - lo if read else x + h + lo)
+                    for side in (np.inf, -np.inf):
+                        y = v
+                        for _ in range(5):
+                            out.append(y)
+                            y = np.nextafter(y, np.float32(side))
+        rows.append(np.array(out, np.float32))
+    return np.stack(rows), w[:, None]
+
+
+def _domain_of(lbm, n):
+    assert n % 8 == 0
+    return lbm.Domain((n // 8, 4, 2), 0.01)
+
+
+def test_fp32_reads_are_the_rounded_fp64_reads(lib):
+    """FP32 storage, deviations next to ties of the sum and random ones: the FP32 populations
+    are the FP64 ones rounded once, bit for bit."""
+    from paper_1807_02284_gb300 import lbm
+    dev, w = _ties(True)
+    rng = np.random.default_rng(6)
+    r = (w * rng.normal(size=(27, 1 << 14)) * 10.0 ** rng.uniform(-8, 1, size=(27, 1 << 14))).astype(np.float32)
+    dev = np.concatenate([dev, r], axis=1)
+    dev = np.pad(dev, ((0, 0), (0, -dev.shape[1] % 8)))
+    d = _domain_of(lbm, dev.shape[1])
+    d.write_field(lbm.LBM_FIELD_F, w + dev.astype(np.float64))
+    f64 = d.read_field(lbm.LBM_FIELD_F, lbm.LBM_F64)
+    f32 = d.read_field(lbm.LBM_FIELD_F, lbm.LBM_F32)
+    assert np.array_equal(f32.view(np.uint32), f64.astype(np.float32).view(np.uint32))
+    d.close()
+
+
+def test_fp32_writes_equal_fp64_writes(lib):
+    """The same floats handed over as FP32 and as FP64, next to ties of the difference, random and
+    special ones: the same stored deviations, bit for bit."""
+    from paper_1807_02284_gb300 import lbm
+    f, w = _ties(False)
+    rng = np.random.default_rng(7)
+    r = (w * (1 + rng.normal(size=(27, 1 << 14)) * 10.0 ** rng.uniform(-8, 1, size=(27, 1 << 14)))).astype(np.float32)
+    special = np.tile(np.array([np.inf, -np.inf, np.nan, 3e38, -3e38, 1e-45, 0.0, -0.0], np.float32), (27, 1))
+    f = np.concatenate([f, r, special, w.astype(np.float32)], axis=1)
+    f = np.pad(f, ((0, 0), (0, -f.shape[1] % 8)))
+    a, b = _domain_of(lbm, f.shape[1]), _domain_of(lbm, f.shape[1])
+    a.write_field(lbm.LBM_FIELD_F, f)
+    b.write_field(lbm.LBM_FIELD_F, f.astype(np.float64))
+    fa, fb = (d.read_field(lbm.LBM_FIELD_F, lbm.LBM_F64) for d in (a, b))
+    assert np.array_equal(fa, fb, equal_nan=True)
+    a.close()
+    b.close()
