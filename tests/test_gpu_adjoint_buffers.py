@@ -114,3 +114,33 @@ def test_a_released_tape_holds_no_memory(lib, blocks):
     d.init_macro(f32(sc.blocks[0].u0))
     assert held() == bare
     d.close()
+
+
+@pytest.mark.parametrize("blocks", [1, 2])
+def test_gradients_do_not_depend_on_what_the_memory_held(lib, blocks):
+    """Checkpoint intervals changed from rollout to rollout on one domain, its buffers taken from
+    memory full of NaN: the gradient of a fresh domain each time.  Bound: as above."""
+    sc = _scene(blocks)
+    n = sc.blocks[0].flags.size
+    dc = torch.rand(n, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+
+    def rollout(d, every):
+        for i, b in enumerate(sc.blocks):
+            d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0), block=i)
+        dirty = [torch.full((1 << 22,), float("nan"), device="cuda") for _ in range(4)]
+        torch.cuda.synchronize()
+        del dirty
+        g = torch.empty(3 * n, device="cuda")
+        d.set_tape(every)
+        d.step(5)
+        d.adjoint_step(5, dc, g)
+        d.sync()
+        return g.cpu().numpy().astype(np.float64)
+
+    d = _domain(sc)
+    for every in (2, 5, 1, 3, 2):
+        fresh = _domain(sc)
+        ref = rollout(fresh, every)
+        fresh.close()
+        assert np.isfinite(ref).all() and rel(rollout(d, every), ref) <= 1e-5, every
+    d.close()

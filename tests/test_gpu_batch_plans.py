@@ -127,3 +127,27 @@ def test_batch_on_a_stream_that_cannot_be_captured(lib):
         assert abs(x[0] - d.reduce()[0]) <= 1e-6 * x[0]
     for d in a + b:
         d.close()
+
+
+@pytest.mark.parametrize("streams", [1, 3])
+@pytest.mark.parametrize("steps", [17, 20])
+def test_more_members_than_branches_with_diagnostics(lib, streams, steps):
+    """40 members share 32 branches; a whole 16-step graph and its rest: the states of single
+    steps bit for bit, the diagnostics those of lbm_step_reduce (the same records, summed in FP64:
+    1e-13 of the sums' sizes), for both forms of the call and from both levels."""
+    from paper_1807_02284_gb300 import lbm
+    a, b = (_members(40, [torch.cuda.Stream() for _ in range(streams)], lo=6, hi=14) for _ in range(2))
+    out = torch.zeros((40, 5), dtype=torch.float64, pin_memory=True)
+    for k in range(3):
+        if k == 1:
+            a[0].wait_results(lbm.step_batch_reduce_async(a, steps, out))
+            r = out.numpy()
+        else:
+            r = lbm.step_batch_reduce(a, steps)
+        for d, x in zip(b, r):
+            y = d.step_reduce(steps)
+            n = d.n_nodes()
+            assert np.abs(x - y).max() <= 1e-13 * n
+        _same(a, b)
+    for d in a + b:
+        d.close()

@@ -35,3 +35,29 @@ def test_removing_the_last_block_restores_the_shape(lib, storage, kind):
     assert _shape(d) == alone
     d.close()
     fresh.close()
+
+
+def test_steps_after_a_block_was_removed(lib):
+    """A domain that had a refined and then a far-field block steps like one that never had."""
+    import numpy as np
+    from paper_1807_02284_gb300 import lbm
+    from tests.helpers import f32, gpu_domain
+    sc = synth.random_scene(dims=(36, 30, 28), seed=4, periodic=(False,) * 3, nu=0.01,
+                            spheres=[(18.0, 15.0, 14.0, 4.0)])
+    b = sc.blocks[0]
+    d, ref = gpu_domain(sc), gpu_domain(sc)
+    k = d.add_scale_block((4.0, 4.0, 4.0), 0.5, (12, 12, 12))
+    d.step(3)
+    d.remove_scale_block(k)
+    fb = synth.far_block(b, 2.0, 8.0, seed=9)
+    k = d.add_scale_block(fb.origin, fb.h, fb.dims)
+    d.step(2)
+    d.remove_scale_block(k)
+    d.init_macro(f32(b.u0), rho=f32(b.rho0), c=f32(b.c0))
+    for n in (5, 5, 20, 1):
+        d.step(n)
+        ref.step(n)
+    for f in (lbm.LBM_FIELD_F, lbm.LBM_FIELD_U, lbm.LBM_FIELD_SCALAR):
+        assert np.array_equal(d.read_field(f, lbm.LBM_F32), ref.read_field(f, lbm.LBM_F32))
+    d.close()
+    ref.close()

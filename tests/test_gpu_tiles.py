@@ -65,3 +65,46 @@ def test_pairs_with_ghost_and_obstacle_nodes_equal_single_nodes(lib, monkeypatch
         dom.close()
     for o in out[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(out[0], o))
+
+
+def _terms(d):
+    """Per-node terms of the five diagnostics of the stored state in 64 bits (5, nodes): rho - 1,
+    j, |j|^2 / (2 rho), over the nodes that count."""
+    from paper_1807_02284_gb300 import lbm
+    from oracle.cmr import C
+    f = d.read_field(lbm.LBM_FIELD_F, lbm.LBM_F64).reshape(27, -1)
+    fl = d.read_field(lbm.LBM_FIELD_FLAGS, lbm.LBM_U8).reshape(-1)
+    keep = (fl & (synth.SOLID | synth.GHOST)) == 0
+    rho = f.sum(0)
+    j = np.einsum("qn,qa->an", f, np.asarray(C, dtype=np.float64))
+    return np.concatenate([(rho - 1.0)[None], j, (0.5 * (j * j).sum(0) / rho)[None]])[:, keep], keep.sum()
+
+
+@pytest.mark.parametrize("dims", [(31, 5, 3), (34, 7, 5), (96, 3, 2), (130, 16, 12)])
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_every_diagnostic_within_its_own_terms(lib, monkeypatch, dims, storage):
+    """lbm_step_reduce of every shape, bounce-back obstacle and inflow included: each of mass,
+    momentum and energy against the 64-bit sums of the stored state, bounded by its own terms.  A
+    term is taken before the collision, which conserves it to the rounding of some 40 operations on
+    moments of at most a tenth (2^-22 of the node's weight of 1); a CTA's sum takes at most 256
+    additions (256 * 2^-24 of the terms' magnitudes); FP16 storage is rounded after the sums are
+    taken, 2^-11 of deviations of at most a tenth of each weight."""
+    from paper_1807_02284_gb300 import lbm
+    spheres = [(dims[0] / 2, dims[1] / 2, dims[2] / 2, 1.2)] if min(dims) > 2 else ()
+    sc = synth.random_scene(dims=dims, seed=33, periodic=(False, False, True), nu=0.01, spheres=spheres)
+    for tile in ("", "32,8,3", "64,1,4", "128,1,4", "64,2,20", "128,1,21"):
+        if tile:
+            monkeypatch.setenv("LBM_TILE", tile)
+        else:
+            monkeypatch.delenv("LBM_TILE", raising=False)
+        d = gpu_domain(sc, storage)
+        d.step(2)
+        diag = d.step_reduce(1)
+        t, n = _terms(d)
+        d.close()
+        per_node = 2.0 ** -22 if storage == "fp32" else 2.0 ** -22 + 0.1 * 2.0 ** -11
+        u = np.sqrt((t[1:4] ** 2).sum(0)).max()
+        exact, size = t.sum(1), np.abs(t).sum(1)
+        exact[0] += n
+        node = np.array([1, 1, 1, 1, 2 * u]) * per_node * n
+        assert np.all(np.abs(diag - exact) <= 256 * 2.0 ** -24 * size + node), (tile, diag, exact)
