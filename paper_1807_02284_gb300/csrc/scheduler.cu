@@ -45,31 +45,38 @@ static std::vector<int> next_levels(const std::vector<lbm::Block>& blocks, std::
 }
 }  // namespace lbm
 
-// Launch shape of a block's collide-stream kernel, from its extents and storage.  Figures: us per
-// step of fluid blocks on GB300, every shape and register bound tried at each size.
+// Launch shape of a block's collide-stream kernel, from its extents, storage and walls.  Figures:
+// us per step on GB300, one node per thread / two.
 void lbm_domain::pick_tiles(int b) {
   Block& B = blocks[b];
   if (B.tile_forced) return;
   const bool half = desc.storage == LBM_FP16_SHIFTED;
-  // walls and refined scales: warps with wall nodes take the node-wise path, and the step runs
-  // beside other blocks' kernels, so pairs pay only from 4 M nodes (196 x 98 x 98 with
-  // obstacle-surface walls 86 us with one node per thread, 100 with two; 128^3 under two refined
-  // scales 112 against 130; 256^3 inside a far-field block 740 against 722, with
-  // obstacle-surface walls 669 with two)
-  const size_t pairs_from = (size_t)1 << (walls || blocks.size() > 1 ? 22 : 20);
+  // Two nodes per thread once the block is bound by bandwidth or issue rather than by latency:
+  // from 2^20 nodes (96^3 40.8 / 42.5, FP16 40.0 / 41.2; 128^3 91 / 84, FP16 96 / 80; 256^3 702 /
+  // 629, FP16 718 / 592).  Beside other blocks' kernels or with wall faces from 2^22 (steps of a
+  // domain with a refined block: 128^3 148 / 152, 150^3 209 / 212, 160^3 235 / 234, 176^3 294 /
+  // 286, 192^3 356 / 343; in a far-field block the two are within 1 % from 144^3 to 192^3; wall
+  // faces: 128^3 97 / 97, 160^3 182 / 180, 176^3 243 / 232, 192^3 307 / 288).  With
+  // obstacle-surface walls from 2^24: a warp that holds a surface node goes through the collision
+  // three times, and with two nodes per thread twice as many nodes go with it, so it depends on
+  // the surface (sphere of radius 0.15 edges: 128^3 95 / 116, 176^3 243 / 278, 224^3 487 / 547,
+  // 256^3 716 / 740, 320^3 1386 / 1419, 384 x 256 x 384 1600 / 1528; 0.09 edges: 160^3 180 / 192,
+  // 192^3 304 / 302, 256^3 709 / 686, 320^3 1371 / 1283; FP16 alike).
+  const bool surfaces = (walls & WALLS_OBSTACLES) && !B.far;
+  const size_t pairs_from = (size_t)1 << (surfaces ? 24 : walls || blocks.size() > 1 ? 22 : 20);
   if (B.nx % 2 == 0 && B.N >= pairs_from) {
-    // two nodes per thread once the block is bound by bandwidth or issue rather than by
-    // latency: from 1 M nodes (96^3 FP32 42.5 against 40.8 us with one node per thread, FP16 41.2
-    // against 40.0; 128^3 84 against 91, FP16 80 against 96; 256^3 629 against 702, FP16 592
-    // against 718).  Tiles of 64 x 2 nodes on whole rows, one-row CTAs running on over ragged
-    // ones (224 x 250 x 190 FP32 410 us against 431 with 64 x 2 tiles, FP16 386 against 428).
+    // tiles of 64 x 2 nodes on whole rows, one-row CTAs running on over ragged ones (two nodes per
+    // thread, 224 x 250 x 190: FP32 410 us against 431 with 64 x 2 tiles, FP16 386 against 428)
     const bool tiles = B.nx % 64 == 0;
     B.bx = tiles ? 64 : 128;
     B.by = tiles ? 2 : 1;
     B.minb = STEP_PAIR + (half ? 5 : 4);
   } else if (B.nx <= 32) {
     // latency-bound: a warp per row keeps the faces in warps of their own, 80 registers take
-    // cell_update's EARLY loads (24^3 2.9 us against 4.0 with one-row CTAs, 32^3 3.5 against 3.8)
+    // cell_update's EARLY loads (12^3 3.8 us against 4.6 with one-row CTAs, 20^3 3.6 against 4.6,
+    // 24^3 2.9 against 4.0, 32^3 3.5 against 3.8, 28 x 60 x 60 6.7 against 7.7; not on larger
+    // blocks of shorter rows, whose idle lanes count: 12 x 60 x 60 6.3 against 5.1,
+    // 16 x 128 x 128 21.5 against 12.9)
     B.bx = 32;
     B.by = 4;
     B.minb = 3;

@@ -61,3 +61,16 @@ def test_steps_after_a_block_was_removed(lib):
         assert np.array_equal(d.read_field(f, lbm.LBM_F32), ref.read_field(f, lbm.LBM_F32))
     d.close()
     ref.close()
+
+
+@pytest.mark.parametrize("dims,faces,obstacles,nodes", [
+    ((176, 160, 152), False, False, 2), ((176, 160, 152), True, False, 2),
+    ((176, 160, 152), False, True, 1), ((176, 160, 152), True, True, 1),
+    ((256, 256, 256), True, True, 2), ((128, 96, 96), True, False, 1)])
+def test_nodes_per_thread_with_walls(lib, dims, faces, obstacles, nodes):
+    """Pairs from 2^20 nodes, with wall faces from 2^22, with obstacle-surface walls from 2^24."""
+    from paper_1807_02284_gb300 import lbm
+    d = lbm.Domain(dims, 0.01, storage="fp16")
+    d.set_walls((0, 0, 0, 0, 1, 1) if faces else (0,) * 6, obstacles=obstacles)
+    assert d.info().nodes_per_thread == nodes
+    d.close()
