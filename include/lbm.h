@@ -316,8 +316,8 @@ lbm_status lbm_reduce(lbm_domain* dom, int32_t block_id, double out[5]);
 /* n >= 1 reference steps (as lbm_step) followed by the lbm_reduce diagnostics of block 0's
    new state, in one call.  On a single-block domain with 27 N < 2^32 the last step's kernel
    sums the moments of the state it stores while storing it (collision conserves rho and j,
-   so a fluid node's are those of its pulled populations; per CTA in FP32 within a warp and
-   FP64 across warps, then a fixed-order FP64 sum): no second pass over the populations.
+   so a fluid node's are those of its pulled populations; FP32 within a CTA, then a
+   fixed-order FP64 sum): no second pass over the populations.
    The values agree with lbm_reduce of the same state to FP32 rounding of the per-node terms
    (with FP16-shifted storage they are those of the FP32 state before it is rounded for
    storage); the stored state is the one lbm_step writes.  Other domains take the steps and
@@ -494,8 +494,9 @@ lbm_status lbm_step_batch_reduce(lbm_domain* const* doms, int32_t n, int32_t ste
 lbm_status lbm_step_batch_reduce_async(lbm_domain* const* doms, int32_t n, int32_t steps,
                                        double* out, int64_t* ticket);
 
-/* Self-test of the library's bounded device-wide barrier (no counterpart in the paper):
-   launches a small cooperative kernel whose barrier waits for `extra` CTAs that do not exist, so every wait expires after about limit_ms (0 < limit_ms <= 5000).  Returns
+/* Self-test of a bounded device-wide barrier (no counterpart in the paper; no other entry point
+   uses one): launches a small cooperative kernel whose barrier waits for `extra` CTAs that do
+   not exist, so every wait expires after about limit_ms (0 < limit_ms <= 5000).  Returns
    LBM_ERR_TIMEOUT when the bounded wait gave up and reported it (extra > 0), LBM_OK when
    the barrier completed (extra = 0); the CUDA context stays usable either way. */
 lbm_status lbm_barrier_selftest(int32_t extra, double limit_ms, void* cuda_stream);

@@ -1185,7 +1185,8 @@ static BlockView view_of(lbm_domain* dom, const Level& from, const Level& to) {
 // level per block.  Bound by DRAM for large levels, by the launches for small ones: three
 // blocks of 64^3, 48^3, 32^3 took 49 copies and 49 memsets per rollout and gradient of two
 // steps, 268 us of device time and a call each on the host (now 19 launches, 160 us; 2755 ->
-// 2471 us as a whole).  One grid row per array, four 16-byte words in flight per thread (arrays off 16 bytes: one float at a time).
+// 2471 us as a whole).  One grid row per array, four 16-byte words in flight per thread (arrays
+// off 16 bytes: one float at a time).
 struct Pieces {
   static constexpr int MAX = 12;
   float* dst[MAX];
@@ -1635,9 +1636,9 @@ static lbm_status alloc_sweep(lbm_domain* dom, TapeState* t, const std::vector<i
 // to first; each segment between checkpoints is replayed once to record every step's start
 // state, and each step once more from there, keeping a version of every value that its
 // operations read (MsOp), before the operations are reversed one after another.  (Replaying
-// the operations before each one from the step's start took K (K + 1) / 2 operations and K
+// the operations before each one from the step's start would take K (K + 1) / 2 operations and K
 // copies of every block for K operations per step, 120 and 48 for a three-block domain of 1/1.5
-// and 1/2.25: a domain of 64^3, 48^3 and 32^3 nodes over two steps 7.6 -> 3.3 ms.)
+// and 1/2.25; a domain of 64^3, 48^3 and 32^3 nodes over two steps, that alone: 7.6 -> 3.3 ms.)
 static lbm_status adjoint_multiblock(lbm_domain* dom, int n_steps, const float* dL_dc,
                                      const float* dL_du, float* dL_du0, float* dL_dinflow) {
   TapeState* t = dom->tape;

@@ -4,16 +4,16 @@
 // in the last step), with the launch shape its size calls for; the members' steps are forked
 // over a few streams, balanced by their nodes, and the whole call is captured in a CUDA graph.
 // Members do not depend on one another, so while one member's last CTAs drain, the other
-// branches' launches fill the SMs, and no step waits for the slowest member.  Measured against
-// one persistent cooperative kernel over a joint chunk list with a device-wide barrier per
-// step (128 registers, since a member's view came from memory instead of the constant bank;
-// one node per thread): 64 plumes of edges 24 to 96, 1.34 -> 0.98 ms per step, and no timing
-// launches at a set's first call (57 -> 24 ms).
+// branches' launches fill the SMs, and no step waits for the slowest member: one persistent
+// kernel over all members with a device-wide barrier per step did, and held 128 registers, since
+// a member's view came from memory instead of the constant bank (64 plumes of edges 24 to 96,
+// uploads, diagnostics and reads: 31.2 ms a pass against 21.7; a new set's first call 57 against
+// 23 ms).
 // Every node runs the same cell_update as a domain stepped on its own, so results are
 // bit-identical to that.
 //
 // The bounded device-wide barrier below (a wait that expires sets the TIMEOUT bit instead of
-// hanging the GPU) is kept with its self-test.
+// hanging the GPU) is used by its self-test alone; no step waits on the device.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -4,8 +4,8 @@
 
 namespace lbm {
 
-// MINB: CTAs of 256 threads per SM the registers are bounded for (3: 80 registers, no
-// spills; 4: 64 registers with a small spill, more loads in flight); pick_tiles chooses.
+// MINB: CTAs of 256 threads per SM the registers are bounded for (3: 80 registers; 4: 64
+// registers, more warps in flight; no spills but 4 bytes of FP16 at 64); pick_tiles chooses.
 template <typename T, typename IT, bool ALIGN, int MINB, bool WALLS, bool LINEAR>
 __global__ void __launch_bounds__(256, MINB) k_step(BlockView v) {
   int x, y;
@@ -15,7 +15,8 @@ __global__ void __launch_bounds__(256, MINB) k_step(BlockView v) {
 }
 
 // Two nodes (x, x + 1) per thread, x = 2 (thread's column): MINB CTAs of at most 128 threads
-// per SM (128 registers per thread at 4; 96 at 5 and 80 at 6, with small spills).
+// per SM (128 registers per thread at 4 and, for FP16, 96 at 5 without spills; FP32 at 5 and
+// either at 6 spill).
 template <typename T, typename IT, int MINB, bool WALLS, bool LINEAR>
 __global__ void __launch_bounds__(128, MINB) k_step2(BlockView v) {
   int x, y;

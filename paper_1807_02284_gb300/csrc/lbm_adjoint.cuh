@@ -7,10 +7,9 @@
 // whatever the other axes do.  So the adjoint of u over all three axes needs one set of
 // moments at each end of the collision (the post-collision raw ones, the pre-collision
 // central ones) and 18 multiply-adds per axis and end, instead of every intermediate stage of
-// every sweep (the stages cost three relaxations and six inverse sweeps more; together with
-// the reverse-mode equilibrium below, against forward-mode dual numbers with four partials:
-// the reverse step's pass A at 128^3 272 -> 245 us, at 72 x 60 x 51 with open faces 76 -> 64 us,
-// the transposed mappings of a 64^3 three-block domain 50 -> 43 us per launch).
+// every sweep, which would take three relaxations and six inverse sweeps more.  The equilibrium
+// offsets are differentiated in reverse, not with dual numbers of four partials.  (Both
+// together, all else equal: pass A at 128^3 272 -> 245 us.)
 #pragma once
 #include "lbm_device.cuh"
 

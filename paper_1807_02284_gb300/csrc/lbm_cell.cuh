@@ -12,8 +12,8 @@ namespace lbm {
 // plane, or (LINEAR, one-row CTAs) take consecutive columns of the plane in x-fastest order,
 // running on into the next rows, so that no lane idles when nx is not a multiple of the CTA.
 // False for threads past the end.  A separate instance: the column of a linear thread comes
-// out of a division and is held (a few spills, 2 % on whole rows), a tile's is recomputed from
-// the thread index.
+// out of a division and is held (2 % on whole rows), a tile's is recomputed from the thread
+// index.
 template <bool LINEAR>
 __device__ __forceinline__ bool thread_column(int nx, int ny, int& x, int& y) {
   if constexpr (LINEAR) {
@@ -433,9 +433,9 @@ __device__ __forceinline__ void cell_update(const BlockView& v, int x, int y, in
 
 
 // ---- two nodes per thread (k_step2): nodes x and x + 1 of one row, x even, nx even, so that
-// their stored values are aligned pairs.  The pair path covers inner_yz fluid nodes without
-// bounce-back, walls or inflow (almost all nodes of a block); any other pair takes
-// cell_update node by node.  Every value equals cell_update's for the same node: the loads,
+// their stored values are aligned pairs.  The pair path covers inner_yz nodes without walls or
+// inflow (almost all nodes of a block; obstacle voxels, scale-boundary nodes and nodes next to an
+// obstacle are among them); any other pair takes cell_update node by node.  Every value equals cell_update's for the same node: the loads,
 // the lane arithmetic (float2 forms of the same rounded operations) and the stores are the
 // per-node ones, only issued two at a time.
 
@@ -535,9 +535,9 @@ __device__ __forceinline__ float scalar_value_slots(const BlockView& v, int x, i
 
 // FP16 storage takes the scalar corners through shared memory: its pair kernel is bound by
 // the registers that hold loads in flight (occupancy), and without the corners' 22 live
-// registers it runs at 5 CTAs per SM without spills (256^3 plume: 26.7 -> 27.4 GLUPS).  The
-// FP32 pair kernel is bound by DRAM bandwidth and runs faster with the corners in registers
-// (24.9 against 23.8 GLUPS).
+// registers it runs at 5 CTAs per SM without spills (256^3 plume, the corners alone changed:
+// 26.7 -> 27.4 GLUPS).  The FP32 pair kernel is bound by DRAM bandwidth and runs faster with the
+// corners in registers (24.9 against 23.8 GLUPS).
 template <typename T>
 constexpr bool pair_corners_async() { return sizeof(T) == 2; }
 

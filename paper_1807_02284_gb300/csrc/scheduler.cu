@@ -300,9 +300,11 @@ lbm_status lbm_domain::advance_graph(int n, bool eager, bool* done) {
 // Without a tape: whole chunks from chunk graphs; the rest of a continuous-scale domain step by
 // step from one-step graphs (the schedule of one step is 16 launches with forks and joins on
 // several streams; replaying it as one graph leaves the GPU no gaps between them), the rest
-// of a small single block (a step shorter than its launch takes the host: 3.8 us against
-// about 7 on a 32^3 block) from a graph of its length once it has come twice, of a larger one
-// launch by launch.
+// of a small single block (up to 2^18 nodes, 3 steps or more) from a graph of its length once it
+// has come twice, of a larger one launch by launch.  A graph has smaller gaps between steps and
+// one call for the host: 4 steps one after another 32^3 30.5 -> 24.1 us, 64^3 62.6 -> 53.4.  The
+// limit is no crossover: larger blocks gain less but gain too (80^3 122.7 -> 112.6, 96^3 181.5 ->
+// 172.6, 128^3 357 -> 347); it keeps the graphs of every run length to blocks where they matter.
 lbm_status lbm_domain::advance(int n) {
   if (blocks.size() > 1) {  // stream and events of the fork/join schedule exist before capture
     cudaStream_t a = nullptr;

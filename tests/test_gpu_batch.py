@@ -1,6 +1,6 @@
-"""Batched persistent stepping (one cooperative launch per call over the joint work list of
-many domains of uneven sizes): bit-identical to stepping each domain alone, parity with the
-oracle, and the bounded device barrier reporting a timeout instead of hanging."""
+"""Batched stepping (every member's own launches on forked branches of one graph, many domains
+of uneven sizes): bit-identical to stepping each domain alone, parity with the oracle, and the
+bounded device barrier reporting a timeout instead of hanging."""
 import numpy as np
 import pytest
 
