@@ -897,7 +897,7 @@ def run_batch(args):
                         "blocking_value": N * E * ws / t_sync / 1e6,
                         "blocking_api": "per step: lbm_set_inflow_batch + "
                                         "lbm_step_batch_reduce(1, host)"},
-                "gpu_launches": 1, "clocks": clk}
+                "gpu_launches": K * len(mine), "clocks": clk}
         print(json.dumps(line), flush=True)
     for d in doms:
         d.close()
@@ -1252,6 +1252,20 @@ def run_slab(args, emit=True):
     return out
 
 
+def _five_digits(x):
+    if isinstance(x, dict):
+        return {k: _five_digits(v) for k, v in x.items()}
+    if isinstance(x, list):
+        return [_five_digits(v) for v in x]
+    return float("%.5g" % x) if isinstance(x, float) else x
+
+
+def _rates_only(x):
+    """A nested record without its series."""
+    return {k: _rates_only(v) if isinstance(v, dict) else v for k, v in x.items()
+            if not isinstance(v, list)}
+
+
 def _variants(args):
     """Measured summaries of the other hot-path variants for the default bench line."""
     import copy
@@ -1278,10 +1292,14 @@ def _variants(args):
             with redirect_stdout(buf):
                 fn(a)
             d = json.loads(buf.getvalue().strip().splitlines()[-1])
-            res[name] = {k: d[k] for k in ("value", "unit", "ms_per_step", "roofline", "e2e",
-                                           "forward_with_tape_mlups", "config", "detect",
-                                           "ringing")
-                         if k in d}
+            # (the whole record, spectra included, is that workload's own line: this one is read
+            # by programs that keep a few KB of it)
+            if "ringing" in d:
+                d["ringing"] = _rates_only(d["ringing"])
+            res[name] = _five_digits({k: d[k] for k in ("value", "unit", "ms_per_step", "roofline",
+                                                        "e2e", "forward_with_tape_mlups", "config",
+                                                        "detect", "ringing")
+                                      if k in d})
         except Exception as ex:  # report, do not hide
             res[name] = {"error": f"{type(ex).__name__}: {ex}"}
     return res

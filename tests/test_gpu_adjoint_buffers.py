@@ -13,20 +13,30 @@ pytestmark = pytest.mark.gpu
 
 
 class Allocations:
-    """Counts the library's device allocations; number `fail_at` fails (the caller's allocator
-    raises, the library gets NULL)."""
+    """Counts the library's device allocations and what they hold; number `fail_at` fails (the
+    caller's allocator raises, the library gets NULL)."""
 
     def __init__(self, monkeypatch):
-        self.count, self.fail_at = 0, -1
-        real = torch.cuda.caching_allocator_alloc
+        self.count, self.fail_at, self.live = 0, -1, {}
+        real, real_free = torch.cuda.caching_allocator_alloc, torch.cuda.caching_allocator_delete
 
         def alloc(nbytes, device=None, stream=None):
             self.count += 1
             if self.count - 1 == self.fail_at:
                 raise RuntimeError("no memory")
-            return real(nbytes, device, stream)
+            p = real(nbytes, device, stream)
+            self.live[p] = nbytes
+            return p
+
+        def free(p):
+            self.live.pop(p, None)         # (None: taken before this test)
+            real_free(p)
 
         monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", alloc)
+        monkeypatch.setattr(torch.cuda, "caching_allocator_delete", free)
+
+    def held(self):
+        return sum(self.live.values())
 
 
 def _scene(blocks):
@@ -90,11 +100,11 @@ def test_reverse_sweep_after_a_failed_allocation(lib, monkeypatch, blocks):
 
 
 @pytest.mark.parametrize("blocks", [1, 2])
-def test_a_released_tape_holds_no_memory(lib, blocks):
+def test_a_released_tape_holds_no_memory(lib, monkeypatch, blocks):
     """lbm_init_macro releases the tape and with it all of its memory, whatever comes next (a step,
     a batched step, another domain's rollout): nothing but the domain's own is held then."""
     sc = _scene(blocks)
-    held = torch.cuda.memory_allocated
+    held = Allocations(monkeypatch).held
     n = sc.blocks[0].flags.size
     dc, g = torch.rand(n, device="cuda"), torch.empty(3 * n, device="cuda")
     torch.cuda.synchronize()
