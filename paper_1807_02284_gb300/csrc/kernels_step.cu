@@ -342,7 +342,7 @@ cudaError_t launch_inflow_records(const void* rec, int n, uint8_t* flags, float*
 // FP32, but forms the sum in floats: w = wh + wl exactly, s + e = wh + d exactly (two_sum), and
 // s + (e + wl) is rounded once.  What can still round the other way is a sum within the rounding
 // error of e + wl, or of FP64 itself, of a tie (nearest_sum): a node with such a value, one in
-// about 10^6, is converted again in FP64, out of line (as an inlined branch per value the
+// some 10^4, is converted again in FP64, out of line (as an inlined branch per value the
 // compiler evaluates the FP64 add for all).  FP64 for every value bounds the copies, not HBM:
 // GB300's FP64 issue rate is a small fraction of FP32's.
 template <int K>
@@ -360,12 +360,13 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 }
 
 // The float nearest to the FP64 sum of s + e and the low part of w, t being e plus that part in
-// FP32: true when every sum within the margin of s + t rounds to it.  The margin covers the
-// rounding of t (2^-24 of it) and of the FP64 sum (2^-53 of s); with e = 0 neither rounds.
-__device__ __forceinline__ bool nearest_sum(float s, float e, float t, float& r) {
-  const float m = e == 0.0f ? 0.0f : __fmaf_rn(fabsf(t), 0x1p-22f, fabsf(s) * 0x1p-51f);
-  r = __fadd_rn(s, __fadd_rn(t, m));
-  return r == __fadd_rn(s, __fsub_rn(t, m));
+// FP32: true unless the remainder q = s + t - r (exact: s is 0 or exceeds t) comes within 2^-18
+// of half an ulp of r.  The rounding of t (2^-24 of it, and t is at most about two ulps of s
+// where e is not 0) and of the FP64 sum (2^-53) are less than that; with e = 0 neither rounds.
+__device__ __forceinline__ bool nearest_sum(float s, float t, float& r) {
+  r = __fadd_rn(s, t);
+  const float q = __fsub_rn(t, __fsub_rn(r, s));
+  return __fmaf_rn(q, 0x1.00004p0f, r) == r;
 }
 
 // (`sure` is cleared where the value has to be formed in FP64)
@@ -376,7 +377,7 @@ __device__ __forceinline__ O population(float d, bool& sure) {
   } else {
     float s, e, r;
     two_sum(WeightPair<K>::hi, d, s, e);
-    sure &= nearest_sum(s, e, __fadd_rn(e, WeightPair<K>::lo), r);
+    sure &= nearest_sum(s, __fadd_rn(e, WeightPair<K>::lo), r);
     return r;
   }
 }
@@ -408,7 +409,7 @@ __device__ __forceinline__ void put_deviation(T* p, I f, bool& sure) {
       *p = half_sum(s, __fsub_rn(e, WeightPair<K>::lo));
     } else {
       float r;
-      sure &= nearest_sum(s, e, __fsub_rn(e, WeightPair<K>::lo), r);
+      sure &= nearest_sum(s, __fsub_rn(e, WeightPair<K>::lo), r);
       *p = r;
     }
   }
