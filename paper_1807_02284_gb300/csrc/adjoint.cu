@@ -454,8 +454,8 @@ constexpr int ADJ_THREADS = 128;
 // everything known from the node index alone is requested first (the pull and the velocity
 // neighbourhood in registers, the 31 adjoints by cp.async into this thread's shared-memory
 // column, 4 bytes each), the scalar corners as soon as u is known, and each is waited for
-// only where it is used.  128^3: 245 -> 169 us (1935 instructions per node, 63 % of issue slots,
-// 56 % of DRAM peak; before, the flags, the pull, the corners and the adjoints waited for one
+// only where it is used.  128^3: 245 -> 169 us (1995 instructions per node, 61 % of issue slots,
+// 52 % of DRAM peak; before, the flags, the pull, the corners and the adjoints waited for one
 // another in turn and 19 words per node went to pass B), 72 x 60 x 51 with open faces
 // 64 -> 34 us (rows of 72 nodes left 44 % of a 128-thread row's lanes idle).
 // 4 CTAs per SM (128 registers, no spills) against 3: 169 against 192 us at 128^3.
